@@ -124,20 +124,19 @@ int wfa_set_dt(wfa_grid g, double dt);
  * variant: 0 = automatic; 1..2 = one of the compiled tile shapes of the
  * tiled TMA kernel (depth steps per pass); 3 = the column-march kernel (one
  * step per pass, register queue along z, no shared memory; boundary cells by
- * ghost layers or a short fix-up launch); 4 = the two-step column-march
- * kernel (uniform k; two steps per pass, shared-memory stage plane; with
- * per-cell k it acts as 3); 5 = the column-march kernel with boundary cells
- * and periodic copies inside the pass (one launch per step; for small
+ * ghost layers or a short fix-up launch); 4 and 7 = two steps per pass with
+ * both steps' planes in registers (uniform k without held layers or exchange
+ * faces; elsewhere they act as 3); 5 = the column-march kernel with boundary
+ * cells and periodic copies inside the pass (one launch per step; for small
  * grids); 6 = the column-march kernel with 8 cells a thread (16 for bf16
- * fields with uniform k); 7 = two steps per pass with TMA-staged input
- * planes (uniform k; with per-cell k it acts as 3); -1 = the plain
+ * fields with uniform k); -1 = the plain
  * one-thread-per-column kernel (one step per pass; a
  * second, independent realisation of the same per-cell arithmetic).
  * Results do not depend on the choice: every kernel evaluates the same fixed
  * per-cell expression, so fields are bit-identical. */
 int wfa_set_tuning(wfa_grid g, int depth, int variant);
 
-/* Planes per z chunk of the column-march kernels (variants 3 and 5): each
+/* Planes per z chunk of the column-march kernels (variants 3 to 7): each
  * block of those kernels marches one chunk of the z extent, neighbouring
  * chunks in opposite directions. planes = 0 (the default) lets the tuned or
  * automatic choice stand. A tuning aid with no counterpart in the paper:
@@ -153,7 +152,7 @@ int wfa_set_zchunk(wfa_grid g, int planes);
 int wfa_get_tuning(wfa_grid g, int* depth, int* variant, int* zchunk);
 
 /* No counterpart in the paper (its step has one mapping, a column per tile,
- * Sec. 2.1). Time the compiled kernel configurations (the column-march kernels 3 to 7,
+ * Sec. 2.1). Time the compiled kernel configurations (the column-march kernels 3, 5, 6 and 7,
  * kernel 3 also with z chunks of 8, 12, 32, 64, 128 planes and of half the
  * z extent, kernel 6 with chunks of 12 and 32; the tiled TMA kernel at
  * depths 1..8 and two tile shapes) on this grid and use the fastest from

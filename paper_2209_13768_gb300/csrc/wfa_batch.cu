@@ -550,7 +550,7 @@ int batch_launch(wfa_grid* gs, const long long* steps, int count, int slot, bool
     // halos, held layers and 1/k of grids changed since their last step
     for (int i : order) {
         wfa_grid g = gs[i];
-        if (g->halo_dirty) {
+        if (g->halo_dirty || g->thin[g->cur] == TWINS_NONE) {
             int rc = refresh_halo(g, g->cur);
             if (rc) return rc;
             rc = prepare_coeff_halo(g);
@@ -819,8 +819,8 @@ int batch_launch(wfa_grid* gs, const long long* steps, int count, int slot, bool
         // copy (corners included); the per-round uniform-k passes one layer
         const bool one_layer = mode != 0 && cls[k] % NKIND == 0 &&
                                (mg[k].c.periodic[0] || mg[k].c.periodic[1] || mg[k].c.periodic[2]);
-        if (mg[k].steps >= 1) g->thin[g->cur] = one_layer;
-        if (mg[k].steps >= 2) g->thin[1 - g->cur] = one_layer;
+        if (mg[k].steps >= 1) g->thin[g->cur] = one_layer ? TWINS_ONE : TWINS_FULL;
+        if (mg[k].steps >= 2) g->thin[1 - g->cur] = one_layer ? TWINS_ONE : TWINS_FULL;
         g->steps_done += mg[k].steps;
     }
     return WFA_OK;

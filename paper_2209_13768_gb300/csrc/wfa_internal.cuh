@@ -35,10 +35,12 @@ constexpr int HALO = 8;       // halo width on every side (>= the deepest tempor
 constexpr int MAX_DEPTH = 8;  // steps fused per pass over the grid
 constexpr int NUM_TILE_VARIANTS = 2;  // tile shapes compiled per (storage, k mode, depth)
 constexpr int COL_VARIANT = 3;        // the one-step column-march kernel
-constexpr int FUSED_VARIANT = 4;      // the two-step column-march kernel (uniform k)
+constexpr int FUSED_VARIANT = 4;      // the same kernel as PAIR_VARIANT
 constexpr int INPLACE_VARIANT = 5;    // the one-step column-march kernel, boundaries in place
 constexpr int WIDE_VARIANT = 6;       // the one-step column-march kernel, 8 cells a thread (16 for bf16, uniform k)
-constexpr int T2_VARIANT = 7;         // two steps per pass, TMA-staged planes (uniform k)
+constexpr int PAIR_VARIANT = 7;       // two steps per pass in registers (uniform k)
+
+enum { TWINS_FULL = 0, TWINS_ONE = 1, TWINS_NONE = 2 };
 
 // NVTX range over one API call: a named span on a profiler's timeline
 // (nothing happens unless a tool is attached).
@@ -145,8 +147,9 @@ struct wfa_grid_s {
     void* cg;             // wfa::CgWork (work vectors and graph of the implicit solver)
     int cg_method;        // WFA_CG_CLASSIC / WFA_CG_PIPELINED (wfa_set_cg_method)
     cudaEvent_t xev;      // orders plane exchanges against this grid's stream (wfa_exchange)
-    bool thin[2];         // buffer's periodic copies hold one layer without corners (a thin column
-                          // pass wrote it): enough for one-step kernels, not for the tiled ones
+    unsigned char thin[2];   // periodic copies each buffer holds: TWINS_FULL every layer, TWINS_ONE
+                             // one layer without corners (a thin column pass wrote it: enough for
+                             // one-step kernels), TWINS_NONE stale (the two-step pass wraps its reads)
 };
 
 namespace wfa {

@@ -155,9 +155,8 @@ static int num_sms() {
 // ------------------------------------------------------------ tuning ------
 // Kernel configuration of a pass: variant (COL_VARIANT = column march, one
 // step; INPLACE_VARIANT = the same with boundaries and periodic copies in the
-// pass itself; FUSED_VARIANT = column march, two steps, uniform k;
-// WIDE_VARIANT = column march, 8 cells a thread (16 for bf16 with uniform k);
-// T2_VARIANT = two steps, TMA-staged planes, uniform k; 1..NUM_TILE_VARIANTS
+// pass itself; WIDE_VARIANT = column march, 8 cells a thread (16 for bf16 with uniform k);
+// PAIR_VARIANT (and FUSED_VARIANT) = two steps in registers, uniform k; 1..NUM_TILE_VARIANTS
 // = tiled TMA kernel, `depth` fused steps; -1 = the plain one-column kernel)
 // and depth.
 struct Choice {
@@ -225,8 +224,53 @@ static void tune_save_locked() {
     fclose(f);
 }
 
+// The two-step pass takes this grid: uniform k, no held layers or exchange
+// faces, (bf16) Dirichlet values that the halo's ghost cells hold exactly,
+// and rows of at least 8 cells (a group across a periodic face wraps once).
+static bool pair_applies(const wfa_grid_s* g) {
+    if (g->k || g->n[0] < 8) return false;
+    for (int f = 0; f < 6; ++f) {
+        if (g->bc_kind[f] == WFA_BC_DIRICHLET_CELL || g->bc_kind[f] == WFA_BC_EXCHANGE) return false;
+        if (g->bc_kind[f] == WFA_BC_DIRICHLET && g->storage == WFA_BF16) {
+            const float tb = (float)g->bc_value[f];
+            uint32_t bits;
+            memcpy(&bits, &tb, sizeof bits);
+            if (bits & 0xFFFFu) return false;
+        }
+    }
+    return true;
+}
+
+// The configuration of a grid that was not tuned, from its sizes and faces.
+// Per-cell k: the one-step column march (the two-step pass takes uniform k).
+// Uniform k, us a step on one GB300 (fp32; bf16 is within 15%):
+//   two steps in registers against the column march, no periodic axis:
+//     80^3 3.8 / 5.2, 128^3 6.4 / 8.1, 40x300x500 18.4 / 30.8, 512^3 118 / 212;
+//     rows of 31 cells 9.5 / 9.1 (a warp's 120 cells are mostly empty);
+//   periodic axes: wrapped reads are slower, and a column march without faces
+//     is one launch: 128^3 7.8 / 5.3 to 7.4, 160^3 9.6 / 9.3 to 10.9,
+//     640x500x333 96 / 144, 1024x1024x512 401 / 728; ragged periodic rows
+//     read the two end tiles cell by cell: 90x90x400 18 / 12;
+//   up to 64^3 without a periodic axis the launches dominate and boundary
+//     cells in the pass are fastest: 64^3 2.9 in place, 3.5 two steps, 4.7
+//     column march with its boundary launch.
+static Choice default_choice(const wfa_grid_s* g) {
+    const long long cells = (long long)g->n[0] * g->n[1] * g->n[2];
+    const bool perx = g->bc_kind[0] == WFA_BC_PERIODIC;
+    const bool per = perx || g->bc_kind[2] == WFA_BC_PERIODIC || g->bc_kind[4] == WFA_BC_PERIODIC;
+    if (!pair_applies(g)) return Choice{COL_VARIANT, 1};
+    if (!per) {
+        if (cells <= 300000) return Choice{INPLACE_VARIANT, 1};
+        return g->n[0] >= 40 ? Choice{PAIR_VARIANT, 2} : Choice{COL_VARIANT, 1};
+    }
+    const bool wide = g->n[0] >= (perx && g->n[0] % 4 ? 480 : 100);
+    return wide && cells >= (1LL << 22) ? Choice{PAIR_VARIANT, 2} : Choice{COL_VARIANT, 1};
+}
+
+static bool two_step_variant(int variant) { return variant == FUSED_VARIANT || variant == PAIR_VARIANT; }
+
 static Choice choose(const wfa_grid_s* g) {
-    Choice ch{COL_VARIANT, 1};   // untuned default: the column-march kernel, one step per pass
+    Choice ch = default_choice(g);
     if (g->tuned_variant) {
         ch = Choice{g->tuned_variant, g->tuned_depth, g->tuned_zchunk};
     } else {
@@ -248,7 +292,7 @@ static Choice choose(const wfa_grid_s* g) {
         ch = Choice{COL_VARIANT, 1, ch.zc};
     if (ch.variant < 0 || ch.variant == COL_VARIANT || ch.variant == INPLACE_VARIANT || ch.variant == WIDE_VARIANT)
         ch.depth = 1;
-    if (ch.variant == FUSED_VARIANT || ch.variant == T2_VARIANT) ch.depth = g->k ? 1 : 2;   // per-cell k: one step
+    if (two_step_variant(ch.variant)) ch.depth = pair_applies(g) ? 2 : 1;   // one step where two do not apply
     return ch;
 }
 
@@ -296,41 +340,39 @@ static SweepArgs base_args(wfa_grid_s* g, const SweepCoef& c, int in_buf, int zc
 // Kernels one pass launches (the column kernels add a boundary fix-up and a
 // copy per periodic axis, see col_launch / col2_launch).
 static int pass_launches(const wfa_grid_s* g, const SweepCoef& c, int depth, int variant) {
-    const int periodic = c.periodic[0] + c.periodic[1] + c.periodic[2];
-    if (variant == FUSED_VARIANT && depth == 2 && !g->r) return 1 + periodic;
-    if (variant == COL_VARIANT || variant == WIDE_VARIANT || variant == FUSED_VARIANT || variant == T2_VARIANT) {   // thin pass
+    if (two_step_variant(variant) && depth == 2) return 1;
+    if (variant == COL_VARIANT || variant == WIDE_VARIANT || two_step_variant(variant)) {   // thin pass
         // boundary cells the ghost layers do not hold: one boundary_fix launch
-        // (the one-step column pass keeps held faces itself)
-        const bool col = variant == COL_VARIANT || variant == WIDE_VARIANT ||
-                         ((variant == FUSED_VARIANT || variant == T2_VARIANT) && !(depth == 2 && !g->r));
+        // (the column pass keeps held faces itself)
         bool faces = false;
-        for (int f = 0; f < 6; ++f) faces = faces || (!c.periodic[f >> 1] && !c.ext[f] && !(col && c.held[f]));
+        for (int f = 0; f < 6; ++f) faces = faces || (!c.periodic[f >> 1] && !c.ext[f] && !c.held[f]);
         return 1 + (faces && !c.halo_bc ? 1 : 0);
     }
     return 1;
 }
 
-// The pass reads periodic copies beyond the first layer (or corner copies):
-// the tiled kernels and the two-step column kernel.
-static bool needs_full_twins(const wfa_grid_s* g, int depth, int variant) {
-    if (variant == FUSED_VARIANT || variant == T2_VARIANT) return depth == 2 && !g->r;
-    return variant >= 1 && variant <= NUM_TILE_VARIANTS;
+// The pass reads periodic copies that buffer `buf` does not hold: the tiled
+// kernels read every layer, the one-step kernels one, the two-step one none.
+static bool lacks_twins(const wfa_grid_s* g, int buf, int depth, int variant) {
+    if (two_step_variant(variant) && depth == 2) return false;
+    if (variant >= 1 && variant <= NUM_TILE_VARIANTS) return g->thin[buf] != TWINS_FULL;
+    return g->thin[buf] == TWINS_NONE;
 }
-// The pass writes one layer of periodic copies only (the thin column pass).
-static bool writes_thin_twins(const wfa_grid_s* g, const SweepCoef& c, int depth, int variant) {
-    if (!c.periodic[0] && !c.periodic[1] && !c.periodic[2]) return false;
-    const bool two = (variant == FUSED_VARIANT || variant == T2_VARIANT) && depth == 2 && !g->r;
-    return !two && (variant == COL_VARIANT || variant == WIDE_VARIANT || variant == FUSED_VARIANT || variant == T2_VARIANT);
+// The periodic copies a pass leaves in the buffer it writes.
+static unsigned char twins_written(const SweepCoef& c, int depth, int variant) {
+    if (!c.periodic[0] && !c.periodic[1] && !c.periodic[2]) return TWINS_FULL;
+    if (two_step_variant(variant)) return depth == 2 ? TWINS_NONE : TWINS_ONE;
+    return variant == COL_VARIANT || variant == WIDE_VARIANT ? TWINS_ONE : TWINS_FULL;
 }
 
 // One pass of `depth` fused steps from buffer g->cur into the other buffer
 // (zc: planes per z chunk of the column kernels, 0 = automatic).
 static int one_pass(wfa_grid_s* g, const SweepCoef& c, int depth, int variant, int zc = 0) {
-    if (needs_full_twins(g, depth, variant) && g->thin[g->cur]) {   // complete the copies first
+    if (lacks_twins(g, g->cur, depth, variant)) {   // complete the copies first
         const int rc = refresh_halo(g, g->cur);
         if (rc) return rc;
     }
-    g->thin[1 - g->cur] = writes_thin_twins(g, c, depth, variant);
+    g->thin[1 - g->cur] = twins_written(c, depth, variant);
     g->launches += pass_launches(g, c, depth, variant);
     SweepArgs a = base_args(g, c, g->cur, zc);
     const cudaEvent_t* ev = timing_slot(g);
@@ -346,25 +388,15 @@ static int one_pass(wfa_grid_s* g, const SweepCoef& c, int depth, int variant, i
         g->cur = 1 - g->cur;
         return WFA_OK;
     }
-    if (variant == T2_VARIANT && depth == 2 && !g->r) {   // two steps, TMA-staged planes (uniform k)
-        TmapCache* tm = nullptr;
-        int rc = get_tmaps(g, 80, 20, &tm);
-        if (rc) return rc;
-        cudaError_t e = g->storage == WFA_BF16 ? launch_t2_bf16_u(&tm->t[g->cur], a, g->stream, num_sms(), ev)
-                                               : launch_t2_f32_u(&tm->t[g->cur], a, g->stream, num_sms(), ev);
-        if (e != cudaSuccess) return cuda_fail(e, "sweep_t2 launch");
+    if (two_step_variant(variant) && depth == 2) {   // two steps in registers (uniform k)
+        const cudaError_t e = g->storage == WFA_BF16 ? launch_pair_bf16_u(a, g->stream, num_sms(), ev)
+                                                     : launch_pair_f32_u(a, g->stream, num_sms(), ev);
+        if (e != cudaSuccess) return cuda_fail(e, "sweep_pair launch");
         g->cur = 1 - g->cur;
         return WFA_OK;
     }
-    if (variant == FUSED_VARIANT && depth == 2 && !g->r) {   // two-step column march (uniform k)
-        cudaError_t e = g->storage == WFA_BF16 ? launch_col2_bf16_u(a, g->stream, num_sms(), ev)
-                                               : launch_col2_f32_u(a, g->stream, num_sms(), ev);
-        if (e != cudaSuccess) return cuda_fail(e, "sweep_col2 launch");
-        g->cur = 1 - g->cur;
-        return WFA_OK;
-    }
-    if (variant == COL_VARIANT || variant == FUSED_VARIANT || variant == INPLACE_VARIANT || variant == T2_VARIANT ||
-        variant == WIDE_VARIANT) {   // column march, one step
+    if (variant == COL_VARIANT || variant == INPLACE_VARIANT || variant == WIDE_VARIANT ||
+        two_step_variant(variant)) {   // column march, one step
         const bool inl = variant == INPLACE_VARIANT, wide = variant == WIDE_VARIANT;
         cudaError_t e;
         if (g->storage == WFA_BF16)
@@ -451,7 +483,7 @@ static int run_graph(wfa_grid_s* g, const SweepCoef& c, const Choice& ch, cudaGr
         const cudaStream_t user = g->stream;
         const int cur0 = g->cur;
         const long long launches0 = g->launches;
-        const bool thin0[2] = {g->thin[0], g->thin[1]};
+        const unsigned char thin0[2] = {g->thin[0], g->thin[1]};
         g->stream = gs->stream;
         cudaError_t e = cudaStreamBeginCapture(gs->stream, cudaStreamCaptureModeThreadLocal);
         int rc = WFA_OK;
@@ -487,10 +519,17 @@ int launch_sweep(wfa_grid_s* g, long long nsteps) {
     if (rc) return rc;
     const Choice ch = choose(g);
     const long long cells = (long long)g->n[0] * g->n[1] * g->n[2];
+    if (two_step_variant(ch.variant) && ch.depth == 2 && nsteps % 2) {
+        // an odd count: its single step first, while the periodic copies it
+        // reads are current (the two-step passes leave them stale)
+        rc = one_pass(g, c, 1, ch.variant, ch.zc);
+        if (rc) return rc;
+        --nsteps;
+    }
     const long long runs = nsteps / ((long long)ch.depth * GRAPH_PASSES);
     if (cells <= GRAPH_MAX_CELLS && runs >= 2) {
         cudaGraphExec_t exec = nullptr;
-        if (needs_full_twins(g, ch.depth, ch.variant) && g->thin[g->cur]) {   // not inside the graph
+        if (lacks_twins(g, g->cur, ch.depth, ch.variant)) {   // not inside the graph
             rc = refresh_halo(g, g->cur);
             if (rc) return rc;
         }
@@ -508,7 +547,7 @@ int launch_sweep(wfa_grid_s* g, long long nsteps) {
         }
         g->launches += runs * GRAPH_PASSES * pass_launches(g, c, ch.depth, ch.variant);
         nsteps -= runs * GRAPH_PASSES * ch.depth;
-        g->thin[0] = g->thin[1] = writes_thin_twins(g, c, ch.depth, ch.variant);   // both written by the run
+        g->thin[0] = g->thin[1] = twins_written(c, ch.depth, ch.variant);   // both written by the run
     }
     while (nsteps > 0) {
         const int d = (int)std::min<long long>(ch.depth, nsteps);
@@ -532,7 +571,7 @@ int autotune(wfa_grid_s* g, int* depth_out, int* variant_out) {
         ~Pause() { g->timing_every = every; }
     } pause{g, g->timing_every};
     g->timing_every = 0;
-    std::vector<Choice> cands = {{COL_VARIANT, 1}, {WIDE_VARIANT, 1}, {INPLACE_VARIANT, 1}, {T2_VARIANT, 2}, {FUSED_VARIANT, 2}, {1, 1}, {2, 1},
+    std::vector<Choice> cands = {{COL_VARIANT, 1}, {WIDE_VARIANT, 1}, {INPLACE_VARIANT, 1}, {PAIR_VARIANT, 2}, {1, 1}, {2, 1},
                                  {1, 2}, {2, 2}, {1, 3}, {2, 3}, {1, 4}, {2, 4}, {1, 6}, {1, 8}};
     // the column kernels with other z chunk lengths: longer ones read fewer
     // boundary planes twice (fewer, longer-lived blocks, down to two chunks:
@@ -558,7 +597,7 @@ int autotune(wfa_grid_s* g, int* depth_out, int* variant_out) {
     float best_ms = 1e30f;
     for (const Choice& ch : cands) {
         if (e != cudaSuccess) break;
-        if ((ch.variant == FUSED_VARIANT || ch.variant == T2_VARIANT) && g->k) continue;   // uniform k only
+        if (two_step_variant(ch.variant) && !pair_applies(g)) continue;
         if (has_exchange_face(g) && ch.variant != COL_VARIANT && ch.variant != INPLACE_VARIANT &&
             ch.variant != WIDE_VARIANT)
             continue;

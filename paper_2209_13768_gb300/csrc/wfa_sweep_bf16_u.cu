@@ -1,7 +1,6 @@
 // Compiled sweep kernels: bf16 storage, uniform conductivity, depths 1..8.
 #include "wfa_sweep_col.cuh"
-#include "wfa_sweep_fused.cuh"
-#include "wfa_sweep_t2.cuh"
+#include "wfa_sweep_pair.cuh"
 #include "wfa_sweep_impl.cuh"
 
 namespace wfa {
@@ -62,12 +61,8 @@ cudaError_t launch_col_bf16_u(const SweepArgs& a, cudaStream_t st, int nsm, cons
     return col_launch<S, KVAR>(a, st, nsm, ev, inl, wide);
 }
 
-cudaError_t launch_col2_bf16_u(const SweepArgs& a, cudaStream_t st, int nsm, const cudaEvent_t* ev) {
-    return col2_launch<S>(a, st, nsm, ev);
-}
-
-cudaError_t launch_t2_bf16_u(const CUtensorMap* tmT, const SweepArgs& a, cudaStream_t st, int nsm, const cudaEvent_t* ev) {
-    return t2_launch<S>(tmT, a, st, nsm, ev);
+cudaError_t launch_pair_bf16_u(const SweepArgs& a, cudaStream_t st, int nsm, const cudaEvent_t* ev) {
+    return pair_launch<S>(a, st, nsm, ev);
 }
 
 }  // namespace wfa

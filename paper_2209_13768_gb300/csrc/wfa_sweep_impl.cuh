@@ -37,13 +37,9 @@ cudaError_t launch_col_f32_u(const SweepArgs& a, cudaStream_t st, int nsm, const
 cudaError_t launch_col_f32_k(const SweepArgs& a, cudaStream_t st, int nsm, const cudaEvent_t* ev, bool inl, bool wide);
 cudaError_t launch_col_bf16_u(const SweepArgs& a, cudaStream_t st, int nsm, const cudaEvent_t* ev, bool inl, bool wide);
 cudaError_t launch_col_bf16_k(const SweepArgs& a, cudaStream_t st, int nsm, const cudaEvent_t* ev, bool inl, bool wide);
-// two steps per pass with TMA-staged input planes (variant 7, uniform k only);
-// tmT: the input buffer's tensor map with an 80 x 20 box
-cudaError_t launch_t2_f32_u(const CUtensorMap* tmT, const SweepArgs& a, cudaStream_t st, int nsm, const cudaEvent_t* ev);
-cudaError_t launch_t2_bf16_u(const CUtensorMap* tmT, const SweepArgs& a, cudaStream_t st, int nsm, const cudaEvent_t* ev);
-// two-step column-march kernel (variant 4, uniform k only)
-cudaError_t launch_col2_f32_u(const SweepArgs& a, cudaStream_t st, int nsm, const cudaEvent_t* ev);
-cudaError_t launch_col2_bf16_u(const SweepArgs& a, cudaStream_t st, int nsm, const cudaEvent_t* ev);
+// two steps per pass in registers (variants 4 and 7, uniform k only)
+cudaError_t launch_pair_f32_u(const SweepArgs& a, cudaStream_t st, int nsm, const cudaEvent_t* ev);
+cudaError_t launch_pair_bf16_u(const SweepArgs& a, cudaStream_t st, int nsm, const cudaEvent_t* ev);
 
 template <typename S, bool KVAR, int D, int EX, int EY, int R, int PF>
 cudaError_t tb_launch(const CUtensorMap* tmT, const CUtensorMap* tmK, const SweepArgs& a, int blocks,
