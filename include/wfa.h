@@ -125,8 +125,8 @@ int wfa_set_dt(wfa_grid g, double dt);
  * tiled TMA kernel (depth steps per pass); 3 = the column-march kernel (one
  * step per pass, register queue along z, no shared memory; boundary cells by
  * ghost layers or a short fix-up launch); 4 and 7 = two steps per pass with
- * both steps' planes in registers (uniform k without held layers or exchange
- * faces; elsewhere they act as 3); 5 = the column-march kernel with boundary
+ * both steps' planes in registers (not with held layers, exchange faces, or
+ * zero-flux faces that meet advection with per-cell k: there they act as 3); 5 = the column-march kernel with boundary
  * cells and periodic copies inside the pass (one launch per step; for small
  * grids); 6 = the column-march kernel with 8 cells a thread (16 for bf16
  * fields with uniform k); -1 = the plain

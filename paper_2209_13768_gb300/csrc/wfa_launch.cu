@@ -224,13 +224,16 @@ static void tune_save_locked() {
     fclose(f);
 }
 
-// The two-step pass takes this grid: uniform k, no held layers or exchange
-// faces, (bf16) Dirichlet values that the halo's ghost cells hold exactly,
-// and rows of at least 8 cells (a group across a periodic face wraps once).
+// The two-step pass takes this grid: no held layers or exchange faces, (bf16)
+// Dirichlet values that the halo's ghost cells hold exactly, with per-cell k
+// no zero-flux face that meets advection (see halo_bc in build_coef), and
+// rows of at least 8 cells (a group across a periodic face wraps once).
 static bool pair_applies(const wfa_grid_s* g) {
-    if (g->k || g->n[0] < 8) return false;
+    if (g->n[0] < 8) return false;
+    const bool adv = g->u[0] != 0.0 || g->u[1] != 0.0 || g->u[2] != 0.0;
     for (int f = 0; f < 6; ++f) {
         if (g->bc_kind[f] == WFA_BC_DIRICHLET_CELL || g->bc_kind[f] == WFA_BC_EXCHANGE) return false;
+        if (g->k && adv && g->bc_kind[f] == WFA_BC_ZEROFLUX) return false;
         if (g->bc_kind[f] == WFA_BC_DIRICHLET && g->storage == WFA_BF16) {
             const float tb = (float)g->bc_value[f];
             uint32_t bits;
@@ -241,30 +244,35 @@ static bool pair_applies(const wfa_grid_s* g) {
     return true;
 }
 
-// The configuration of a grid that was not tuned, from its sizes and faces.
-// Per-cell k: the one-step column march (the two-step pass takes uniform k).
-// Uniform k, us a step on one GB300 (fp32; bf16 is within 15%):
-//   two steps in registers against the column march, no periodic axis:
-//     80^3 3.8 / 5.2, 128^3 6.4 / 8.1, 40x300x500 18.4 / 30.8, 512^3 118 / 212;
-//     rows of 31 cells 9.5 / 9.1 (a warp's 120 cells are mostly empty);
-//   periodic axes: wrapped reads are slower, and a column march without faces
-//     is one launch: 128^3 7.8 / 5.3 to 7.4, 160^3 9.6 / 9.3 to 10.9,
-//     640x500x333 96 / 144, 1024x1024x512 401 / 728; ragged periodic rows
-//     read the two end tiles cell by cell: 90x90x400 18 / 12;
-//   up to 64^3 without a periodic axis the launches dominate and boundary
-//     cells in the pass are fastest: 64^3 2.9 in place, 3.5 two steps, 4.7
-//     column march with its boundary launch.
+// The configuration of a grid that was not tuned, from its sizes and faces:
+// two steps a pass where that was faster. us a step on one GB300, two steps
+// against the one-step column march (fp32; bf16 is within 15%):
+//   uniform k, no periodic axis: 80^3 3.8 / 5.2, 128^3 6.4 / 8.1, 40x300x500
+//     18.4 / 30.8, 512^3 118 / 212; rows of 31 cells 9.5 / 9.1 (a warp's 120
+//     cells are mostly empty); up to 64^3 the launches dominate and boundary
+//     cells in the pass are fastest (64^3 2.9, two steps 3.5, column march
+//     with its boundary launch 4.7);
+//   uniform k, periodic axes: wrapped reads are slower, and a column march
+//     without faces is one launch: 128^3 7.8 / 5.3 to 7.4, 160^3 9.6 / 9.3 to
+//     10.9, 640x500x333 96 / 144, 1024x1024x512 401 / 728; ragged periodic
+//     rows read the two end tiles cell by cell: 90x90x400 18 / 12;
+//   per-cell k, no periodic axis: 80^3 3.8 / 3.3, 100^3 4.0 / 5.2, 128^3 4.9 /
+//     6.2, 31x200x160 4.6 / 6.4, 333x250x187 33 / 42, 512^3 213 / 267;
+//   per-cell k, periodic axes: 128^3 8.4 / 6.7, 160^3 11.2 / 13.2, 512^3 232 /
+//     285; ragged periodic rows 333x250x187 65 / 48.
 static Choice default_choice(const wfa_grid_s* g) {
     const long long cells = (long long)g->n[0] * g->n[1] * g->n[2];
     const bool perx = g->bc_kind[0] == WFA_BC_PERIODIC;
     const bool per = perx || g->bc_kind[2] == WFA_BC_PERIODIC || g->bc_kind[4] == WFA_BC_PERIODIC;
-    if (!pair_applies(g)) return Choice{COL_VARIANT, 1};
-    if (!per) {
-        if (cells <= 300000) return Choice{INPLACE_VARIANT, 1};
-        return g->n[0] >= 40 ? Choice{PAIR_VARIANT, 2} : Choice{COL_VARIANT, 1};
+    const Choice one{COL_VARIANT, 1}, two{PAIR_VARIANT, 2};
+    if (!pair_applies(g)) return one;
+    if (per) {
+        const bool wide = !perx || g->n[0] % 4 == 0 ? g->k || g->n[0] >= 100 : g->n[0] >= (g->k ? 960 : 480);
+        return wide && cells >= (1LL << 22) ? two : one;
     }
-    const bool wide = g->n[0] >= (perx && g->n[0] % 4 ? 480 : 100);
-    return wide && cells >= (1LL << 22) ? Choice{PAIR_VARIANT, 2} : Choice{COL_VARIANT, 1};
+    if (g->k) return cells >= 900000 ? two : one;
+    if (cells <= 300000) return Choice{INPLACE_VARIANT, 1};
+    return g->n[0] >= 40 ? two : one;
 }
 
 static bool two_step_variant(int variant) { return variant == FUSED_VARIANT || variant == PAIR_VARIANT; }
@@ -388,9 +396,12 @@ static int one_pass(wfa_grid_s* g, const SweepCoef& c, int depth, int variant, i
         g->cur = 1 - g->cur;
         return WFA_OK;
     }
-    if (two_step_variant(variant) && depth == 2) {   // two steps in registers (uniform k)
-        const cudaError_t e = g->storage == WFA_BF16 ? launch_pair_bf16_u(a, g->stream, num_sms(), ev)
-                                                     : launch_pair_f32_u(a, g->stream, num_sms(), ev);
+    if (two_step_variant(variant) && depth == 2) {   // two steps in registers
+        cudaError_t e;
+        if (g->storage == WFA_BF16)
+            e = g->r ? launch_pair_bf16_k(a, g->stream, num_sms(), ev) : launch_pair_bf16_u(a, g->stream, num_sms(), ev);
+        else
+            e = g->r ? launch_pair_f32_k(a, g->stream, num_sms(), ev) : launch_pair_f32_u(a, g->stream, num_sms(), ev);
         if (e != cudaSuccess) return cuda_fail(e, "sweep_pair launch");
         g->cur = 1 - g->cur;
         return WFA_OK;

@@ -1,5 +1,6 @@
 // Compiled sweep kernels: f32 storage, per-cell conductivity, depths 1..8.
 #include "wfa_sweep_col.cuh"
+#include "wfa_sweep_pair_k.cuh"
 #include "wfa_sweep_impl.cuh"
 
 namespace wfa {
@@ -58,6 +59,10 @@ cudaError_t launch_simple_f32_k(const SweepArgs& a, cudaStream_t st) {
 
 cudaError_t launch_col_f32_k(const SweepArgs& a, cudaStream_t st, int nsm, const cudaEvent_t* ev, bool inl, bool wide) {
     return col_launch<S, KVAR>(a, st, nsm, ev, inl, wide);
+}
+
+cudaError_t launch_pair_f32_k(const SweepArgs& a, cudaStream_t st, int nsm, const cudaEvent_t* ev) {
+    return pair_k_launch<S>(a, st, nsm, ev);
 }
 
 }  // namespace wfa

@@ -37,8 +37,10 @@ cudaError_t launch_col_f32_u(const SweepArgs& a, cudaStream_t st, int nsm, const
 cudaError_t launch_col_f32_k(const SweepArgs& a, cudaStream_t st, int nsm, const cudaEvent_t* ev, bool inl, bool wide);
 cudaError_t launch_col_bf16_u(const SweepArgs& a, cudaStream_t st, int nsm, const cudaEvent_t* ev, bool inl, bool wide);
 cudaError_t launch_col_bf16_k(const SweepArgs& a, cudaStream_t st, int nsm, const cudaEvent_t* ev, bool inl, bool wide);
-// two steps per pass in registers (variants 4 and 7, uniform k only)
+// two steps per pass in registers (variants 4 and 7)
 cudaError_t launch_pair_f32_u(const SweepArgs& a, cudaStream_t st, int nsm, const cudaEvent_t* ev);
+cudaError_t launch_pair_f32_k(const SweepArgs& a, cudaStream_t st, int nsm, const cudaEvent_t* ev);
+cudaError_t launch_pair_bf16_k(const SweepArgs& a, cudaStream_t st, int nsm, const cudaEvent_t* ev);
 cudaError_t launch_pair_bf16_u(const SweepArgs& a, cudaStream_t st, int nsm, const cudaEvent_t* ev);
 
 template <typename S, bool KVAR, int D, int EX, int EY, int R, int PF>

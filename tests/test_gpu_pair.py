@@ -1,5 +1,5 @@
-"""The two-step pass (variant 7) against the plain one-column kernel (-1),
-bitwise: at the edges of its 120-cell x tiles, 4-row tiles and z chunks, with
+"""The two-step passes (variant 7) against the plain one-column kernel (-1),
+bitwise: at the edges of their 120-cell x tiles, 4- or 10-row tiles and z chunks, with
 ragged rows and wrapped reads, and in sequences with the kernels that read
 periodic copies, which it leaves stale."""
 import numpy as np
@@ -21,18 +21,21 @@ FACES = {
 }
 
 
-def _problem(shape, faces, steps=6, seed=0):
+def _problem(shape, faces, steps=6, seed=0, kvar=False, adv=True):
     rng = np.random.default_rng(seed)
-    return W.Problem(shape=shape, T0=rng.uniform(0, 1, shape[::-1]).astype(np.float32), k=0.8,
-                     u=tuple(rng.uniform(-0.4, 0.4, 3)), bc=FACES[faces], h=tuple(rng.uniform(0.8, 1.25, 3)), steps=steps)
+    k = np.exp(0.5 * rng.standard_normal(shape[::-1])).astype(np.float32) if kvar else 0.8
+    return W.Problem(shape=shape, T0=rng.uniform(0, 1, shape[::-1]).astype(np.float32), k=k,
+                     u=tuple(rng.uniform(-0.4, 0.4, 3)) if adv else (0.0, 0.0, 0.0), bc=FACES[faces],
+                     h=tuple(rng.uniform(0.8, 1.25, 3)), steps=steps)
 
 
 @pytest.mark.parametrize("storage", [wfa.F32, wfa.BF16])
+@pytest.mark.parametrize("kvar,adv", [(False, True), (True, False), (True, True)])
 @pytest.mark.parametrize("faces", sorted(FACES))
 @pytest.mark.parametrize("shape", [(8, 2, 2), (9, 3, 4), (64, 5, 7), (119, 4, 6), (120, 9, 5), (121, 8, 9), (124, 6, 8),
-                                   (125, 13, 30), (240, 7, 5), (243, 4, 26), (245, 12, 11), (365, 5, 6)])
-def test_pair_bitwise_at_tile_edges(shape, faces, storage):
-    p = _problem(shape, faces)
+                                   (125, 13, 30), (240, 7, 5), (243, 10, 26), (245, 12, 11), (365, 21, 6)])
+def test_pair_bitwise_at_tile_edges(shape, faces, kvar, adv, storage):
+    p = _problem(shape, faces, kvar=kvar, adv=adv)
     ref = run_gpu(p, storage=storage, variant=-1)
     for zc in (0, 1, 3, 24):
         np.testing.assert_array_equal(run_gpu(p, storage=storage, depth=2, variant=7, zchunk=zc), ref, err_msg=f"zchunk {zc}")
@@ -40,10 +43,11 @@ def test_pair_bitwise_at_tile_edges(shape, faces, storage):
     np.testing.assert_array_equal(run_gpu(p, storage=storage, depth=2, variant=7), run_gpu(p, storage=storage, variant=-1))
 
 
+@pytest.mark.parametrize("kvar", [False, True])
 @pytest.mark.parametrize("faces", ["torus", "x"])
-def test_kernels_after_a_pair_pass_refresh_periodic_copies(faces):
+def test_kernels_after_a_pair_pass_refresh_periodic_copies(faces, kvar):
     """Each of these reads periodic copies of the field a two-step pass wrote."""
-    p = _problem((68, 11, 9), faces)
+    p = _problem((68, 11, 9), faces, kvar=kvar, adv=not kvar)
     ref = run_gpu(p, steps=8, variant=-1)
     for depth, variant in [(1, 3), (1, 5), (1, 6), (1, -1), (2, 1), (3, 2)]:
         with make_grid(p) as g:
@@ -69,13 +73,14 @@ def test_kernels_after_a_pair_pass_refresh_periodic_copies(faces):
 
 
 def test_faces_the_pair_pass_does_not_take():
-    """Held layers, per-cell k, and a bf16 Dirichlet value the halo cannot hold
-    run one step a pass."""
+    """Held layers, zero-flux walls with per-cell k and advection, and a bf16
+    Dirichlet value the halo cannot hold run one step a pass."""
     held = W.Problem(shape=(40, 12, 10), T0=W.uniform01((40, 12, 10), 3), k=1.0, bc=[("dirichlet_cell", 0.5)] * 6, steps=5)
     np.testing.assert_array_equal(run_gpu(held, depth=2, variant=7), run_gpu(held, variant=-1))
     p = _problem((40, 12, 10), "cold")
     p.bc = [(D, 0.3)] * 6     # not a bf16 value
     np.testing.assert_array_equal(run_gpu(p, storage=wfa.BF16, depth=2, variant=7), run_gpu(p, storage=wfa.BF16, variant=-1))
-    with make_grid(p, storage=wfa.BF16) as g:
-        g.set_tuning(2, 7)
-        assert g.tuning()[0] == 1
+    for p, storage in [(p, wfa.BF16), (_problem((40, 12, 10), "walls", kvar=True), wfa.F32), (held, wfa.F32)]:
+        with make_grid(p, storage=storage) as g:
+            g.set_tuning(2, 7)
+            assert g.tuning()[0] == 1
