@@ -12,7 +12,13 @@
 //
 // Default ("rounds"): every round is one launch per class of grid (storage
 // type x conductivity mode x advection x ghost-layer faces) over the active
-// units, one block per unit; the whole sequence is captured into one CUDA
+// units, one block per unit. Classes whose ghost layers hold every face
+// (per-cell k) take two steps a round with the single grid's two-step pass
+// (sweep_pair_k; an odd count takes its single step first): 256 grids of 16 to
+// 128 cells an edge 302 -> 370 GLUPS, 14 grids of 0.1 to 2.7 M cells 345 ->
+// 375, one of 1.9 M cells 132 -> 216. (Uniform k keeps one step a round: the
+// two-step pass there, whose warps recompute their ring rows, ran 191 against
+// 303 GLUPS on 18 such grids.) The whole sequence is captured into one CUDA
 // graph and launched once, so the launch boundary is the barrier between
 // rounds and nothing inside a kernel waits on another block. Grids are
 // independent, so the graph has a branch per class and group of grids
@@ -29,6 +35,7 @@
 // (256 grids of 16..128 cells per edge, side by side with an earlier column
 // march: 200 GLUPS against 168 persistent; the per-round graph now runs
 // about 305).
+#include <math.h>
 #include <stdlib.h>
 #include <string.h>
 
@@ -40,16 +47,22 @@
 #include <vector>
 
 #include "wfa_sweep_col.cuh"
+#include "wfa_sweep_pair_k.cuh"
 
 namespace wfa {
 
 namespace {
 
 constexpr int MG_THREADS = 256;
-// {f32, bf16} x {uniform k, per-cell k, per-cell k with advection, and the
-// last two with every boundary face in the ghost layers}
-constexpr int NKIND = 5;
+// {f32, bf16} x {uniform k, per-cell k, per-cell k with advection, the last
+// two with every boundary face in the ghost layers, and those with a periodic
+// axis (per-round launches only: the two-step pass wraps its reads there)}
+constexpr int NKIND = 7;
+constexpr int KIND_PAIR = 3;
+constexpr bool pair_kind(int kind) { return kind >= KIND_PAIR; }   // per-round launches take two steps
+constexpr int PAIR_THREADS = 32 * PairKCfg::W;
 constexpr int NCLASS = 2 * NKIND;
+constexpr int PKIND = 5, PNCLASS = 2 * PKIND;   // the persistent kernel's kinds: the first five
 // per-round launches: the grids of a class are dealt round-robin (by step
 // count) into NGROUP groups, each its own branch of the graph, so one
 // group's round can fill the GPU while another's drains (the 256-grid batch:
@@ -71,7 +84,11 @@ struct MgGrid {
     // uniform k, per-round launches: a branch-free main pass that stores one
     // layer of periodic copies, then the boundary cells in a launch of its own
     int nbu, bu0;         // boundary-cell units (256 cells) and the first in its class
-    int pad;
+    // ghost-layer faces, per-round launches: two steps a launch, one block per
+    // (x tile, y tile, z chunk); an odd count takes its single step first
+    PairTiles pt;
+    int pzchunk, npblocks, pblock0;
+    int odd;
     long long steps;
 };
 
@@ -92,9 +109,10 @@ __device__ __forceinline__ void mg_unit(const MgGrid& sg, int u, long long step,
 }
 
 // Copy a descriptor into shared memory (all threads; callers synchronise).
+template <int THREADS = MG_THREADS>
 __device__ __forceinline__ void load_desc(MgGrid* dst, const MgGrid* src) {
     static_assert(sizeof(MgGrid) % 4 == 0, "copied as words");
-    for (int i = threadIdx.x; i < (int)(sizeof(MgGrid) / 4); i += MG_THREADS)
+    for (int i = threadIdx.x; i < (int)(sizeof(MgGrid) / 4); i += THREADS)
         reinterpret_cast<int*>(dst)[i] = reinterpret_cast<const int*>(src)[i];
 }
 
@@ -167,6 +185,33 @@ __global__ void __launch_bounds__(MG_THREADS)
         tout[i] = v;
 }
 
+// Two steps of every active grid of a ghost-layer class (per-cell k): the
+// two-step pass of one grid (sweep_pair_k), its tiles spread over the launch.
+template <typename S, bool PER, bool ADV>
+__global__ void __launch_bounds__(PAIR_THREADS, PairKCfg::BLOCKS)
+    mg_pair_k(const MgGrid* __restrict__ grids, const int* __restrict__ block_grid, int pass) {
+    __shared__ MgGrid sg;
+    __shared__ __align__(16) float sm[2 * (PairKCfg::R * PairKCfg::W + 2) * 128];
+    load_desc<PAIR_THREADS>(&sg, &grids[block_grid[blockIdx.x]]);
+    __syncthreads();
+    const int u = (int)blockIdx.x - sg.pblock0, t = sg.pt.gx * sg.pt.gy;
+    const int bz = u / t, by = (u - bz * t) / sg.pt.gx, bx = u - bz * t - by * sg.pt.gx;
+    const int z0 = bz * sg.pzchunk, b = (pass + sg.odd) & 1;
+    pair_k_run<S, PER, true, ADV, PairKCfg::R, PairKCfg::W>(sg.c, sg.tb[b], const_cast<void*>(sg.tb[b ^ 1]), sg.rk, sg.pt, bx,
+                                                            by, z0, min(z0 + sg.pzchunk, sg.c.n[2]), sm);
+}
+
+template <typename S>
+cudaError_t launch_pair(int kind, int blocks, const MgGrid* grids, const int* map, int pass, cudaStream_t st) {
+    switch (kind) {
+        case 3: mg_pair_k<S, false, false><<<blocks, PAIR_THREADS, 0, st>>>(grids, map, pass); break;
+        case 4: mg_pair_k<S, false, true><<<blocks, PAIR_THREADS, 0, st>>>(grids, map, pass); break;
+        case 5: mg_pair_k<S, true, false><<<blocks, PAIR_THREADS, 0, st>>>(grids, map, pass); break;
+        default: mg_pair_k<S, true, true><<<blocks, PAIR_THREADS, 0, st>>>(grids, map, pass); break;
+    }
+    return cudaGetLastError();
+}
+
 template <typename S>
 cudaError_t launch_kind(int kind, int blocks, const MgGrid* grids, const int* block_grid, long long step, int* status,
                         cudaStream_t st) {
@@ -174,7 +219,8 @@ cudaError_t launch_kind(int kind, int blocks, const MgGrid* grids, const int* bl
         case 0: mg_sweep<S, false, false, false><<<blocks, MG_THREADS, 0, st>>>(grids, block_grid, step, status); break;
         case 1: mg_sweep<S, true, false, false><<<blocks, MG_THREADS, 0, st>>>(grids, block_grid, step, status); break;
         case 2: mg_sweep<S, true, true, false><<<blocks, MG_THREADS, 0, st>>>(grids, block_grid, step, status); break;
-        case 3: mg_sweep<S, true, false, true><<<blocks, MG_THREADS, 0, st>>>(grids, block_grid, step, status); break;
+        case 3:
+        case 5: mg_sweep<S, true, false, true><<<blocks, MG_THREADS, 0, st>>>(grids, block_grid, step, status); break;
         default: mg_sweep<S, true, true, true><<<blocks, MG_THREADS, 0, st>>>(grids, block_grid, step, status); break;
     }
     return cudaGetLastError();
@@ -276,8 +322,8 @@ __device__ __forceinline__ void unit_dispatch(const MgGrid& sg, int u, long long
 
 // Class -> (storage, conductivity mode, advection, ghost-layer faces).
 template <int CLS> struct ClassOf {
-    using S = typename std::conditional<(CLS >= NKIND), __nv_bfloat16, float>::type;
-    static constexpr int kind = CLS % NKIND;
+    using S = typename std::conditional<(CLS >= PKIND), __nv_bfloat16, float>::type;
+    static constexpr int kind = CLS % PKIND;
     static constexpr bool kvar = kind != 0, adv = kind == 2 || kind == 4, ghost = kind >= 3;
 };
 
@@ -397,8 +443,8 @@ struct BatchCtx {
     cudaStream_t cap_stream = nullptr; // where per-round launches are captured
     cudaStream_t cls_stream[NBRANCH] = {};   // one branch per (class, group) inside the capture
     cudaEvent_t fork = nullptr, join[NBRANCH] = {};
-    int blocks[NCLASS + 1] = {};       // launch size per persistent kernel (index cls + 1)
-    cudaGraphExec_t exec[NCLASS + 1] = {};
+    int blocks[PNCLASS + 1] = {};      // launch size per persistent kernel (index cls + 1)
+    cudaGraphExec_t exec[PNCLASS + 1] = {};
     // a launch not waited for: its graph, an event behind it and its status word read back
     bool pending = false;
     cudaGraphExec_t pending_exec = nullptr;
@@ -547,10 +593,17 @@ int batch_launch(wfa_grid* gs, const long long* steps, int count, int slot, bool
         max_steps = std::max(max_steps, steps[i]);
     }
     if (order.empty()) return WFA_OK;
+    // WFA_BATCH_MODE: "rounds" (default: one launch per round and class,
+    // captured into one graph, a branch per class), "persistent" (one
+    // persistent kernel) or "stream" (the per-round launches issued in order
+    // on the stream)
+    const char* mode_env = getenv("WFA_BATCH_MODE");
+    const int mode = !mode_env ? 1 : !strcmp(mode_env, "persistent") ? 0 : !strcmp(mode_env, "stream") ? 2 : 1;
     // halos, held layers and 1/k of grids changed since their last step
     for (int i : order) {
         wfa_grid g = gs[i];
-        if (g->halo_dirty || g->thin[g->cur] == TWINS_NONE) {
+        const bool pairs = mode != 0 && g->r && g->thin[g->cur] == TWINS_ONE;   // the two-step pass reads 4 columns
+        if (g->halo_dirty || g->thin[g->cur] >= TWINS_NONE || pairs) {
             int rc = refresh_halo(g, g->cur);
             if (rc) return rc;
             rc = prepare_coeff_halo(g);
@@ -574,16 +627,23 @@ int batch_launch(wfa_grid* gs, const long long* steps, int count, int slot, bool
         b.rk = g->r ? g->r + off : nullptr;
         bool adv = false;
         for (int f = 0; f < 6; ++f) adv = adv || b.c.adv[f] != 0.0f;
-        const int kind = g->r ? (adv ? 2 : 1) + (b.c.halo_bc ? 2 : 0) : 0;
-        cls[k] = (g->storage == WFA_BF16 ? NKIND : 0) + kind;
+        int kind = g->r ? (adv ? 2 : 1) + (b.c.halo_bc ? 2 : 0) : 0;
+        if (mode == 0) {   // the persistent kernel's classes
+            cls[k] = (g->storage == WFA_BF16 ? PKIND : 0) + kind;
+        } else {
+            if (pair_kind(kind) && !pair_applies(g)) kind -= 2;
+            if (pair_kind(kind) && (b.c.periodic[0] || b.c.periodic[1] || b.c.periodic[2])) kind += 2;
+            cls[k] = (g->storage == WFA_BF16 ? NKIND : 0) + kind;
+        }
         b.ncx = (g->n[0] + 3) / 4;
         b.ncols = b.ncx * g->n[1];
-        // z chunks of about 16 planes (the 256-grid batch: 1% faster than 12,
-        // 1.2% than 8, 1.5% than 24), shorter (down to 4) while a grid has
+        // z chunks of about 16 planes with per-cell k (boundary cells in the pass)
+        // and 8 with uniform k, whose blocks are light (18 grids of 0.1 to 2.6 M
+        // cells: 302 GLUPS at 16, 310 at 8, 307 at 4); shorter while a grid has
         // fewer pairs than a block has threads
-        const int nz = g->n[2];
-        int nch = std::max((nz + 15) / 16, (MG_THREADS + b.ncols - 1) / b.ncols);
-        nch = std::max(1, std::min(nch, nz / 4));
+        const int nz = g->n[2], zq = g->r ? 16 : 8;
+        int nch = std::max((nz + zq - 1) / zq, (MG_THREADS + b.ncols - 1) / b.ncols);
+        nch = std::max(1, std::min(nch, g->r ? nz / 4 : nz / 2));
         b.zchunk = (nz + nch - 1) / nch;
         b.nch = (nz + b.zchunk - 1) / b.zchunk;
         const long long pairs = (long long)b.ncols * b.nch;
@@ -593,13 +653,8 @@ int batch_launch(wfa_grid* gs, const long long* steps, int count, int slot, bool
         }
         b.nblocks = (int)((pairs + MG_THREADS - 1) / MG_THREADS);
         b.steps = steps[order[k]];
+        b.pt = pair_k_tiles(b.c);
     }
-    // WFA_BATCH_MODE: "rounds" (default: one launch per round and class,
-    // captured into one graph, a branch per class), "persistent" (one
-    // persistent kernel) or "stream" (the per-round launches issued in order
-    // on the stream)
-    const char* mode_env = getenv("WFA_BATCH_MODE");
-    const int mode = !mode_env ? 1 : !strcmp(mode_env, "persistent") ? 0 : !strcmp(mode_env, "stream") ? 2 : 1;
     BatchCtx* c = context_for(st, slot);
     int rc = batch_wait(st, slot);   // a launch of this slot still in flight
     if (rc) return rc;
@@ -693,12 +748,48 @@ int batch_launch(wfa_grid* gs, const long long* steps, int count, int slot, bool
         std::vector<MgGrid> sorted(ng);
         long long total_blocks = 0;
         auto uniform_class = [](int t) { return (t / NGROUP) % NKIND == 0; };   // t: a branch
+        auto pair_class = [](int t) { return pair_kind((t / NGROUP) % NKIND); };
+        int dev = 0, sms = 1;
+        WFA_CUDA(cudaGetDevice(&dev));
+        WFA_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
         for (int t = 0; t < NBRANCH; ++t) {
-            long long b0 = 0, bu = 0;
+            long long b0 = 0, bu = 0, bp = 0;
+            // two-step passes: the z chunk length (4 to 64 planes) whose first round
+            // costs least, in waves of resident blocks (whole ones while there are
+            // few) times the planes a block steps
+            int zmax = 64;
+            if (pair_class(t) && cls_first[t] < cls_first[t + 1]) {
+                const double resident = (double)sms * PairKCfg::BLOCKS;
+                double best = 1e300;
+                for (int z = 64; z >= 4; z = z > 16 ? z * 7 / 8 : z - 1) {
+                    long long n = 0;
+                    int zc = 0;
+                    for (int j = cls_first[t]; j < cls_first[t + 1]; ++j) {
+                        const MgGrid& m = mg[idx[j]];
+                        const int nch = (m.c.n[2] + z - 1) / z;
+                        n += (long long)m.pt.gx * m.pt.gy * nch;
+                        zc = std::max(zc, (m.c.n[2] + nch - 1) / nch);
+                    }
+                    const double waves = n < 4 * resident ? ceil((double)n / resident) : (double)n / resident + 0.5;
+                    if (waves * (zc + 4) < 0.99 * best) {
+                        best = waves * (zc + 4);
+                        zmax = z;
+                    }
+                }
+            }
             for (int j = cls_first[t]; j < cls_first[t + 1]; ++j) {
                 MgGrid& m = sorted[j];
                 m = mg[idx[j]];
                 m.cls = t / NGROUP;
+                if (pair_class(t)) {
+                    const int nz = m.c.n[2], nch = (nz + zmax - 1) / zmax;
+                    m.odd = (int)(m.steps & 1);
+                    m.pzchunk = (nz + nch - 1) / nch;
+                    m.npblocks = m.pt.gx * m.pt.gy * ((nz + m.pzchunk - 1) / m.pzchunk);
+                    m.pblock0 = (int)bp;
+                    bp += m.npblocks;
+                    if (!m.odd) continue;   // no single step: no units
+                }
                 m.block0 = (int)b0;
                 b0 += m.nblocks;
                 if (uniform_class(t)) {   // boundary-cell units
@@ -712,11 +803,11 @@ int batch_launch(wfa_grid* gs, const long long* steps, int count, int slot, bool
                     bu += m.nbu;
                 }
             }
-            if (b0 > (1LL << 30) || bu > (1LL << 30)) {
+            if (b0 > (1LL << 30) || bu > (1LL << 30) || bp > (1LL << 30)) {
                 set_error("wfa_batch_run: too many blocks in one launch");
                 return WFA_ERR_ARG;
             }
-            total_blocks += b0 + bu;
+            total_blocks += b0 + bu + bp;
         }
         // device tables: the descriptors, then per class the block -> grid
         // maps (main units; for uniform k also boundary units)
@@ -731,9 +822,14 @@ int batch_launch(wfa_grid* gs, const long long* steps, int count, int slot, bool
             long long o = 0;
             for (int t = 0; t < NBRANCH; ++t) {
                 cls_map[t] = o;
-                for (int j = cls_first[t]; j < cls_first[t + 1]; ++j)
+                for (int j = cls_first[t]; j < cls_first[t + 1]; ++j) {
+                    if (pair_class(t) && !sorted[j].odd) continue;
                     for (int b = 0; b < sorted[j].nblocks; ++b) bmap[o++] = j;
+                }
                 cls_bmap[t] = o;
+                if (pair_class(t))
+                    for (int j = cls_first[t]; j < cls_first[t + 1]; ++j)
+                        for (int b = 0; b < sorted[j].npblocks; ++b) bmap[o++] = j;
                 if (uniform_class(t))
                     for (int j = cls_first[t]; j < cls_first[t + 1]; ++j)
                         for (int b = 0; b < sorted[j].nbu; ++b) bmap[o++] = j;
@@ -768,6 +864,24 @@ int batch_launch(wfa_grid* gs, const long long* steps, int count, int slot, bool
             cudaStream_t cs = mode == 1 ? c->cls_stream[t] : ls;
             if (mode == 1) e = cudaStreamWaitEvent(cs, c->fork, 0);
             int active = cls_first[t + 1];
+            if (pair_class(t)) {
+                // the odd counts' single steps together, then two steps a launch
+                const int type = t / NGROUP;
+                const int units = (int)(cls_bmap[t] - cls_map[t]);
+                if (units > 0) e = launch_class(type, units, dgrids, dmap + cls_map[t], 0, status, cs);
+                for (long long ps = 0; 2 * ps < max_steps && e == cudaSuccess; ++ps) {
+                    while (active > cls_first[t] && sorted[active - 1].steps / 2 <= ps) --active;
+                    if (active == cls_first[t]) break;
+                    const MgGrid& last = sorted[active - 1];
+                    const int blocks = last.pblock0 + last.npblocks;
+                    e = type < NKIND ? launch_pair<float>(type, blocks, dgrids, dmap + cls_bmap[t], (int)(ps & 1), cs)
+                                     : launch_pair<__nv_bfloat16>(type - NKIND, blocks, dgrids, dmap + cls_bmap[t],
+                                                                  (int)(ps & 1), cs);
+                }
+                if (mode == 1 && e == cudaSuccess) e = cudaEventRecord(c->join[t], cs);
+                if (mode == 1 && e == cudaSuccess) e = cudaStreamWaitEvent(ls, c->join[t], 0);
+                continue;
+            }
             for (long long s = 0; s < max_steps && e == cudaSuccess; ++s) {
                 while (active > cls_first[t] && sorted[active - 1].steps <= s) --active;
                 if (active == cls_first[t]) break;
@@ -814,11 +928,21 @@ int batch_launch(wfa_grid* gs, const long long* steps, int count, int slot, bool
     }
     for (int k = 0; k < ng; ++k) {
         wfa_grid g = gs[order[k]];
+        const bool per = mg[k].c.periodic[0] || mg[k].c.periodic[1] || mg[k].c.periodic[2];
+        if (mode != 0 && pair_kind(cls[k] % NKIND)) {   // two steps a pass, an odd count's single step first
+            const long long odd = mg[k].steps & 1, pairs = mg[k].steps / 2;
+            g->cur = (int)((g->cur + odd + pairs) & 1);
+            // a single step writes every copy, a two-step pass 4 columns beyond the row ends
+            const unsigned char left = !per ? TWINS_FULL : mg[k].c.periodic[0] ? TWINS_X : TWINS_NONE;
+            g->thin[g->cur] = pairs ? left : TWINS_FULL;
+            if (odd + pairs >= 2) g->thin[1 - g->cur] = pairs >= 2 ? left : TWINS_FULL;
+            g->steps_done += mg[k].steps;
+            continue;
+        }
         g->cur = (int)((g->cur + mg[k].steps) & 1);
         // the persistent kernel and the per-cell-k passes write every periodic
         // copy (corners included); the per-round uniform-k passes one layer
-        const bool one_layer = mode != 0 && cls[k] % NKIND == 0 &&
-                               (mg[k].c.periodic[0] || mg[k].c.periodic[1] || mg[k].c.periodic[2]);
+        const bool one_layer = mode != 0 && cls[k] % NKIND == 0 && per;
         if (mg[k].steps >= 1) g->thin[g->cur] = one_layer ? TWINS_ONE : TWINS_FULL;
         if (mg[k].steps >= 2) g->thin[1 - g->cur] = one_layer ? TWINS_ONE : TWINS_FULL;
         g->steps_done += mg[k].steps;

@@ -276,14 +276,17 @@ __device__ __forceinline__ bool exchange_row(const HaloSpec& h, int z) {
 }
 
 // Dirichlet face whose ghost layer holds the halo cell c (outside the domain
-// on exactly one axis, and that axis not periodic), or -1.
+// on exactly one of the axes that are not periodic), or -1. Beyond a periodic
+// axis too: a ghost layer's copies (the two-step pass steps the cells one
+// column beyond a periodic face, whose neighbours across a Dirichlet face
+// these are).
 __device__ __forceinline__ int ghost_face(const HaloSpec& h, const int c[3]) {
     int face = -1, outside = 0;
     for (int a = 0; a < 3; ++a) {
+        if (h.periodic[a]) continue;
         if (c[a] < 0 || c[a] >= h.n[a]) {
             ++outside;
             face = 2 * a + (c[a] >= h.n[a]);
-            if (h.periodic[a]) face = -1;
         }
     }
     return outside == 1 && face >= 0 && h.dirichlet[face] ? face : -1;

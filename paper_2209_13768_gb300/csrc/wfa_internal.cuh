@@ -40,7 +40,7 @@ constexpr int INPLACE_VARIANT = 5;    // the one-step column-march kernel, bound
 constexpr int WIDE_VARIANT = 6;       // the one-step column-march kernel, 8 cells a thread (16 for bf16, uniform k)
 constexpr int PAIR_VARIANT = 7;       // two steps per pass in registers (uniform k)
 
-enum { TWINS_FULL = 0, TWINS_ONE = 1, TWINS_NONE = 2 };
+enum { TWINS_FULL = 0, TWINS_ONE = 1, TWINS_NONE = 2, TWINS_X = 3 };
 
 // NVTX range over one API call: a named span on a profiler's timeline
 // (nothing happens unless a tool is attached).
@@ -149,7 +149,8 @@ struct wfa_grid_s {
     cudaEvent_t xev;      // orders plane exchanges against this grid's stream (wfa_exchange)
     unsigned char thin[2];   // periodic copies each buffer holds: TWINS_FULL every layer, TWINS_ONE
                              // one layer without corners (a thin column pass wrote it: enough for
-                             // one-step kernels), TWINS_NONE stale (the two-step pass wraps its reads)
+                             // one-step kernels), TWINS_NONE stale (the two-step pass wraps its reads),
+                             // TWINS_X 4 columns beyond the row ends only (the two-step pass, ragged rows)
 };
 
 namespace wfa {
@@ -168,6 +169,7 @@ inline bool has_exchange_face(const wfa_grid_s* g) {
 int build_coef(const wfa_grid_s* g, SweepCoef* c);       // host: fp64 -> fp32 coefficients
 int refresh_halo(wfa_grid_s* g, int buf);                 // twins + held layers of one buffer
 int launch_sweep(wfa_grid_s* g, long long nsteps);        // advance nsteps on g->stream
+bool pair_applies(const wfa_grid_s* g);                   // the two-step passes take this grid
 int check_status(wfa_grid_s* g);                          // sync + report a device-side timeout
 int autotune(wfa_grid_s* g, int* depth, int* variant);    // pick the fastest kernel configuration
 int prepare_coeff_halo(wfa_grid_s* g);                    // k periodic twins, then 1/k

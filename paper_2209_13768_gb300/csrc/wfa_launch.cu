@@ -228,7 +228,7 @@ static void tune_save_locked() {
 // Dirichlet values that the halo's ghost cells hold exactly, with per-cell k
 // no zero-flux face that meets advection (see halo_bc in build_coef), and
 // rows of at least 8 cells (a group across a periodic face wraps once).
-static bool pair_applies(const wfa_grid_s* g) {
+bool pair_applies(const wfa_grid_s* g) {
     if (g->n[0] < 8) return false;
     const bool adv = g->u[0] != 0.0 || g->u[1] != 0.0 || g->u[2] != 0.0;
     for (int f = 0; f < 6; ++f) {
@@ -255,11 +255,11 @@ static bool pair_applies(const wfa_grid_s* g) {
 //   uniform k, periodic axes: wrapped reads are slower, and a column march
 //     without faces is one launch: 128^3 7.8 / 5.3 to 7.4, 160^3 9.6 / 9.3 to
 //     10.9, 640x500x333 96 / 144, 1024x1024x512 401 / 728; ragged periodic
-//     rows read the two end tiles cell by cell: 90x90x400 18 / 12;
+//     rows store copies cell by cell: 90x90x400 14.6 / 12.3, 333x250x187 39 / 37;
 //   per-cell k, no periodic axis: 80^3 3.8 / 3.3, 100^3 4.0 / 5.2, 128^3 4.9 /
 //     6.2, 31x200x160 4.6 / 6.4, 333x250x187 33 / 42, 512^3 213 / 267;
-//   per-cell k, periodic axes: 128^3 8.4 / 6.7, 160^3 11.2 / 13.2, 512^3 232 /
-//     285; ragged periodic rows 333x250x187 65 / 48.
+//   per-cell k, periodic axes: 128^3 8.4 / 6.7, 160^3 11.2 / 13.2, 333x250x187
+//     42 / 48, 512^3 232 / 285.
 static Choice default_choice(const wfa_grid_s* g) {
     const long long cells = (long long)g->n[0] * g->n[1] * g->n[2];
     const bool perx = g->bc_kind[0] == WFA_BC_PERIODIC;
@@ -267,7 +267,7 @@ static Choice default_choice(const wfa_grid_s* g) {
     const Choice one{COL_VARIANT, 1}, two{PAIR_VARIANT, 2};
     if (!pair_applies(g)) return one;
     if (per) {
-        const bool wide = !perx || g->n[0] % 4 == 0 ? g->k || g->n[0] >= 100 : g->n[0] >= (g->k ? 960 : 480);
+        const bool wide = g->k || g->n[0] >= (perx && g->n[0] % 4 ? 480 : 100);
         return wide && cells >= (1LL << 22) ? two : one;
     }
     if (g->k) return cells >= 900000 ? two : one;
@@ -359,17 +359,22 @@ static int pass_launches(const wfa_grid_s* g, const SweepCoef& c, int depth, int
     return 1;
 }
 
+// The two-step pass reads the copies beyond the ends of periodic rows that are
+// no whole number of 4-cell groups (elsewhere it wraps).
+static bool pair_reads_copies(const wfa_grid_s* g) { return g->bc_kind[0] == WFA_BC_PERIODIC && g->n[0] % 4 != 0; }
+
 // The pass reads periodic copies that buffer `buf` does not hold: the tiled
-// kernels read every layer, the one-step kernels one, the two-step one none.
+// kernels read every layer, the one-step kernels one.
 static bool lacks_twins(const wfa_grid_s* g, int buf, int depth, int variant) {
-    if (two_step_variant(variant) && depth == 2) return false;
-    if (variant >= 1 && variant <= NUM_TILE_VARIANTS) return g->thin[buf] != TWINS_FULL;
-    return g->thin[buf] == TWINS_NONE;
+    const int have = g->thin[buf];
+    if (two_step_variant(variant) && depth == 2) return pair_reads_copies(g) && (have == TWINS_ONE || have == TWINS_NONE);
+    if (variant >= 1 && variant <= NUM_TILE_VARIANTS) return have != TWINS_FULL;
+    return have == TWINS_NONE || have == TWINS_X;
 }
 // The periodic copies a pass leaves in the buffer it writes.
-static unsigned char twins_written(const SweepCoef& c, int depth, int variant) {
+static unsigned char twins_written(const wfa_grid_s* g, const SweepCoef& c, int depth, int variant) {
     if (!c.periodic[0] && !c.periodic[1] && !c.periodic[2]) return TWINS_FULL;
-    if (two_step_variant(variant)) return depth == 2 ? TWINS_NONE : TWINS_ONE;
+    if (two_step_variant(variant)) return depth != 2 ? TWINS_ONE : pair_reads_copies(g) ? TWINS_X : TWINS_NONE;
     return variant == COL_VARIANT || variant == WIDE_VARIANT ? TWINS_ONE : TWINS_FULL;
 }
 
@@ -380,7 +385,7 @@ static int one_pass(wfa_grid_s* g, const SweepCoef& c, int depth, int variant, i
         const int rc = refresh_halo(g, g->cur);
         if (rc) return rc;
     }
-    g->thin[1 - g->cur] = twins_written(c, depth, variant);
+    g->thin[1 - g->cur] = twins_written(g, c, depth, variant);
     g->launches += pass_launches(g, c, depth, variant);
     SweepArgs a = base_args(g, c, g->cur, zc);
     const cudaEvent_t* ev = timing_slot(g);
@@ -558,7 +563,7 @@ int launch_sweep(wfa_grid_s* g, long long nsteps) {
         }
         g->launches += runs * GRAPH_PASSES * pass_launches(g, c, ch.depth, ch.variant);
         nsteps -= runs * GRAPH_PASSES * ch.depth;
-        g->thin[0] = g->thin[1] = twins_written(c, ch.depth, ch.variant);   // both written by the run
+        g->thin[0] = g->thin[1] = twins_written(g, c, ch.depth, ch.variant);   // both written by the run
     }
     while (nsteps > 0) {
         const int d = (int)std::min<long long>(ch.depth, nsteps);

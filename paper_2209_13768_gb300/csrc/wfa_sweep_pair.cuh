@@ -37,8 +37,9 @@
 // others the same body with weights, self terms and ghost rows chosen by
 // select (no branch inside a row: branches there cost 40%). A Dirichlet value
 // comes from the halo's ghost layer, a zero-flux face has weight 0. Periodic
-// axes wrap the rows and planes that are read, so no copies are stored: after
-// this pass a buffer's periodic copies are stale (TWINS_NONE). The fixed
+// axes wrap the rows, planes and groups that are read, so no copies are
+// stored (ragged rows: the 4 columns beyond a row's ends only) and a buffer's
+// other periodic copies are stale after this pass (TWINS_NONE, TWINS_X). The fixed
 // per-cell expression is that of every other kernel, rounded to the storage
 // type after each step, so a pass gives bitwise the field of two single
 // steps.
@@ -100,24 +101,11 @@ template <typename S> struct RowBuf;
 template <> struct RowBuf<float> {
     float4 q;
     __device__ __forceinline__ void load(const char* p) { q = __ldg(reinterpret_cast<const float4*>(p)); }
-    // cell by cell, byte offsets o[i] from p
-    __device__ __forceinline__ void gather(const char* p, const int (&o)[4]) {
-        q.x = __ldg(reinterpret_cast<const float*>(p + o[0]));
-        q.y = __ldg(reinterpret_cast<const float*>(p + o[1]));
-        q.z = __ldg(reinterpret_cast<const float*>(p + o[2]));
-        q.w = __ldg(reinterpret_cast<const float*>(p + o[3]));
-    }
     __device__ __forceinline__ void get(f2 (&o)[2]) const { o[0] = f2_make(q.x, q.y); o[1] = f2_make(q.z, q.w); }
 };
 template <> struct RowBuf<__nv_bfloat16> {
     uint2 q;
     __device__ __forceinline__ void load(const char* p) { q = __ldg(reinterpret_cast<const uint2*>(p)); }
-    __device__ __forceinline__ void gather(const char* p, const int (&o)[4]) {
-        unsigned v[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) v[i] = __ldg(reinterpret_cast<const unsigned short*>(p + o[i]));
-        q = make_uint2(v[0] | v[1] << 16, v[2] | v[3] << 16);
-    }
     __device__ __forceinline__ void get(f2 (&o)[2]) const { o[0] = unpack2(q.x); o[1] = unpack2(q.y); }
 };
 template <typename S> __device__ __forceinline__ f2 round2(f2 v) {
@@ -210,6 +198,17 @@ __device__ __forceinline__ void pair_put(const float (&o)[4], int left, char* p)
             if (i < left) reinterpret_cast<S*>(p)[i] = from_f32<S>(o[i]);
     }
 }
+// The copies of the first and last 4 cells of a row one period (n_x cells) away.
+template <typename S>
+__device__ __forceinline__ void pair_put_copies(const float (&o)[4], int gx, int nx, char* p) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int x = gx + i;
+        if (x < 4 && x < nx) reinterpret_cast<S*>(p)[i + nx] = from_f32<S>(o[i]);
+        if (x < nx && x >= nx - 4) reinterpret_cast<S*>(p)[i - nx] = from_f32<S>(o[i]);
+    }
+}
+
 // PER: some axis is periodic. RAG: n_x is not a multiple of 4 (a row's last
 // group holds cells beyond the face).
 template <typename S, bool PER, bool RAG, int R, int WPB, int BLOCKS>
@@ -224,23 +223,10 @@ __global__ void __launch_bounds__(32 * WPB, BLOCKS) sweep_pair(const __grid_cons
     const int z0 = blockIdx.z * a.zchunk, z1 = min(z0 + a.zchunk, nz);
     const bool perx = PER && c.periodic[0], pery = PER && c.periodic[1], perz = PER && c.periodic[2];
     const long long sy = c.sy * E, sz = c.sz * E;
-    // Where this lane's group is read: across a periodic x face one period
-    // away (cell by cell where that is no group of the row: `split`), beyond
-    // a row's end otherwise from its halo.
-    int lx = min(gx, (nx + 3) & ~3);
-    bool split = false;
-    int off[4] = {0, E, 2 * E, 3 * E};
-    if (perx) {
-        lx = gx < 0 ? gx + nx : gx < nx ? gx : min(gx - nx, nx);
-        if (RAG) {
-            split = gx < 0 || gx + 4 > nx;
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int x = lx + i;
-                off[i] = (x >= nx ? x - nx : x) * E;
-            }
-        }
-    }
+    // Where this lane's group is read: beyond a row's end from its halo; across
+    // a periodic x face one period away, or (where a period is no whole number
+    // of groups) from the halo's copies, which the RAG passes store
+    const int lx = !RAG && perx ? (gx < 0 ? gx + nx : gx < nx ? gx : min(gx - nx, nx)) : min(gx, (nx + 3) & ~3);
     const char* const tX = reinterpret_cast<const char*>((const S*)a.tin);   // cell (0, 0, 0)
     const char* tP = tX + (long long)lx * E + y0 * sy + (z0 - 1) * sz;       // this lane's group, row y0, plane q
     char* oP = reinterpret_cast<char*>((S*)a.tout) + (long long)gx * E + y0 * sy + (z0 - 2) * sz;
@@ -259,11 +245,11 @@ __global__ void __launch_bounds__(32 * WPB, BLOCKS) sweep_pair(const __grid_cons
     w.zm = f2_make(c.w_in[4], c.w_in[4]);
     w.nzp = f2_make(-c.w_in[5], -c.w_in[5]);
     const bool mine = lane >= 1 && lane <= 30 && gx < nx;   // this lane's cells are stored
-    // edge body: a row of the tile or its ring on or beyond a y face, (zero-flux
-    // faces with advection) a cell of the tile or its ring on an x face, or
-    // (ragged rows) a group that a periodic x face splits
+    // edge body: a row of the tile or its ring on or beyond a y face, or
+    // (zero-flux faces with advection) a cell of the tile or its ring on an x face
     const bool x_tile = blockIdx.x == 0 || (int)(blockIdx.x + 1) * PAIR_TX + 4 >= nx - 1;
-    const bool edge_xy = y0 <= 1 || y0 + R >= ny - 1 || (c.any_self && !perx && x_tile) || (RAG && perx && x_tile);
+    const bool edge_xy = y0 <= 1 || y0 + R >= ny - 1 || (c.any_self && !perx && x_tile);
+    const bool copies = RAG && perx && mine && (gx < 4 || gx + 3 >= nx - 4);   // its cells have x copies
 
     // rows y0-1 .. y0+R: T at plane q and the rows beyond (H), at q + 1,
     // T(q - 1) - T(q) (D); the same for the first step's field S (planes q - 1, q)
@@ -279,9 +265,7 @@ __global__ void __launch_bounds__(32 * WPB, BLOCKS) sweep_pair(const __grid_cons
         int y = y0 + j;
         if (pery) y = y < 0 ? y + ny : y >= ny ? y - ny : y;
         if (perz) z = z < 0 ? z + nz : z >= nz ? z - nz : z;
-        const char* const row = tX + y * sy + z * sz;
-        if (RAG && split) t.gather(row, off);
-        else t.load(row + (long long)lx * E);
+        t.load(tX + (long long)lx * E + y * sy + z * sz);
     };
 #pragma unroll
     for (int j = 0; j < R + 2; ++j) {
@@ -382,6 +366,7 @@ __global__ void __launch_bounds__(32 * WPB, BLOCKS) sweep_pair(const __grid_cons
                 f2_get(f2_add(Sc[j][0], acc[0]), o[0], o[1]);
                 f2_get(f2_add(Sc[j][1], acc[1]), o[2], o[3]);
                 if (mine && y < ny) pair_put<S, RAG>(o, nx - gx, oP + (j - 1) * sy);
+                if (RAG && PER && copies && y < ny) pair_put_copies<S>(o, gx, nx, oP + (j - 1) * sy);
 #pragma unroll
                 for (int i = 0; i < 2; ++i) {
                     DS[j - 1][i] = fz[i];

@@ -87,13 +87,12 @@ struct PairTiles {
     int gx, gy;       // tiles along x and y
     int sx, sy;       // cells and rows from one tile to the next
 };
-template <typename Cfg> __host__ __device__ inline PairTiles pair_tiles(const SweepCoef& c) {
+__host__ __device__ inline PairTiles pair_k_tiles(const SweepCoef& c) {
     PairTiles t;
     const int per = c.periodic[0] ? 8 : 0;   // ring cells beyond the row's ends
     t.lx = c.n[0] + per <= 32 ? 8 : c.n[0] + per <= 64 ? 16 : 32;
-    const int rows = Cfg::R * Cfg::W * (32 / t.lx);
     t.sx = 4 * t.lx - 8;
-    t.sy = rows - 2;
+    t.sy = PairKCfg::R * PairKCfg::W * (32 / t.lx) - 2;
     const int ex = c.n[0] + per - 8, ey = c.n[1] + (c.periodic[1] ? 0 : -2);
     t.gx = ex <= t.sx ? 1 : (ex + t.sx - 1) / t.sx;
     t.gy = ey <= t.sy ? 1 : (ey + t.sy - 1) / t.sy;
@@ -115,20 +114,7 @@ __device__ __forceinline__ void pair_k_run(const SweepCoef& c, const void* tin, 
     const int gx = bx * tl.sx + (perx ? -4 : 0) + 4 * xi;
     const int y0 = by * tl.sy + (pery ? -1 : 0) + r0;
     const long long sy = c.sy, sz = c.sz;   // elements
-    int lx = min(gx, (nx + 3) & ~3);
-    bool split = false;
-    int off[4] = {0, 1, 2, 3};
-    if (perx) {
-        lx = gx < 0 ? gx + nx : gx < nx ? gx : min(gx - nx, nx);
-        if (RAG) {
-            split = gx < 0 || gx + 4 > nx;
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int x = lx + i;
-                off[i] = x >= nx ? x - nx : x;
-            }
-        }
-    }
+    const int lx = !RAG && perx ? (gx < 0 ? gx + nx : gx < nx ? gx : min(gx - nx, nx)) : min(gx, (nx + 3) & ~3);
     const S* const tX = (const S*)tin;
     // rows past n_y + 1 (the last block's) are read as that row: never stored
     const int yl = min(y0, ny + 1);
@@ -138,6 +124,7 @@ __device__ __forceinline__ void pair_k_run(const SweepCoef& c, const void* tin, 
     // x faces: what lies beyond the row's ends (the value and 1/k of the ghost cell)
     const int el = perx ? -8 : nx - 1 - gx;
     const bool x_first = !perx && gx == 0, x_last = el == 3;
+    const float tb0 = c.tb[0], tb1 = c.tb[1];
     const float kg0 = c.bkind[0] == WFA_BC_DIRICHLET ? 0.0f : INFINITY, kg1 = c.bkind[1] == WFA_BC_DIRICHLET ? 0.0f : INFINITY;
     // rows this thread stores: inside its tile's ring, or at a face the tile ends at
     const bool mine_x = gx < nx && (xi >= 1 || x_first) && (xi <= LX - 2 || (!perx && gx + 4 >= nx));
@@ -147,8 +134,8 @@ __device__ __forceinline__ void pair_k_run(const SweepCoef& c, const void* tin, 
         const int r = r0 + j, y = y0 + j;
         if (mine_x && y < ny && (r >= 1 || (!pery && y == 0)) && (r <= rows - 2 || (!pery && y == ny - 1))) mine |= 1u << j;
     }
-    const bool x_tile = bx == 0 || (bx + 1) * tl.sx + 8 >= nx;
-    const bool edge_xy = __any_sync(0xffffffffu, y0 < 1 || y0 + R >= ny) || (RAG && perx && x_tile);
+    const bool edge_xy = __any_sync(0xffffffffu, y0 < 1 || y0 + R >= ny);
+    const bool copies = RAG && perx && (gx < 4 || gx + 3 >= nx - 4);   // its cells have x copies (see sweep_pair)
     float* const own = sm + (1 + r0) * 4 * LX + 4 * xi;       // row r0 of slot 0
     const int slot_f = (rows + 2) * 4 * LX;
     const f2 tcx = f2_make(c.tcd[0], c.tcd[0]), tcy = f2_make(c.tcd[1], c.tcd[1]), tcz = f2_make(c.tcd[2], c.tcd[2]);
@@ -170,15 +157,8 @@ __device__ __forceinline__ void pair_k_run(const SweepCoef& c, const void* tin, 
         if (pery) y = y < 0 ? y + ny : y >= ny ? y - ny : y;
         if (perz) z = z < 0 ? z + nz : z >= nz ? z - nz : z;
         const long long row = y * sy + z * sz;
-        if (RAG && split) {
-            const int to[4] = {off[0] * E, off[1] * E, off[2] * E, off[3] * E};
-            const int ko[4] = {off[0] * 4, off[1] * 4, off[2] * 4, off[3] * 4};
-            t.gather(reinterpret_cast<const char*>(tX + row), to);
-            k.gather(reinterpret_cast<const char*>(rk + row), ko);
-        } else {
-            t.load(reinterpret_cast<const char*>(tX + row + lx));
-            k.load(reinterpret_cast<const char*>(rk + row + lx));
-        }
+        t.load(reinterpret_cast<const char*>(tX + row + lx));
+        k.load(reinterpret_cast<const char*>(rk + row + lx));
     };
 #pragma unroll
     for (int j = 0; j < R; ++j) {
@@ -231,8 +211,8 @@ __device__ __forceinline__ void pair_k_run(const SweepCoef& c, const void* tin, 
             for (int j = 0; j < R; ++j) {
                 float xl = __shfl_up_sync(0xffffffffu, f2_hi(Sc[j][1]), 1, LX),
                       xr = __shfl_down_sync(0xffffffffu, f2_lo(Sc[j][0]), 1, LX);
-                xl = x_first ? c.tb[0] : xl;
-                xr = x_last ? c.tb[1] : xr;
+                xl = x_first ? tb0 : xl;
+                xr = x_last ? tb1 : xr;
                 f2 ym[2], yp[2], gm[2];
                 add_adv<ADV>(ym, WY[j], c.adv[2]);
                 add_adv<ADV>(yp, WY[j + 1], c.adv[3]);
@@ -266,8 +246,8 @@ __device__ __forceinline__ void pair_k_run(const SweepCoef& c, const void* tin, 
                       xr = __shfl_down_sync(0xffffffffu, f2_lo(t[0]), 1, LX);
                 float kl = __shfl_up_sync(0xffffffffu, f2_hi(k[1]), 1, LX),
                       kr = __shfl_down_sync(0xffffffffu, f2_lo(k[0]), 1, LX);
-                xl = x_first ? c.tb[0] : xl;
-                xr = x_last ? c.tb[1] : xr;
+                xl = x_first ? tb0 : xl;
+                xr = x_last ? tb1 : xr;
                 kl = x_first ? kg0 : kl;
                 kr = x_last ? kg1 : kr;
                 float k0, k1, k2, k3;
@@ -349,8 +329,10 @@ __device__ __forceinline__ void pair_k_run(const SweepCoef& c, const void* tin, 
             float o[4];
             f2_get(f2_add(Sc[j][0], f2_fma(gp[0], f2_sub(Sn[j][0], Sc[j][0]), acc2[j][0])), o[0], o[1]);
             f2_get(f2_add(Sc[j][1], f2_fma(gp[1], f2_sub(Sn[j][1], Sc[j][1]), acc2[j][1])), o[2], o[3]);
-            if ((mine >> j & 1u) && p >= z0)
+            if ((mine >> j & 1u) && p >= z0) {
                 pair_put<S, RAG>(o, nx - gx, reinterpret_cast<char*>(oP + j * sy));
+                if (RAG && PER && copies) pair_put_copies<S>(o, gx, nx, reinterpret_cast<char*>(oP + j * sy));
+            }
             float v[4];
             f2_get(Sn[j][0], v[0], v[1]);
             f2_get(Sn[j][1], v[2], v[3]);
@@ -420,7 +402,7 @@ inline int pair_k_chunk(int nz, long long tiles, long long resident) {
 template <typename S>
 cudaError_t pair_k_launch(const SweepArgs& a_in, cudaStream_t st, int nsm, const cudaEvent_t* ev) {
     SweepArgs a = a_in;
-    const PairTiles tl = pair_tiles<PairKCfg>(a.c);
+    const PairTiles tl = pair_k_tiles(a.c);
     a.zchunk = a_in.zchunk > 0 ? std::min(a_in.zchunk, a.c.n[2])
                                : pair_k_chunk(a.c.n[2], (long long)tl.gx * tl.gy, (long long)nsm * PairKCfg::BLOCKS);
     const dim3 grid(tl.gx, tl.gy, (a.c.n[2] + a.zchunk - 1) / a.zchunk);

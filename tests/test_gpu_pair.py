@@ -84,3 +84,27 @@ def test_faces_the_pair_pass_does_not_take():
         with make_grid(p, storage=storage) as g:
             g.set_tuning(2, 7)
             assert g.tuning()[0] == 1
+
+
+@pytest.mark.parametrize("storage", [wfa.F32, wfa.BF16])
+def test_batched_pairs_bitwise(storage):
+    """Batched rounds of two steps (per-cell k) at odd and even counts, row
+    widths on both sides of 8, 16 and 32 lanes a row, periodic axes and the
+    short rows that keep single steps; then again from where they stopped."""
+    probs = []
+    for i, (shape, faces) in enumerate([((7, 9, 8), "cold"), ((8, 5, 6), "torus"), ((24, 50, 9), "x"), ((25, 20, 9), "x"),
+                                        ((32, 47, 5), "walls"), ((33, 49, 12), "cold"), ((56, 24, 7), "torus"),
+                                        ((64, 23, 70), "cold"), ((65, 12, 9), "yz"), ((128, 13, 6), "cold"),
+                                        ((129, 12, 10), "walls"), ((131, 9, 8), "torus")]):
+        adv = faces in ("cold", "torus") and i % 2 == 0
+        probs.append(_problem(shape, faces, kvar=True, adv=adv, seed=i, steps=(i * 5) % 9 + (0 if i == 3 else 1)))
+    grids = [make_grid(p, storage=storage) for p in probs]
+    wfa.batch_run(grids, [p.steps for p in probs])
+    for p, g in zip(probs, grids):
+        np.testing.assert_array_equal(g.read_field(), run_gpu(p, storage=storage, variant=-1), err_msg=str(p.shape))
+    wfa.batch_run(grids, [5] * len(grids))
+    for p, g in zip(probs, grids):
+        g.step(2)
+        np.testing.assert_array_equal(g.read_field(), run_gpu(p, steps=p.steps + 7, storage=storage, variant=-1),
+                                      err_msg=str(p.shape))
+        g.close()
