@@ -462,12 +462,14 @@ def cg_kernel_hash():
     return h.hexdigest()[:16]
 
 
-def cg_bytes_per_cell(kvar):
-    """Algorithmic HBM bytes per cell per CG iteration: cg_spmv reads r and
-    p_old and writes p and q (16 B, + 4 B of 1/k for per-cell k); cg_update
-    reads x, p, q, r and writes x, r (24 B). The pipelined kernel moves the
-    same 40 B (+4): reads r, w, s, p, x, writes them."""
-    return 40 + (4 if kvar else 0)
+def cg_bytes_per_cell(kvar, method="classic"):
+    """Algorithmic HBM bytes per cell per CG iteration: cg_dir reads r, p_old
+    and x and writes p and x (20 B; per-cell k reads 1/k and writes q too: 28
+    B); cg_res reads p (per-cell k: q) and r and writes r (12 B). The pipelined
+    kernel reads r, w, s, p, x and writes them: 40 B (+4 of 1/k)."""
+    if method == "pipelined":
+        return 44 if kvar else 40
+    return 40 if kvar else 32
 
 
 def implicit_bench(args, rank, world, dist):
@@ -512,7 +514,7 @@ def implicit_bench(args, rank, world, dist):
     total_s = sum(a.elapsed_time(b) for a, b in ev) / 1e3
     total_s = max_over_ranks(total_s, dist, "cuda")
     value = world * cells * iters / total_s / 1e9
-    bpc = cg_bytes_per_cell(kvar)
+    bpc = cg_bytes_per_cell(kvar, args.cg)
     achieved = bpc * cells * iters / total_s / 1e9
     peaks = {}
     try:
@@ -521,7 +523,7 @@ def implicit_bench(args, rank, world, dist):
     except OSError:
         pass
     peak = peaks.get("hbm_gbs", 6800.0)
-    traffic = None   # DRAM bytes of one CG iteration (cg_spmv + cg_update) from ncu, if current
+    traffic = None   # DRAM bytes of one CG iteration (cg_dir + cg_res) from ncu, if current
     try:
         with open(TRAFFIC_FILE) as f:
             ent = json.load(f).get(f"implicit:{'k' if kvar else 'u'}:cg_iteration")
@@ -577,9 +579,9 @@ def implicit_bench(args, rank, world, dist):
                              "frac": achieved / peak, "traffic": traffic, "traffic_unit": "bytes per CG iteration",
                              "peak_source": "measured" if "hbm_gbs" in peaks else "fallback",
                              "bytes_per_cell_per_iteration": bpc, "frac_of_nominal_8TBps": achieved / 8000.0,
-                             "scope": "the whole solve: every kernel of the timed steps (cg_init, cg_spmv, "
-                                      "cg_update and the loop-control kernels; pipelined: cg_init, cg_spmv once a "
-                                      "step, cg_pipe), one graph launch a call"},
+                             "scope": "the whole solve: every kernel of the timed steps (cg_init, cg_dir, "
+                                      "cg_res, cg_xfin and the loop-control kernels; pipelined: cg_init, cg_dir once "
+                                      "a step, cg_pipe), one graph launch a call"},
                 "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": gpu_launches, "clocks": clocks}
         print(json.dumps(line), flush=True)
 

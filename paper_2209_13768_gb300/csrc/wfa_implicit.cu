@@ -16,15 +16,19 @@
 //
 // GB300 mapping. The field x is the grid's fp32 buffer, updated in place;
 // r, p (two buffers) and q are fp32 work vectors in the same padded layout.
-// Each iteration is two HBM-bound kernels:
-//   cg_spmv   p = r + beta p_old on the fly (for the cell and its six
-//             neighbours), q = A p, and the block partials of p.q; reads r and
-//             p_old, writes p and q (16 B a cell, + 4 B of 1/k for per-cell k);
-//   cg_update x += alpha p, r -= alpha q, and the block partials of r.r
-//             (reads x, p, q, r, writes x, r: 24 B a cell).
-// The last block of each kernel to finish (an atomic ticket, no waiting) sums
-// the partials in a fixed order and computes alpha (resp. beta and the
-// convergence test) on the device, so no host round trip sits between
+// Each iteration is two HBM-bound kernels and a one-block control kernel:
+//   cg_dir    p = r + beta p_old on the fly (for the cell and its six
+//             neighbours), the block partials of p.(A p), and the x += alpha p
+//             of the iteration before (its p is read here anyway); reads r,
+//             p_old and x, writes p and x (20 B a cell); per-cell k: reads 1/k
+//             and writes q = A p too (28 B);
+//   cg_res    r -= alpha q and the block partials of r.r: uniform k forms
+//             q = A p again (cg_res_u: reads p and r, writes r, 12 B), per-cell
+//             k reads it (cg_res_k: q and r, writes r, 12 B);
+//   cg_ctl_iter  r.r, beta and the convergence test from the partials.
+// 32 B a cell and iteration (40 with per-cell k); storing q and updating x in
+// cg_res takes 40 (44). cg_xfin adds the last iteration's alpha p.
+// Every scalar is computed on the device, so no host round trip sits between
 // iterations: a whole call is one graph launch whose conditional WHILE nodes
 // loop over the time steps and the iterations (device loops, below); where
 // those cannot be built, captured runs of iterations are replayed with the
@@ -48,13 +52,16 @@
 #include <new>
 
 #include "wfa_internal.cuh"
+#include "wfa_sweep_pair.cuh"
 
 namespace wfa {
 
-constexpr int CG_TX = 16, CG_TY = 16;   // cg_spmv block: 64 x 16 cells, 4 x cells a thread
+constexpr int CG_TX = 16, CG_TY = 16;   // cg_init / cg_pipe block: 64 x 16 cells, 4 x cells a thread
 constexpr int CG_THREADS = 256;
+constexpr int CG_CTL = 512;             // threads of the one-block control kernels (16 warps: see block_sum)
 constexpr int CG_MAX_PART = 16384;      // per-block partials of one launch
-constexpr bool CG_SPMV_SM_DEFAULT = false;   // cg_spmv (L1 neighbours) unless WFA_CG_SPMV=sm
+constexpr int CG_FOLD = 512;            // most blocks of cg_dir whose partials every block of cg_res sums
+constexpr int CG_R = 2, CG_W = 4;       // cg_dir / cg_res_u: rows a thread, warps of a block
 constexpr int CG_NRUN = 4;              // captured runs of 1, 2, 4 and 8 iterations
 constexpr int CG_RUN_LEN[CG_NRUN] = {1, 2, 4, 8};
 
@@ -68,6 +75,7 @@ struct CgState {   // fits one 64-byte pinned word
     int iter;         // iterations of the current step
     int max_iter;
     unsigned ticket;  // blocks of the current launch that have finished
+    int pending;      // classic CG: x lacks the last iteration's alpha p (1), or only its periodic twins (2)
 };
 
 static_assert(sizeof(CgState) <= 64, "CgState is read back into a 64-byte pinned word");
@@ -92,14 +100,16 @@ struct CgArgs {
     float* p0;
     float* p1;
     float* q;
-    double* part;      // per-block partials (two arrays of CG_MAX_PART for cg_init)
+    double* part;      // per-block partials, two arrays of CG_MAX_PART: p.q and r.r (cg_init: r.r and b.b)
     CgState* s;
     float* r2;         // pipelined CG: second r, w and s buffers (r, w and s ping-pong, read at
     float* w2;         // neighbours: r in r / r2, w in q / w2, s in p1 / s2; p in p0)
     float* s2;
-    int zchunk;        // cg_spmv planes per block
+    int zchunk;        // planes per block
     int nblk;          // blocks of this launch
-    int q_twins;       // cg_spmv also writes q's periodic twins (q is the pipelined solver's first w)
+    int lanes;         // cg_dir / cg_res_u: threads side by side along x (32, 16 or 8)
+    int dblk;          // partials of p.q that cg_res sums itself (0: the last block of cg_dir has)
+    int q_twins;       // cg_dir also writes q's periodic twins (q is the pipelined solver's first w)
 };
 
 __device__ __forceinline__ long long cg_at(const CgCoef& c, int x, int y, int z) {
@@ -117,18 +127,6 @@ __device__ __forceinline__ bool cg_held_m(const CgCoef& c, int x, int y, int z) 
     return ((FM & 1) && c.held[0] && x == 0) || ((FM & 2) && c.held[1] && x == c.n[0] - 1) ||
            ((FM & 4) && c.held[2] && y == 0) || ((FM & 8) && c.held[3] && y == c.n[1] - 1) ||
            ((FM & 16) && c.held[4] && z == 0) || ((FM & 32) && c.held[5] && z == c.n[2] - 1);
-}
-
-__device__ __forceinline__ void prefetch_l2(const void* p) {
-    asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
-}
-
-__device__ __forceinline__ void sts4(float* p, const float v[4]) {
-    *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
-}
-__device__ __forceinline__ void lds4(const float* p, float v[4]) {
-    const float4 t = *reinterpret_cast<const float4*>(p);
-    v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
 }
 
 __device__ __forceinline__ void ld4(const float* p, float v[4]) {
@@ -175,8 +173,9 @@ struct KahanF {
     __device__ __forceinline__ double value() const { return (double)s - (double)c; }
 };
 
-// Block sum of one double per thread (fixed shuffle tree, then the warps in
-// order); the result is valid in thread 0.
+// Block sum of one double per thread (fixed shuffle trees: the warps, then the
+// first warp over their sums); the result is valid in thread 0. A dependent
+// fp64 add takes some 60 cycles here, so the chain is kept short.
 __device__ __forceinline__ double block_sum(double v, double* red) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
@@ -185,8 +184,10 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
     if ((tid & 31) == 0) red[tid >> 5] = v;
     __syncthreads();
     double t = 0.0;
-    if (tid == 0)
-        for (int w = 0; w < nw; ++w) t += red[w];
+    if (tid < 32) {
+        t = tid < nw ? red[tid] : 0.0;
+        for (int o = nw > 8 ? 8 : 4; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+    }
     __syncthreads();
     return t;
 }
@@ -200,6 +201,7 @@ __device__ __forceinline__ bool publish(const CgArgs& a, double* slot, double v,
         __threadfence();
         const unsigned t = atomicAdd(&a.s->ticket, 1u);
         *last = t == (unsigned)a.nblk - 1;
+        if (t == (unsigned)a.nblk - 1) __threadfence();
     }
     __syncthreads();
     return *last;
@@ -209,8 +211,8 @@ __device__ __forceinline__ bool publish(const CgArgs& a, double* slot, double v,
 __device__ __forceinline__ double sum_partials(const double* part, int n, double* red) {
     const int tid = threadIdx.x + threadIdx.y * blockDim.x;
     const int nt = blockDim.x * blockDim.y;
-    __threadfence();
     double t = 0.0;
+#pragma unroll 8
     for (int i = tid; i < n; i += nt) t += __ldcg(part + i);
     return block_sum(t, red);
 }
@@ -322,17 +324,15 @@ __device__ __forceinline__ void cg_r4(const CgCoef& c, const CgEdge& e, int gx, 
 
 // ---------------------------------------------------------------- cg_init --
 // r = b - A T (dt times the explicit step's accumulation), b.b and r.r, on
-// the column-march layout of cg_spmv (4 x cells a thread, z queue). The
+// a column-march layout (4 x cells a thread, z queue). The
 // field's periodic twins are current (refresh_halo before the first step,
-// cg_update after every iteration). b adds to T the known values: Dirichlet
+// cg_xfin after every step). b adds to T the known values: Dirichlet
 // faces and held neighbours. O32: every array is under 4 GiB, so the loop
 // addresses its planes by a 32-bit byte offset from the array's start (one
 // integer add an address); otherwise by a 64-bit one.
 template <bool KVAR, bool O32>
-__global__ void __launch_bounds__(CG_TX * CG_TY, CgOcc<KVAR>::blocks) cg_init(const __grid_constant__ CgArgs a, double tol2,
-                                                                         int max_iter) {
+__global__ void __launch_bounds__(CG_TX * CG_TY, CgOcc<KVAR>::blocks) cg_init(const __grid_constant__ CgArgs a) {
     __shared__ double red[CG_TX * CG_TY / 32];
-    __shared__ bool last;
     const CgCoef& c = a.c;
     const float* __restrict__ xv = a.x;
     const float* __restrict__ rk = a.rk;
@@ -386,7 +386,7 @@ __global__ void __launch_bounds__(CG_TX * CG_TY, CgOcc<KVAR>::blocks) cg_init(co
             const bool inner_z = perz || (z > 1 && z < nz - 2);
             const bool fast = inner_xy && inner_z;
             const unsigned am = __activemask();
-            if (__all_sync(am, fast))   // warp-uniform choice, as in cg_spmv
+            if (__all_sync(am, fast))   // warp-uniform choice
                 cg_r4<KVAR, false>(c, edge, gx, gy, z, tc, tm, tp, ym, yp, xm, xp, kc, km, kp, kym, kyp, kxm, kxp, rv,
                                    sr, sb);
             else if (__all_sync(am, inner_y && inner_z))   // near an x face only
@@ -416,48 +416,13 @@ __global__ void __launch_bounds__(CG_TX * CG_TY, CgOcc<KVAR>::blocks) cg_init(co
     const int blk = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
     const double rs = block_sum(rr.value(), red);
     const double bsum = block_sum(bb.value(), red);
-    if (threadIdx.x == 0 && threadIdx.y == 0) a.part[CG_MAX_PART + blk] = bsum;
-    if (!publish(a, a.part + blk, rs, &last)) return;
-    const double R = sum_partials(a.part, a.nblk, red);
-    const double B = sum_partials(a.part + CG_MAX_PART, a.nblk, red);
-    if (threadIdx.x == 0 && threadIdx.y == 0) {
-        CgState* s = a.s;
-        s->rr = R;
-        s->bb = B;
-        s->alpha = 0.0;
-        s->beta = 0.0;
-        s->tol2 = tol2;
-        s->iter = 0;
-        s->max_iter = max_iter;
-        s->done = (R <= tol2 * B || max_iter <= 0 || !(R == R)) ? 1 : 0;
-        s->ticket = 0;
+    if (threadIdx.x == 0 && threadIdx.y == 0) {   // summed by cg_ctl_start
+        a.part[blk] = rs;
+        a.part[CG_MAX_PART + blk] = bsum;
     }
 }
 
-// ---------------------------------------------------------------- cg_spmv --
-// p(this iteration) = r + beta p(previous), formed for each cell where it is
-// read, so p is never re-read from DRAM after being written; q = A p.
-struct PNew {
-    const float* r;
-    const float* po;
-    float beta;
-    bool first;   // first iteration: p = r
-};
-
-__device__ __forceinline__ void pnew4(const PNew& P, long long o, float v[4]) {
-    ld4(P.r + o, v);
-    if (!P.first) {
-        float w[4];
-        ld4(P.po + o, w);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) v[i] = __fmaf_rn(P.beta, w[i], v[i]);
-    }
-}
-__device__ __forceinline__ float pnew1(const PNew& P, long long o) {
-    const float v = __ldg(P.r + o);
-    return P.first ? v : __fmaf_rn(P.beta, __ldg(P.po + o), v);
-}
-
+// ---------------------------------------------------------------- q = A p --
 // q = A p for the 4 cells of a thread at plane z, and their p.q (cells inside
 // the domain). EDGE (chosen warp-uniformly) puts ghost values across
 // boundary faces and masks held cells and cells beyond the x end; without
@@ -521,273 +486,425 @@ __device__ __forceinline__ float cg_q4(const CgCoef& c, const CgEdge& e, int gx,
     return psum;
 }
 
+// Row operands of a thread: 4 cells of two rows as pairs.
+__device__ __forceinline__ void ldp(const float* p, f2 (&v)[2]) {
+    const float4 t = __ldg(reinterpret_cast<const float4*>(p));
+    v[0] = f2_make(t.x, t.y);
+    v[1] = f2_make(t.z, t.w);
+}
+__device__ __forceinline__ void unp(const f2 (&v)[2], float o[4]) {
+    f2_get(v[0], o[0], o[1]);
+    f2_get(v[1], o[2], o[3]);
+}
+// v = r + beta p_old, both as loaded. On the first iteration p_old is r itself
+// and beta 0, so that no load waits behind a branch.
+__device__ __forceinline__ void pnew_pairs(const float4& r, const float4& o, f2 beta, f2 (&v)[2]) {
+    v[0] = f2_fma(beta, f2_make(o.x, o.y), f2_make(r.x, r.y));
+    v[1] = f2_fma(beta, f2_make(o.z, o.w), f2_make(r.z, r.w));
+}
+__device__ __forceinline__ float4 ldv(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
+__device__ __forceinline__ f2 lo2(const float4& v) { return f2_make(v.x, v.y); }
+__device__ __forceinline__ f2 hi2(const float4& v) { return f2_make(v.z, v.w); }
+
+// q = A p of one interior row (every neighbour a free cell), cg_q4's
+// expression on pairs; uniform k.
+__device__ __forceinline__ void cg_row_u(const CgCoef& c, const f2 (&pc)[2], const f2 (&pm)[2], const f2 (&pp)[2],
+                                         const f2 (&ym)[2], const f2 (&yp)[2], float xm, float xp, f2 (&q)[2]) {
+    float v[4];
+    unp(pc, v);
+    const f2 n0 = f2_make(-c.cu[0], -c.cu[0]), n1 = f2_make(-c.cu[1], -c.cu[1]), n2 = f2_make(-c.cu[2], -c.cu[2]);
+    const f2 x[2] = {f2_make(__fadd_rn(xm, v[1]), __fadd_rn(v[0], v[2])), f2_make(__fadd_rn(v[1], v[3]), __fadd_rn(v[2], xp))};
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        f2 acc = f2_mul(f2_make(c.du, c.du), pc[i]);
+        acc = f2_fma(n0, x[i], acc);
+        acc = f2_fma(n1, f2_add(ym[i], yp[i]), acc);
+        q[i] = f2_fma(n2, f2_add(pm[i], pp[i]), acc);
+    }
+}
+// Per-cell k: gm / gp the faces below and above the row, zm / zp along z.
+__device__ __forceinline__ void cg_row_k(const CgCoef& c, const f2 (&pc)[2], const f2 (&pm)[2], const f2 (&pp)[2],
+                                         const f2 (&ym)[2], const f2 (&yp)[2], float xm, float xp, const f2 (&kc)[2],
+                                         float kxm, float kxp, const f2 (&gm)[2], const f2 (&gp)[2], const f2 (&zm)[2],
+                                         const f2 (&zp)[2], f2 (&q)[2]) {
+    float v[4], k[4];
+    unp(pc, v);
+    unp(kc, k);
+    const float x0 = face_r(kxm, k[0], c.tcd[0]), x1 = face_r(k[0], k[1], c.tcd[0]), x2 = face_r(k[1], k[2], c.tcd[0]),
+                x3 = face_r(k[2], k[3], c.tcd[0]), x4 = face_r(k[3], kxp, c.tcd[0]);
+    f2 acc[2];
+    acc[0] = f2_mul(f2_make(x0, x1), f2_make(__fsub_rn(v[0], xm), __fsub_rn(v[1], v[0])));
+    acc[1] = f2_mul(f2_make(x2, x3), f2_make(__fsub_rn(v[2], v[1]), __fsub_rn(v[3], v[2])));
+    acc[0] = f2_fma(f2_make(x1, x2), f2_make(__fsub_rn(v[0], v[1]), __fsub_rn(v[1], v[2])), acc[0]);
+    acc[1] = f2_fma(f2_make(x3, x4), f2_make(__fsub_rn(v[2], v[3]), __fsub_rn(v[3], xp)), acc[1]);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        acc[i] = f2_fma(gm[i], f2_sub(pc[i], ym[i]), acc[i]);
+        acc[i] = f2_fma(gp[i], f2_sub(pc[i], yp[i]), acc[i]);
+        acc[i] = f2_fma(zm[i], f2_sub(pc[i], pm[i]), acc[i]);
+        acc[i] = f2_fma(zp[i], f2_sub(pc[i], pp[i]), acc[i]);
+        q[i] = f2_add(pc[i], acc[i]);
+    }
+}
+
+// What a thread of cg_dir / cg_res_u covers: 4 x cells of CG_R rows; a.lanes
+// (32, 16 or 8) threads lie side by side along x, so narrow grids fill their warps.
+struct CgPlace {
+    int gx, gy;            // first cell and row
+    long long row;         // its place in memory at plane 0 (threads beyond a row or the rows read its halo)
+    int lane, lanes;       // position along x, shuffle width
+    bool rows, in;         // some row of the warp, some cell of the thread inside the domain
+    bool ends;             // first or last lane: its outer x neighbour is another thread group's
+    int eo;                // that neighbour's offset from the first cell
+    bool inner_y;          // warp: every row away from the y faces
+    bool xlo, xhi;         // the thread's first / last cell lies on a (non-periodic) x face
+    bool ragged;           // warp: some thread's cells reach beyond the x end or into a held x layer
+    int ih;                // index of its cell on the +x face, 4 when none
+    unsigned dead;         // bit i: cell i is beyond the x end or in a held x layer
+    __device__ __forceinline__ CgPlace(const CgArgs& a) {
+        const CgCoef& c = a.c;
+        const int nx = c.n[0], ny = c.n[1];
+        lanes = a.lanes;
+        lane = threadIdx.x & (lanes - 1);
+        const int tile = blockDim.x / lanes;   // row groups of a block
+        gx = (blockIdx.x * lanes + lane) * 4;
+        gy = (blockIdx.y * tile + threadIdx.x / lanes) * CG_R;
+        row = min(gx, (nx + 3) & ~3) + (long long)min(gy, ny) * c.sy;
+        in = gx < nx && gy < ny;
+        rows = __any_sync(0xffffffffu, in);
+        ends = lane == 0 || lane == lanes - 1;
+        eo = lane == 0 ? -1 : 4;
+        const bool iy = gy + CG_R <= ny && (c.periodic[1] || (gy > 0 && gy + CG_R < ny));
+        inner_y = __all_sync(0xffffffffu, !in || iy);
+        ih = !c.periodic[0] && gx < nx && nx - 1 - gx < 4 ? nx - 1 - gx : 4;
+        xlo = !c.periodic[0] && gx == 0;
+        xhi = ih == 3;
+        dead = 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (gx + i >= nx || (c.held[0] && gx + i == 0) || (c.held[1] && gx + i == nx - 1)) dead |= 1u << i;
+        ragged = __any_sync(0xffffffffu, dead != 0);
+    }
+};
+
+// q = A p of a thread's rows at plane z and their p.q. Away from the y and z
+// faces the pair form serves every warp: across an x face the neighbour is the
+// ghost value (cg_q4's) put in its place, and cells that are not free get
+// q = 0; next to a y or z face cg_q4 goes row by row. zf: the faces towards
+// z - 1 on entry, towards z + 1 on return; kz: 1/k of the first row at z - 1.
 template <bool KVAR>
-__global__ void __launch_bounds__(CG_TX * CG_TY, CgOcc<KVAR>::blocks) cg_spmv(const __grid_constant__ CgArgs a) {
-    __shared__ double red[CG_TX * CG_TY / 32];
+__device__ __forceinline__ float cg_rows(const CgCoef& c, const CgPlace& t, int z, f2 (&pc)[CG_R][2],
+                                         const f2 (&pm)[CG_R][2], const f2 (&pp)[CG_R][2], const f2 (&h)[2][2],
+                                         const float (&e)[CG_R], f2 (&kc)[KVAR ? CG_R : 1][2],
+                                         f2 (&zf)[KVAR ? CG_R : 1][2], const f2 (&kp)[KVAR ? CG_R : 1][2],
+                                         const f2 (&kh)[2][2], const float (&ke)[CG_R], const float* kz, f2 (&q)[CG_R][2]) {
+    constexpr unsigned FULL = 0xffffffffu;
+    const int ny = c.n[1], nz = c.n[2];
+    float xm[CG_R], xp[CG_R], kxm[CG_R], kxp[CG_R];
+    const float g0 = c.dface[0] ? -1.0f : 1.0f, g1 = c.dface[1] ? -1.0f : 1.0f;
+#pragma unroll
+    for (int j = 0; j < CG_R; ++j) {
+        const float u = __shfl_up_sync(FULL, f2_hi(pc[j][1]), 1, t.lanes);
+        const float d = __shfl_down_sync(FULL, f2_lo(pc[j][0]), 1, t.lanes);
+        xm[j] = t.lane == 0 ? e[j] : u;
+        xp[j] = t.lane == t.lanes - 1 ? e[j] : d;
+        xm[j] = t.xlo ? __fmul_rn(g0, f2_lo(pc[j][0])) : xm[j];
+        xp[j] = t.xhi ? __fmul_rn(g1, f2_hi(pc[j][1])) : xp[j];
+        kxm[j] = kxp[j] = 0.0f;
+        if (KVAR) {
+            const int jk = KVAR ? j : 0;
+            const float ku = __shfl_up_sync(FULL, f2_hi(kc[jk][1]), 1, t.lanes);
+            const float kd = __shfl_down_sync(FULL, f2_lo(kc[jk][0]), 1, t.lanes);
+            kxm[j] = t.lane == 0 ? ke[j] : ku;
+            kxp[j] = t.lane == t.lanes - 1 ? ke[j] : kd;
+            kxm[j] = t.xlo ? f2_lo(kc[jk][0]) : kxm[j];
+            kxp[j] = t.xhi ? f2_hi(kc[jk][1]) : kxp[j];
+        }
+    }
+    if (t.ragged) {   // the +x face inside the thread's cells: the ghost goes into the cell beyond it
+#pragma unroll
+        for (int j = 0; j < CG_R; ++j) {
+            float v[4], k[4];
+            unp(pc[j], v);
+            if (KVAR) unp(kc[KVAR ? j : 0], k);
+#pragma unroll
+            for (int i = 2; i >= 0; --i)
+                if (t.ih == i) {
+                    v[i + 1] = __fmul_rn(g1, v[i]);
+                    if (KVAR) k[i + 1] = k[i];
+                }
+            pc[j][0] = f2_make(v[0], v[1]);
+            pc[j][1] = f2_make(v[2], v[3]);
+            if (KVAR) {
+                kc[KVAR ? j : 0][0] = f2_make(k[0], k[1]);
+                kc[KVAR ? j : 0][1] = f2_make(k[2], k[3]);
+            }
+        }
+    }
+    const f2(&pr)[CG_R][2] = pc;
+    const f2(&kr)[KVAR ? CG_R : 1][2] = kc;
+    f2 gp[KVAR ? CG_R : 1][2];
+    if (KVAR) {
+        const f2 tz = f2_make(c.tcd[2], c.tcd[2]);
+#pragma unroll
+        for (int j = 0; j < (KVAR ? CG_R : 1); ++j)
+#pragma unroll
+            for (int i = 0; i < 2; ++i) gp[j][i] = pair_face(kc[j][i], kp[j][i], tz);
+    }
+    float s = 0.0f;
+    if (t.inner_y && (c.periodic[2] || (z > 0 && z < nz - 1))) {
+        f2 gy[2][2];
+        const f2 ty = f2_make(c.tcd[1], c.tcd[1]);
+        if (KVAR) {
+#pragma unroll
+            for (int i = 0; i < 2; ++i) gy[0][i] = pair_face(kh[0][i], kc[0][i], ty);
+        }
+        f2 d = f2_make(0.0f, 0.0f);
+#pragma unroll
+        for (int j = 0; j < CG_R; ++j) {
+            const int jk = KVAR ? j : 0;
+            const f2(&ym)[2] = j == 0 ? h[0] : pr[j > 0 ? j - 1 : 0];
+            const f2(&yp)[2] = j == CG_R - 1 ? h[1] : pr[j < CG_R - 1 ? j + 1 : 0];
+            if (KVAR) {
+                const f2(&kn)[2] = j == CG_R - 1 ? kh[1] : kr[KVAR && j < CG_R - 1 ? j + 1 : 0];
+#pragma unroll
+                for (int i = 0; i < 2; ++i) gy[1][i] = pair_face(kc[jk][i], kn[i], ty);
+                cg_row_k(c, pc[j], pm[j], pp[j], ym, yp, xm[j], xp[j], kc[jk], kxm[j], kxp[j], gy[0], gy[1], zf[jk], gp[jk],
+                         q[j]);
+#pragma unroll
+                for (int i = 0; i < 2; ++i) gy[0][i] = gy[1][i];
+            } else {
+                cg_row_u(c, pc[j], pm[j], pp[j], ym, yp, xm[j], xp[j], q[j]);
+            }
+            if (t.ragged) {
+                float v[4];
+                unp(q[j], v);
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (t.dead >> i & 1u) v[i] = 0.0f;
+                q[j][0] = f2_make(v[0], v[1]);
+                q[j][1] = f2_make(v[2], v[3]);
+            }
+            d = f2_fma(pc[j][0], q[j][0], d);
+            d = f2_fma(pc[j][1], q[j][1], d);
+        }
+        s = t.in ? __fadd_rn(f2_lo(d), f2_hi(d)) : 0.0f;
+    } else {
+#pragma unroll
+        for (int j = 0; j < CG_R; ++j) {
+            const int y = t.gy + j, jk = KVAR ? j : 0;
+            const CgEdge edge = cg_edge(c, t.gx, y);
+            float pcv[4], pmv[4], ppv[4], ymv[4], ypv[4], kcv[4], kmv[4], kpv[4], kymv[4], kypv[4], qv[4];
+            unp(pc[j], pcv);
+            unp(pm[j], pmv);
+            unp(pp[j], ppv);
+            unp(j == 0 ? h[0] : pr[j > 0 ? j - 1 : 0], ymv);
+            unp(j == CG_R - 1 ? h[1] : pr[j < CG_R - 1 ? j + 1 : 0], ypv);
+            if (KVAR) {
+                ld4(kz + (long long)j * c.sy, kmv);   // the plane below is not kept
+                unp(kc[jk], kcv);
+                unp(kp[jk], kpv);
+                unp(j == 0 ? kh[0] : kr[KVAR && j > 0 ? j - 1 : 0], kymv);
+                unp(j == CG_R - 1 ? kh[1] : kr[KVAR && j < CG_R - 1 ? j + 1 : 0], kypv);
+            }
+            const float sj = cg_q4<KVAR, true>(c, edge, t.gx, y, z, pcv, pmv, ppv, ymv, ypv, xm[j], xp[j], kcv, kmv, kpv, kymv,
+                                               kypv, kxm[j], kxp[j], qv);
+            if (t.in && y < ny) s = __fadd_rn(s, sj);
+            q[j][0] = f2_make(qv[0], qv[1]);
+            q[j][1] = f2_make(qv[2], qv[3]);
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < (KVAR ? CG_R : 1); ++j)
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+            if (KVAR) zf[j][i] = gp[j][i];
+    return s;
+}
+
+// Where a thread's cells lie: byte offset from the start of the padded arrays
+// (the same in all of them; O32: every array is under 4 GiB, so an address is
+// one 32-bit add from the array's base).
+template <bool O32>
+struct CgAddr {
+    using OT = typename std::conditional<O32, unsigned, unsigned long long>::type;
+    long long org;         // elements before the domain origin
+    OT o, dy, dz;          // first cell at the current plane, row and plane strides
+    __device__ __forceinline__ CgAddr(const CgCoef& c, const CgPlace& t, int z)
+        : org(HALO * c.sz + HALO * c.sy + HALO), o((OT)((org + t.row + (long long)z * c.sz) * 4)), dy((OT)(c.sy * 4)),
+          dz((OT)(c.sz * 4)) {}
+    template <typename T>
+    __device__ __forceinline__ char* base(T* p) const { return reinterpret_cast<char*>(const_cast<float*>(p) - org); }
+};
+template <typename OT>
+__device__ __forceinline__ const float* cg_f(const char* b, OT o) { return reinterpret_cast<const float*>(b + o); }
+
+// Store a row's cells at byte offset o; twins: the array keeps its periodic twins.
+template <typename OT>
+__device__ __forceinline__ void cg_put(char* b, OT o, const CgCoef& c, const CgPlace& t, int j, const f2 (&v)[2]) {
+    if (!t.in || (j > 0 && t.gy + j >= c.n[1])) return;
+    float w[4];
+    unp(v, w);
+    st4_row(reinterpret_cast<float*>(b + o), t.gx, c.n[0], w);
+}
+__device__ __forceinline__ void cg_put_twins(float* dom, int z, const CgCoef& c, const CgPlace& t, int j, const f2 (&v)[2]) {
+    if (!t.in || t.gy + j >= c.n[1]) return;
+    float w[4];
+    unp(v, w);
+    st4_twins(dom, c, t.gx, t.gy + j, z, w);
+}
+
+// ----------------------------------------------------------------- cg_dir --
+// One iteration's direction: p = r + beta p_old, p.(A p), and the update of x
+// that the previous iteration left pending, x += alpha_old p_old (p_old is
+// read here anyway). STOREQ: q = A p is stored for cg_res_k (per-cell k); with
+// uniform k cg_res_u forms it again from p, which costs less than its 8 bytes.
+// Bound by HBM with uniform k and close to it with per-cell k: what decides is
+// loads in flight, so every load of a plane is issued before its first use (a
+// branch around p_old's loads alone: 618 us instead of 471 on 512^3), a thread
+// has CG_R rows whose y neighbours and faces are its own registers, x
+// neighbours come by shuffle, and an address is one add (O32; 64-bit address
+// arithmetic: +30 us with per-cell k). Warps on an x face run the same body
+// with ghost values (cg_rows). 16 lanes along x: 32 and 8 are 1 - 3% slower on
+// 512^3 and 390 x 322 x 257; chunks of 32 planes 2%, of 64 planes 10% slower.
+// 512^3, uniform k: 444 us (2.8 GB, 6.3 TB/s) + cg_res_u 254 us (1.68 GB, 6.6
+// TB/s), where q stored and x updated with r took 371 + 481 us; 390 x 322 x
+// 257, per-cell k: 197 us (1.03 GB, 5.2 TB/s) + cg_res_k 66 us for 183 + 123.
+template <bool KVAR, bool STOREQ, bool O32>
+__global__ void __launch_bounds__(32 * CG_W, 16 / CG_W) cg_dir(const __grid_constant__ CgArgs a) {
+    __shared__ double red[CG_W];
     __shared__ bool last;
     const CgCoef& c = a.c;
     if (a.s->done) return;
-    const int par = a.s->iter & 1;   // iteration i reads p[i mod 2], writes p[(i + 1) mod 2]
-    PNew P;
-    P.r = a.r;
-    P.po = par ? a.p1 : a.p0;
-    P.beta = (float)a.s->beta;
-    P.first = a.s->iter == 0;
+    const int iter = a.s->iter;
+    const double rr = a.s->rr;
+    const bool first = iter == 0;
+    const int par = iter & 1;   // iteration i reads p[i mod 2], writes p[(i + 1) mod 2]
+    const float* __restrict__ rv = a.r;
+    const float* __restrict__ po = first ? a.r : par ? a.p1 : a.p0;
+    const float bs = first ? 0.0f : (float)a.s->beta;
+    const f2 beta = f2_make(bs, bs);
+    const float alpha = (float)a.s->alpha;
+    const f2 al = f2_make(alpha, alpha);
     float* __restrict__ pn = par ? a.p0 : a.p1;
-    float* __restrict__ qv = a.q;
     const float* __restrict__ rk = a.rk;
-    const int nx = c.n[0], ny = c.n[1], nz = c.n[2];
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    const int gx = blockIdx.x * 64 + 4 * tx, gy = blockIdx.y * CG_TY + ty;
-    const int z0 = blockIdx.z * a.zchunk, z1 = min(z0 + a.zchunk, nz);
-    const bool perx = c.periodic[0], pery = c.periodic[1], perz = c.periodic[2];
+    const int z0 = blockIdx.z * a.zchunk, z1 = min(z0 + a.zchunk, c.n[2]);
+    const CgPlace t(a);
+    const bool twins = c.periodic[0] || c.periodic[1] || c.periodic[2];
     KahanF dot;
-    if (gx < nx && gy < ny) {
-        const long long sy = c.sy, sz = c.sz;
-        const long long row = cg_at(c, gx, gy, 0);
-        const bool inner_y = pery || (gy > 0 && gy < ny - 1);
-        const bool inner_xy = gx + 3 < nx && (perx || (gx > 0 && gx + 4 < nx)) && inner_y;
-        const CgEdge edge = cg_edge(c, gx, gy);
-        float pm[4], pc[4], km[4], kc[4];
-        pnew4(P, row + (long long)(z0 - 1) * sz, pm);
-        pnew4(P, row + (long long)z0 * sz, pc);
-        if (KVAR) {
-            ld4(rk + row + (long long)(z0 - 1) * sz, km);
-            ld4(rk + row + (long long)z0 * sz, kc);
+    if (t.rows) {
+        using OT = typename CgAddr<O32>::OT;
+        const CgAddr<O32> A(c, t, z0);
+        const OT dy = A.dy, dz = A.dz;
+        OT o = A.o;
+        const char *const rB = A.base(rv), *const oB = A.base(po), *const kB = KVAR ? A.base(rk) : nullptr;
+        char *const xB = A.base(a.x), *const pB = A.base(pn), *const qB = STOREQ ? A.base(a.q) : nullptr;
+        f2 pm[CG_R][2], pc[CG_R][2], pp[CG_R][2], zf[KVAR ? CG_R : 1][2], kc[KVAR ? CG_R : 1][2], kp[KVAR ? CG_R : 1][2];
+        // x += alpha_old p_old of a thread's row
+        auto xadd = [&](int j, OT oj, const float4& x, const float4& old) {
+            const f2 v[2] = {f2_fma(al, lo2(old), lo2(x)), f2_fma(al, hi2(old), hi2(x))};
+            cg_put(xB, oj, c, t, j, v);
+        };
+#pragma unroll
+        for (int j = 0; j < CG_R; ++j) {
+            const OT oj = o + j * dy;
+            const float4 r0 = ldv(cg_f(rB, oj - dz)), o0 = ldv(cg_f(oB, oj - dz)), r1 = ldv(cg_f(rB, oj)), o1 = ldv(cg_f(oB, oj));
+            pnew_pairs(r0, o0, beta, pm[j]);
+            pnew_pairs(r1, o1, beta, pc[j]);
+            if (!first) xadd(j, oj, *reinterpret_cast<const float4*>(xB + oj), o1);
+            if constexpr (KVAR) {
+                f2 km[2];
+                ldp(cg_f(kB, oj - dz), km);
+                ldp(cg_f(kB, oj), kc[j]);
+#pragma unroll
+                for (int i = 0; i < 2; ++i) zf[j][i] = pair_face(km[i], kc[j][i], f2_make(c.tcd[2], c.tcd[2]));
+            }
         }
-        for (int z = z0; z < z1; ++z) {
-            const long long o = row + (long long)z * sz;
-            if ((tx & 7) == 0) {   // one thread per 128-byte line asks L2 for plane z + 3
-                prefetch_l2(P.r + o + 3 * sz);
-                if (!P.first) prefetch_l2(P.po + o + 3 * sz);
-            }
-            float pp[4], ym[4], yp[4];
-            pnew4(P, o + sz, pp);
-            pnew4(P, o - sy, ym);
-            pnew4(P, o + sy, yp);
-            const float xm = pnew1(P, o - 1), xp = pnew1(P, o + 4);
-            float kp[4], kym[4], kyp[4], kxm = 0.0f, kxp = 0.0f;
-            if (KVAR) {
-                ld4(rk + o + sz, kp);
-                ld4(rk + o - sy, kym);
-                ld4(rk + o + sy, kyp);
-                kxm = __ldg(rk + o - 1);
-                kxp = __ldg(rk + o + 4);
-            }
-            float q[4];
-            const bool inner_z = perz || (z > 0 && z < nz - 1);
-            const bool fast = inner_xy && inner_z;
-            const unsigned am = __activemask();
-            const float psum =
-                __all_sync(am, fast)
-                    ? cg_q4<KVAR, false>(c, edge, gx, gy, z, pc, pm, pp, ym, yp, xm, xp, kc, km, kp, kym, kyp, kxm, kxp,
-                                         q)
-                : __all_sync(am, inner_y && inner_z)   // near an x face only
-                    ? cg_q4<KVAR, true, 3>(c, edge, gx, gy, z, pc, pm, pp, ym, yp, xm, xp, kc, km, kp, kym, kyp, kxm,
-                                           kxp, q)
-                    : cg_q4<KVAR, true>(c, edge, gx, gy, z, pc, pm, pp, ym, yp, xm, xp, kc, km, kp, kym, kyp, kxm, kxp,
-                                        q);
-            dot.add(psum);
-            st4_twins(pn, c, gx, gy, z, pc);
-            if (a.q_twins) {
-                st4_twins(qv, c, gx, gy, z, q);
-            } else if (gx + 3 < nx) {
-                *reinterpret_cast<float4*>(qv + o) = make_float4(q[0], q[1], q[2], q[3]);
-            } else {
+        for (int z = z0; z < z1; ++z, o += dz) {
+            float4 rn[CG_R], on[CG_R], xn[CG_R], rh[2], oh[2];
+            float e[CG_R], eo[CG_R], ke[CG_R];
+            f2 h[2][2], kh[2][2];
+            const bool xup = !first && z + 1 < z1;
 #pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    if (gx + i < nx) qv[o + i] = q[i];
+            for (int j = 0; j < CG_R; ++j) {
+                const OT oj = o + dz + j * dy;
+                rn[j] = ldv(cg_f(rB, oj));
+                on[j] = ldv(cg_f(oB, oj));
+                xn[j] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                if (xup) xn[j] = *reinterpret_cast<const float4*>(xB + oj);
+                if constexpr (KVAR) ldp(cg_f(kB, oj), kp[j]);
             }
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                pm[i] = pc[i];
-                pc[i] = pp[i];
-                if (KVAR) {
-                    km[i] = kc[i];
-                    kc[i] = kp[i];
+            for (int j = 0; j < 2; ++j) {
+                const OT oj = j == 0 ? o - dy : o + CG_R * dy;
+                rh[j] = ldv(cg_f(rB, oj));
+                oh[j] = ldv(cg_f(oB, oj));
+                if constexpr (KVAR) ldp(cg_f(kB, oj), kh[j]);
+            }
+#pragma unroll
+            for (int j = 0; j < CG_R; ++j) {
+                e[j] = eo[j] = ke[j] = 0.0f;
+                if (t.ends) {
+                    const OT oj = o + j * dy + (OT)(t.eo * 4);
+                    e[j] = __ldg(cg_f(rB, oj));
+                    eo[j] = __ldg(cg_f(oB, oj));
+                    if constexpr (KVAR) ke[j] = __ldg(cg_f(kB, oj));
+                }
+            }
+            if ((threadIdx.x & 7) == 0) {   // one thread per 128-byte line asks L2 for plane z + 3
+#pragma unroll
+                for (int j = 0; j < CG_R; ++j) {
+                    const OT oj = o + 3 * dz + j * dy;
+                    prefetch_l2(cg_f(rB, oj));
+                    if (!first) {
+                        prefetch_l2(cg_f(oB, oj));
+                        prefetch_l2(xB + oj);
+                    }
+                    if constexpr (KVAR) prefetch_l2(cg_f(kB, oj));
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < CG_R; ++j) {
+                pnew_pairs(rn[j], on[j], beta, pp[j]);
+                e[j] = __fmaf_rn(bs, eo[j], e[j]);
+                if (xup) xadd(j, o + dz + j * dy, xn[j], on[j]);
+            }
+            pnew_pairs(rh[0], oh[0], beta, h[0]);
+            pnew_pairs(rh[1], oh[1], beta, h[1]);
+            f2 q[CG_R][2];
+            dot.add(cg_rows<KVAR>(c, t, z, pc, pm, pp, h, e, kc, zf, kp, kh, ke, KVAR ? cg_f(kB, o - dz) : nullptr, q));
+#pragma unroll
+            for (int j = 0; j < CG_R; ++j) {
+                if (twins) {
+                    cg_put_twins(pn, z, c, t, j, pc[j]);
+                    if (STOREQ && a.q_twins) cg_put_twins(a.q, z, c, t, j, q[j]);
+                } else {
+                    cg_put(pB, o + j * dy, c, t, j, pc[j]);
+                }
+                if (STOREQ && !(twins && a.q_twins)) cg_put(qB, o + j * dy, c, t, j, q[j]);
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    pm[j][i] = pc[j][i];
+                    pc[j][i] = pp[j][i];
+                    if constexpr (KVAR) kc[j][i] = kp[j][i];
                 }
             }
         }
     }
     const double bsum = block_sum(dot.value(), red);
     const int blk = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
+    if (a.dblk) {
+        if (threadIdx.x == 0) a.part[blk] = bsum;
+        return;
+    }
     if (!publish(a, a.part + blk, bsum, &last)) return;
     const double pq = sum_partials(a.part, a.nblk, red);
-    if (threadIdx.x == 0 && threadIdx.y == 0) {
+    if (threadIdx.x == 0) {
         CgState* s = a.s;
-        if (pq > 0.0 && pq < INFINITY) {
-            s->alpha = s->rr / pq;
-        } else {
-            s->alpha = 0.0;
-            s->done = 1;   // p = 0 (exact solution) or a breakdown
-        }
-        s->ticket = 0;
-    }
-}
-
-// cg_spmv_sm: the same step with the x / y neighbours of p from shared
-// memory. Each thread forms p for its own 4 cells of plane z + 1 (two 128-bit
-// loads), edge threads also for the one-cell ring of the 64 x 16 tile, and
-// writes them into a two-plane shared ring; after one barrier a plane, q at
-// plane z reads its x / y neighbours there (the z neighbours stay in the
-// register queue). Two global loads a thread and plane instead of ten.
-constexpr int SM_W = 72;   // shared row: x = -4 .. 67 of the tile, x = 0 at index 4
-
-template <bool KVAR>
-__global__ void __launch_bounds__(CG_TX * CG_TY, CgOcc<KVAR>::blocks) cg_spmv_sm(const __grid_constant__ CgArgs a) {
-    __shared__ double red[CG_TX * CG_TY / 32];
-    __shared__ bool last;
-    __shared__ __align__(16) float sp[2][CG_TY + 2][SM_W];
-    const CgCoef& c = a.c;
-    if (a.s->done) return;
-    const int par = a.s->iter & 1;
-    PNew P;
-    P.r = a.r;
-    P.po = par ? a.p1 : a.p0;
-    P.beta = (float)a.s->beta;
-    P.first = a.s->iter == 0;
-    float* __restrict__ pn = par ? a.p0 : a.p1;
-    float* __restrict__ qv = a.q;
-    const float* __restrict__ rk = a.rk;
-    const int nx = c.n[0], ny = c.n[1], nz = c.n[2];
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    const int x0 = blockIdx.x * 64, y0 = blockIdx.y * CG_TY;
-    const int gx = x0 + 4 * tx, gy = y0 + ty;
-    const int z0 = blockIdx.z * a.zchunk, z1 = min(z0 + a.zchunk, nz);
-    const bool perx = c.periodic[0], pery = c.periodic[1], perz = c.periodic[2];
-    const long long sy = c.sy, sz = c.sz;
-    // every load below stays within the one-cell ring of the domain
-    // ([-1, n] on each axis), inside the padded arrays' halo
-    const bool own = gx < nx && gy < ny;
-    // threads on the one-cell ring of the domain load too: on a periodic
-    // axis their cells are the twins the domain's edge cells read
-    const bool ld = gx <= nx && gy <= ny;
-    const int ry = ty == 0 ? y0 - 1 : y0 + CG_TY;                       // y-ring row of this thread (ty 0 / 15)
-    const bool yr = (ty == 0 || ty == CG_TY - 1) && gx < nx && ry <= ny;
-    const int rx = tx == 0 ? x0 - 1 : x0 + 64;                          // x-ring cell of this row (tx 0 / 15)
-    const bool xr = gy < ny && (tx == 0 || (tx == CG_TX - 1 && x0 + 63 < nx));
-    const int srow = ty + 1, scol = 4 + 4 * tx;
-    const int yrow = ty == 0 ? 0 : CG_TY + 1, xcol = tx == 0 ? 3 : 4 + 64;
-    const long long own_o = cg_at(c, gx, gy, 0), yr_o = cg_at(c, gx, ry, 0), xr_o = cg_at(c, rx, gy, 0);
-    const bool inner_xy = own && gx + 3 < nx && (perx || (gx > 0 && gx + 4 < nx)) && (pery || (gy > 0 && gy < ny - 1));
-    const CgEdge edge = cg_edge(c, gx, gy);
-
-    // shared planes start at 0: cells no thread writes (outside the ring of
-    // the domain) stay finite
-    for (int i = threadIdx.x + CG_TX * threadIdx.y; i < 2 * (CG_TY + 2) * SM_W; i += CG_TX * CG_TY)
-        (&sp[0][0][0])[i] = 0.0f;
-    __syncthreads();
-
-    float pm[4], pc[4], km[4], kc[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) pm[i] = pc[i] = km[i] = kc[i] = 0.0f;
-    if (ld) {
-        pnew4(P, own_o + (long long)(z0 - 1) * sz, pm);
-        pnew4(P, own_o + (long long)z0 * sz, pc);
-    }
-    if (own) {
-        if (KVAR) {
-            ld4(rk + own_o + (long long)(z0 - 1) * sz, km);
-            ld4(rk + own_o + (long long)z0 * sz, kc);
-        }
-    }
-    {   // plane z0 into shared slot z0 & 1
-        float* sl = &sp[z0 & 1][0][0];
-        sts4(sl + srow * SM_W + scol, pc);
-        if (yr) {
-            float v[4];
-            pnew4(P, yr_o + (long long)z0 * sz, v);
-            sts4(sl + yrow * SM_W + scol, v);
-        }
-        if (xr) sl[srow * SM_W + xcol] = pnew1(P, xr_o + (long long)z0 * sz);
-    }
-    __syncthreads();
-
-    KahanF dot;
-    for (int z = z0; z < z1; ++z) {
-        const int cs = z & 1;
-        const long long o = own_o + (long long)z * sz;
-        float pp[4];
-        if (ld) {
-            if ((tx & 7) == 0) {   // one thread per 128-byte line asks L2 for plane z + 3
-                prefetch_l2(P.r + o + 3 * sz);
-                if (!P.first) prefetch_l2(P.po + o + 3 * sz);
-            }
-            pnew4(P, o + sz, pp);
-        } else {
-#pragma unroll
-            for (int i = 0; i < 4; ++i) pp[i] = 0.0f;
-        }
-        {   // plane z + 1 into the other slot (free since the last barrier)
-            float* sl = &sp[cs ^ 1][0][0];
-            sts4(sl + srow * SM_W + scol, pp);
-            if (yr) {
-                float v[4];
-                pnew4(P, yr_o + (long long)(z + 1) * sz, v);
-                sts4(sl + yrow * SM_W + scol, v);
-            }
-            if (xr) sl[srow * SM_W + xcol] = pnew1(P, xr_o + (long long)(z + 1) * sz);
-        }
-        float kp[4], kym[4], kyp[4], kxm = 0.0f, kxp = 0.0f;
-        if (KVAR) {
-#pragma unroll
-            for (int i = 0; i < 4; ++i) kp[i] = kym[i] = kyp[i] = 1.0f;
-            if (own) {
-                ld4(rk + o + sz, kp);
-                ld4(rk + o - sy, kym);
-                ld4(rk + o + sy, kyp);
-                kxm = __ldg(rk + o - 1);
-                kxp = __ldg(rk + o + 4);
-            }
-        }
-        const float* sl = &sp[cs][0][0];
-        float ym[4], yp[4];
-        lds4(sl + (srow - 1) * SM_W + scol, ym);
-        lds4(sl + (srow + 1) * SM_W + scol, yp);
-        const float xm = sl[srow * SM_W + scol - 1], xp = sl[srow * SM_W + scol + 4];
-        float q[4];
-        // threads without own cells do not hold the warp back from the
-        // interior formula (as in cg_spmv, where they do not take part)
-        const bool fast = !own || (inner_xy && (perz || (z > 0 && z < nz - 1)));
-        const float psum = __all_sync(__activemask(), fast)
-                               ? cg_q4<KVAR, false>(c, edge, gx, gy, z, pc, pm, pp, ym, yp, xm, xp, kc, km, kp, kym, kyp,
-                                                    kxm, kxp, q)
-                               : cg_q4<KVAR, true>(c, edge, gx, gy, z, pc, pm, pp, ym, yp, xm, xp, kc, km, kp, kym, kyp,
-                                                   kxm, kxp, q);
-        if (own) {
-            dot.add(psum);
-            st4_twins(pn, c, gx, gy, z, pc);
-            if (gx + 3 < nx) {
-                *reinterpret_cast<float4*>(qv + o) = make_float4(q[0], q[1], q[2], q[3]);
-            } else {
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    if (gx + i < nx) qv[o + i] = q[i];
-            }
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            pm[i] = pc[i];
-            pc[i] = pp[i];
-            if (KVAR) {
-                km[i] = kc[i];
-                kc[i] = kp[i];
-            }
-        }
-        __syncthreads();
-    }
-    const double bsum = block_sum(dot.value(), red);
-    const int blk = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
-    if (!publish(a, a.part + blk, bsum, &last)) return;
-    const double pq = sum_partials(a.part, a.nblk, red);
-    if (threadIdx.x == 0 && threadIdx.y == 0) {
-        CgState* s = a.s;
-        if (pq > 0.0 && pq < INFINITY) {
-            s->alpha = s->rr / pq;
-        } else {
-            s->alpha = 0.0;
-            s->done = 1;
-        }
+        const bool ok = pq > 0.0 && pq < INFINITY;   // else p = 0 (exact solution) or a breakdown
+        s->alpha = ok ? rr / pq : 0.0;
+        if (!ok) s->done = 1;
+        s->pending = !ok && !first ? 2 : 0;
         s->ticket = 0;
     }
 }
@@ -963,17 +1080,48 @@ __global__ void __launch_bounds__(CG_TX * CG_TY, PipeOcc<KVAR>::blocks) cg_pipe(
     }
 }
 
-// -------------------------------------------------------------- cg_update --
-// x += alpha p, r -= alpha q over the domain cells (4 along x per item),
-// r.r partials; then beta and the convergence test.
-__global__ void __launch_bounds__(CG_THREADS) cg_update(const __grid_constant__ CgArgs a) {
+// ----------------------------------------------------------------- cg_res --
+// The new residual and its r.r (cg_ctl_iter sums the partials); x takes its
+// alpha p later (the next cg_dir, or cg_xfin after the last iteration).
+
+// alpha = r.r / p.q as cg_dir's last block left it, or, on a small grid, from
+// the blocks' partials in every block of cg_res: a load and a short sum at its
+// start for the ticket and the tail at cg_dir's end (3 us of an iteration's 19
+// on 64^3). False: p = 0 or a breakdown, which ends the solve.
+__device__ __forceinline__ bool cg_alpha(const CgArgs& a, double* red, float (&sh)[2], float* alpha) {
+    if (!a.dblk) {
+        *alpha = (float)a.s->alpha;
+        return true;
+    }
+    const double rr = a.s->rr;
+    const int iter = a.s->iter;
+    const double pq = sum_partials(a.part, a.dblk, red);
+    if (threadIdx.x == 0) {
+        const bool ok = pq > 0.0 && pq < INFINITY;
+        const double al = ok ? rr / pq : 0.0;
+        sh[0] = (float)al;
+        sh[1] = ok ? 1.0f : 0.0f;
+        if (blockIdx.x + blockIdx.y + blockIdx.z == 0) {   // the others neither read these nor, without ok, go on
+            a.s->alpha = al;
+            if (!ok) {
+                a.s->pending = iter > 0 ? 2 : 0;
+                a.s->done = 1;
+            }
+        }
+    }
+    __syncthreads();
+    *alpha = sh[0];
+    return sh[1] != 0.0f;
+}
+
+// r -= alpha q over the domain cells (4 along x per item), q stored by cg_dir.
+__global__ void __launch_bounds__(CG_THREADS) cg_res_k(const __grid_constant__ CgArgs a) {
     __shared__ double red[CG_THREADS / 32];
-    __shared__ bool last;
+    __shared__ float sh[2];
     const CgCoef& c = a.c;
     if (a.s->done) return;
-    const int par = a.s->iter & 1;
-    const float alpha = (float)a.s->alpha;
-    const float* __restrict__ p = par ? a.p0 : a.p1;
+    float alpha;
+    if (!cg_alpha(a, red, sh, &alpha)) return;
     const int nx = c.n[0], ny = c.n[1], nz = c.n[2];
     const int xg = (nx + 3) / 4;
     const long long items = (long long)xg * ny * nz;
@@ -989,20 +1137,16 @@ __global__ void __launch_bounds__(CG_THREADS) cg_update(const __grid_constant__ 
     for (long long it = it0; it < items; it += stride) {
         const int gx = 4 * ixg;
         const long long o = cg_at(c, gx, y, z);
-        float xv[4], pv[4], qv[4], rv[4];
-        ld4(a.x + o, xv);
-        ld4(p + o, pv);
+        float qv[4], rv[4];
         ld4(a.q + o, qv);
         ld4(a.r + o, rv);
         float s = 0.0f;
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            xv[i] = __fmaf_rn(alpha, pv[i], xv[i]);
             rv[i] = __fmaf_rn(-alpha, qv[i], rv[i]);
             if (gx + i < nx) s = __fmaf_rn(rv[i], rv[i], s);
         }
         rr.add(s);
-        st4_twins(a.x, c, gx, y, z, xv);   // the field's twins feed the next step's cg_init
         st4_twins(a.r, c, gx, y, z, rv);
         ixg += dxg;
         y += dy;
@@ -1017,16 +1161,93 @@ __global__ void __launch_bounds__(CG_THREADS) cg_update(const __grid_constant__ 
         }
     }
     const double bsum = block_sum(rr.value(), red);
-    if (!publish(a, a.part + blockIdx.x, bsum, &last)) return;
-    const double R = sum_partials(a.part, a.nblk, red);
-    if (threadIdx.x == 0) {
-        CgState* s = a.s;
-        s->beta = s->rr > 0.0 ? R / s->rr : 0.0;
-        s->rr = R;
-        s->iter += 1;
-        if (R <= s->tol2 * s->bb || s->iter >= s->max_iter || !(R == R)) s->done = 1;
-        s->ticket = 0;
+    if (threadIdx.x == 0) a.part[CG_MAX_PART + blockIdx.x] = bsum;
+}
+
+// r -= alpha A p with A p formed from p again (uniform k), on cg_dir's layout.
+template <bool O32>
+__global__ void __launch_bounds__(32 * CG_W, 24 / CG_W) cg_res_u(const __grid_constant__ CgArgs a) {
+    __shared__ double red[CG_W];
+    __shared__ float sh[2];
+    const CgCoef& c = a.c;
+    if (a.s->done) return;
+    float alpha;
+    if (!cg_alpha(a, red, sh, &alpha)) return;
+    const f2 nal = f2_make(-alpha, -alpha);
+    const float* __restrict__ p = (a.s->iter & 1) ? a.p0 : a.p1;
+    const int z0 = blockIdx.z * a.zchunk, z1 = min(z0 + a.zchunk, c.n[2]);
+    const CgPlace t(a);
+    const bool twins = c.periodic[0] || c.periodic[1] || c.periodic[2];
+    KahanF rr;
+    if (t.rows) {
+        using OT = typename CgAddr<O32>::OT;
+        const CgAddr<O32> A(c, t, z0);
+        const OT dy = A.dy, dz = A.dz;
+        OT o = A.o;
+        const char* const pB = A.base(p);
+        char* const rB = A.base(a.r);
+        f2 pm[CG_R][2], pc[CG_R][2], pp[CG_R][2];
+        f2 kd[1][2] = {{0, 0}}, zf[1][2] = {{0, 0}};
+        const f2 kh[2][2] = {{0, 0}, {0, 0}};
+        const float ke[CG_R] = {};
+        const bool row1 = t.in && t.gy + 1 < c.n[1];
+#pragma unroll
+        for (int j = 0; j < CG_R; ++j) {
+            ldp(cg_f(pB, o + j * dy - dz), pm[j]);
+            ldp(cg_f(pB, o + j * dy), pc[j]);
+        }
+        for (int z = z0; z < z1; ++z, o += dz) {
+            f2 h[2][2], r[CG_R][2], q[CG_R][2];
+            float e[CG_R];
+#pragma unroll
+            for (int j = 0; j < CG_R; ++j) {
+                ldp(cg_f(pB, o + dz + j * dy), pp[j]);
+                const float4 v = *reinterpret_cast<const float4*>(rB + (o + j * dy));
+                r[j][0] = lo2(v);
+                r[j][1] = hi2(v);
+            }
+            ldp(cg_f(pB, o - dy), h[0]);
+            ldp(cg_f(pB, o + CG_R * dy), h[1]);
+#pragma unroll
+            for (int j = 0; j < CG_R; ++j) {
+                e[j] = 0.0f;
+                if (t.ends) e[j] = __ldg(cg_f(pB, o + j * dy + (OT)(t.eo * 4)));
+            }
+            if ((threadIdx.x & 7) == 0) {
+#pragma unroll
+                for (int j = 0; j < CG_R; ++j) {
+                    prefetch_l2(cg_f(pB, o + 3 * dz + j * dy));
+                    prefetch_l2(rB + (o + 2 * dz + j * dy));
+                }
+            }
+            cg_rows<false>(c, t, z, pc, pm, pp, h, e, kd, zf, kd, kh, ke, nullptr, q);
+            float s = 0.0f;
+#pragma unroll
+            for (int j = 0; j < CG_R; ++j) {
+                r[j][0] = f2_fma(nal, q[j][0], r[j][0]);
+                r[j][1] = f2_fma(nal, q[j][1], r[j][1]);
+                if (j == 0 ? t.in : row1) {
+                    float v[4];
+                    unp(r[j], v);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const float u = i == 0 || t.gx + i < c.n[0] ? v[i] : 0.0f;
+                        s = __fmaf_rn(u, u, s);
+                    }
+                }
+                if (twins) cg_put_twins(a.r, z, c, t, j, r[j]);
+                else cg_put(rB, o + j * dy, c, t, j, r[j]);
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    pm[j][i] = pc[j][i];
+                    pc[j][i] = pp[j][i];
+                }
+            }
+            rr.add(s);
+        }
     }
+    const double bsum = block_sum(rr.value(), red);
+    if (threadIdx.x == 0) a.part[CG_MAX_PART + blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z)] = bsum;
 }
 
 // ---------------------------------------------------------- device loops --
@@ -1046,14 +1267,63 @@ struct CgLoop {
 };
 static_assert(sizeof(CgLoop) <= 64, "CgLoop is read back into a 64-byte pinned word");
 
-__global__ void cg_ctl_start(CgState* s, CgLoop* L, cudaGraphConditionalHandle inner) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        L->inner_count = 0;
-        cudaGraphSetConditional(inner, s->done ? 0u : 1u);
+// The scalar work after cg_init: r.r and b.b from the blocks' partials, the
+// solver's state for a new step. L is null in the host-checked runs.
+__global__ void __launch_bounds__(CG_CTL) cg_ctl_start(const __grid_constant__ CgArgs a, CgLoop* L,
+                                                       cudaGraphConditionalHandle inner, double tol2, int max_iter) {
+    __shared__ double red[CG_CTL / 32];
+    const double R = sum_partials(a.part, a.nblk, red);
+    const double B = sum_partials(a.part + CG_MAX_PART, a.nblk, red);
+    if (threadIdx.x == 0) {
+        CgState* s = a.s;
+        s->rr = R;
+        s->bb = B;
+        s->alpha = 0.0;
+        s->beta = 0.0;
+        s->tol2 = tol2;
+        s->iter = 0;
+        s->max_iter = max_iter;
+        s->pending = 0;
+        const int done = (R <= tol2 * B || max_iter <= 0 || !(R == R)) ? 1 : 0;
+        s->done = done;
+        s->ticket = 0;
+        if (L) {
+            L->inner_count = 0;
+            cudaGraphSetConditional(inner, done ? 0u : 1u);
+        }
     }
 }
 
-__global__ void cg_ctl_iter(CgState* s, CgLoop* L, cudaGraphConditionalHandle inner, int max_iter) {
+// The scalar work after cg_res: r.r from the blocks' partials, beta and the
+// convergence test. It is a kernel of its own in the device loop anyway (the
+// loop's condition), so cg_res ends without a ticket and a last block's tail.
+__global__ void __launch_bounds__(CG_CTL) cg_ctl_iter(const __grid_constant__ CgArgs a, CgLoop* L,
+                                                      cudaGraphConditionalHandle inner, int max_iter) {
+    __shared__ double red[CG_CTL / 32];
+    CgState* s = a.s;
+    int done = s->done, iter = s->iter;
+    const double rr = s->rr, lim = s->tol2 * s->bb;
+    const int mi = s->max_iter;
+    const unsigned k = L ? L->inner_count + 1 : 0;
+    const double R = sum_partials(a.part + CG_MAX_PART, a.nblk, red);
+    if (threadIdx.x != 0) return;
+    if (!done) {
+        iter += 1;
+        done = (R <= lim || iter >= mi || !(R == R)) ? 1 : 0;
+        s->iter = iter;
+        s->rr = R;
+        s->beta = rr > 0.0 ? R / rr : 0.0;
+        s->pending = 1;
+        s->done = done;
+    }
+    if (L) {
+        L->inner_count = k;
+        cudaGraphSetConditional(inner, (!done && k < (unsigned)max_iter + 2u) ? 1u : 0u);
+    }
+}
+
+// The pipelined method's (cg_pipe has done the scalar work).
+__global__ void cg_ctl_pipe(CgState* s, CgLoop* L, cudaGraphConditionalHandle inner, int max_iter) {
     if (threadIdx.x == 0 && blockIdx.x == 0) {
         const unsigned k = ++L->inner_count;
         cudaGraphSetConditional(inner, (!s->done && k < (unsigned)max_iter + 2u) ? 1u : 0u);
@@ -1062,6 +1332,60 @@ __global__ void cg_ctl_iter(CgState* s, CgLoop* L, cudaGraphConditionalHandle in
 
 __global__ void cg_ctl_step(CgState* s, CgLoop* L, cudaGraphConditionalHandle outer) {
     if (threadIdx.x == 0 && blockIdx.x == 0) {
+        L->total_iters += s->iter;
+        L->last_rr = s->rr;
+        L->last_bb = s->bb;
+        L->steps_left -= 1;
+        L->steps_done += 1;
+        cudaGraphSetConditional(outer, (L->steps_left > 0 && L->steps_done < L->steps_limit) ? 1u : 0u);
+    }
+}
+
+// ---------------------------------------------------------------- cg_xfin --
+// The end of a classic step: the pending x += alpha p, with x's periodic twins
+// (they feed the next step's cg_init; cg_dir's updates leave them stale), and
+// the step's bookkeeping (L: device loops).
+__global__ void __launch_bounds__(CG_THREADS) cg_xfin(const __grid_constant__ CgArgs a, CgLoop* L, cudaGraphConditionalHandle outer) {
+    const CgCoef& c = a.c;
+    const int pending = a.s->pending;
+    if (pending) {
+        const float alpha = (float)a.s->alpha;
+        const float* __restrict__ p = (a.s->iter & 1) ? a.p1 : a.p0;   // written by iteration iter - 1
+        const int nx = c.n[0], ny = c.n[1], nz = c.n[2];
+        const int xg = (nx + 3) / 4;
+        const long long items = (long long)xg * ny * nz;
+        const long long it0 = blockIdx.x * (long long)CG_THREADS + threadIdx.x;
+        const long long stride = (long long)gridDim.x * CG_THREADS;
+        const int dxg = (int)(stride % xg);
+        const long long drow = stride / xg;
+        const int dy = (int)(drow % ny), dz = (int)(drow / ny);
+        int ixg = (int)(it0 % xg), y = (int)((it0 / xg) % ny), z = (int)(it0 / xg / ny);
+        for (long long it = it0; it < items; it += stride) {
+            const int gx = 4 * ixg;
+            const long long o = cg_at(c, gx, y, z);
+            const float4 x = *reinterpret_cast<const float4*>(a.x + o);
+            float xv[4] = {x.x, x.y, x.z, x.w}, pv[4];
+            if (pending == 1) {
+                ld4(p + o, pv);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) xv[i] = __fmaf_rn(alpha, pv[i], xv[i]);
+            }
+            st4_twins(a.x, c, gx, y, z, xv);
+            ixg += dxg;
+            y += dy;
+            z += dz;
+            if (ixg >= xg) {
+                ixg -= xg;
+                ++y;
+            }
+            if (y >= ny) {
+                y -= ny;
+                ++z;
+            }
+        }
+    }
+    if (L && blockIdx.x == 0 && threadIdx.x == 0) {
+        const CgState* s = a.s;
         L->total_iters += s->iter;
         L->last_rr = s->rr;
         L->last_bb = s->bb;
@@ -1092,7 +1416,9 @@ struct CgWork {
     CgArgs key;        // arguments the graph was captured with
     int kvar = -1;
     int method = -1;   // WFA_CG_CLASSIC / WFA_CG_PIPELINED of the captured graphs
-    int spmv_grid[3] = {0, 0, 0};
+    int spmv_grid[3] = {0, 0, 0};   // cg_init, cg_pipe
+    int dir_grid[3] = {0, 0, 0};    // cg_dir, cg_res_u
+    int dir_threads = 0, dir_chunk = 0, dir_lanes = 0;
     int upd_blocks = 0;
     long long prev_iters = 0;   // iterations the last step needed (sizes the first run of the next)
     bool o32 = false;           // every array under 4 GiB: cg_init takes 32-bit byte offsets
@@ -1177,6 +1503,60 @@ static void cg_coef(const wfa_grid_s* g, double dt, CgCoef* c) {
     c->sz = g->px * g->py;
 }
 
+// A kernel of the solver with its grid and arguments, launched on a stream or
+// added to a graph.
+struct CgKernel {
+    const void* fn;
+    dim3 grid, block;
+    CgArgs a;
+    cudaError_t run(cudaStream_t st, void** args = nullptr) const {
+        void* own[] = {const_cast<CgArgs*>(&a)};
+        return cudaLaunchKernel(fn, grid, block, args ? args : own, 0, st);
+    }
+};
+struct CgLaunch {
+    CgKernel init, start, dir, res, iter, pipe;
+    CgLaunch(const CgWork* w, const CgArgs& base, bool kvar, int method) {
+        const bool storeq = kvar || method == WFA_CG_PIPELINED;
+        if (w->o32)
+            dir.fn = kvar ? (const void*)cg_dir<true, true, true>
+                          : storeq ? (const void*)cg_dir<false, true, true> : (const void*)cg_dir<false, false, true>;
+        else
+            dir.fn = kvar ? (const void*)cg_dir<true, true, false>
+                          : storeq ? (const void*)cg_dir<false, true, false> : (const void*)cg_dir<false, false, false>;
+        dir.grid = dim3(w->dir_grid[0], w->dir_grid[1], w->dir_grid[2]);
+        dir.block = dim3(w->dir_threads);
+        dir.a = base;
+        dir.a.lanes = w->dir_lanes;
+        dir.a.zchunk = w->dir_chunk;
+        dir.a.nblk = w->dir_grid[0] * w->dir_grid[1] * w->dir_grid[2];
+        if (method != WFA_CG_PIPELINED && dir.a.nblk <= CG_FOLD) dir.a.dblk = dir.a.nblk;
+        res = dir;
+        res.fn = w->o32 ? (const void*)cg_res_u<true> : (const void*)cg_res_u<false>;
+        if (kvar) {
+            res.fn = (const void*)cg_res_k;
+            res.grid = dim3(w->upd_blocks);
+            res.block = dim3(CG_THREADS);
+            res.a.nblk = w->upd_blocks;
+        }
+        iter.fn = (const void*)cg_ctl_iter;
+        iter.grid = dim3(1);
+        iter.block = dim3(CG_CTL);
+        iter.a = res.a;
+        pipe.fn = kvar ? (const void*)cg_pipe<true> : (const void*)cg_pipe<false>;
+        pipe.grid = dim3(w->spmv_grid[0], w->spmv_grid[1], w->spmv_grid[2]);
+        pipe.block = dim3(CG_TX, CG_TY);
+        pipe.a = base;
+        pipe.a.nblk = w->spmv_grid[0] * w->spmv_grid[1] * w->spmv_grid[2];
+        init = pipe;
+        init.fn = kvar ? (w->o32 ? (const void*)cg_init<true, true> : (const void*)cg_init<true, false>)
+                       : (w->o32 ? (const void*)cg_init<false, true> : (const void*)cg_init<false, false>);
+        start = iter;
+        start.fn = (const void*)cg_ctl_start;
+        start.a = init.a;
+    }
+};
+
 static int cg_capture(wfa_grid_s* g, CgWork* w, const CgArgs& base, bool kvar, int method) {
     if (w->exec[0] && w->kvar == (int)kvar && w->method == method && memcmp(&w->key, &base, sizeof base) == 0)
         return WFA_OK;
@@ -1185,40 +1565,25 @@ static int cg_capture(wfa_grid_s* g, CgWork* w, const CgArgs& base, bool kvar, i
             cudaGraphExecDestroy(e);
             e = nullptr;
         }
-    CgArgs sp = base, up = base;
-    sp.nblk = w->spmv_grid[0] * w->spmv_grid[1] * w->spmv_grid[2];
-    up.nblk = w->upd_blocks;
-    const dim3 sgrid(w->spmv_grid[0], w->spmv_grid[1], w->spmv_grid[2]), sblock(CG_TX, CG_TY);
+    const CgLaunch kl(w, base, kvar, method);
     if (!w->cap) WFA_CUDA(cudaStreamCreateWithFlags(&w->cap, cudaStreamNonBlocking));
     const cudaStream_t st = w->cap;
-    // q = A p from L1-cached neighbour loads (cg_spmv) or through a shared
-    // plane (cg_spmv_sm); WFA_CG_SPMV=l1|sm overrides the default
-    const char* pick = getenv("WFA_CG_SPMV");
-    const bool use_sm = pick ? strcmp(pick, "sm") == 0 : CG_SPMV_SM_DEFAULT;
     for (int k = 0; k < CG_NRUN; ++k) {
         WFA_CUDA(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
         cudaError_t e = cudaSuccess;
         for (int it = 0; it < CG_RUN_LEN[k] && e == cudaSuccess; ++it) {
             if (method == WFA_CG_PIPELINED) {   // one kernel, one reduction an iteration
-                if (kvar)
-                    cg_pipe<true><<<sgrid, sblock, 0, st>>>(sp);
-                else
-                    cg_pipe<false><<<sgrid, sblock, 0, st>>>(sp);
-                e = cudaGetLastError();
+                e = kl.pipe.run(st);
                 continue;
             }
-            if (kvar && use_sm)
-                cg_spmv_sm<true><<<sgrid, sblock, 0, st>>>(sp);
-            else if (kvar)
-                cg_spmv<true><<<sgrid, sblock, 0, st>>>(sp);
-            else if (use_sm)
-                cg_spmv_sm<false><<<sgrid, sblock, 0, st>>>(sp);
-            else
-                cg_spmv<false><<<sgrid, sblock, 0, st>>>(sp);
-            e = cudaGetLastError();
+            e = kl.dir.run(st);
+            if (e == cudaSuccess) e = kl.res.run(st);
             if (e == cudaSuccess) {
-                cg_update<<<w->upd_blocks, CG_THREADS, 0, st>>>(up);
-                e = cudaGetLastError();
+                CgLoop* none = nullptr;
+                cudaGraphConditionalHandle h0 = 0;
+                int mi = 0;
+                void* args[] = {const_cast<CgArgs*>(&kl.iter.a), &none, &h0, &mi};
+                e = kl.iter.run(st, args);
             }
         }
         cudaGraph_t gr = nullptr;
@@ -1262,8 +1627,9 @@ static cudaError_t add_while(cudaGraph_t gr, cudaGraphNode_t* node, cudaGraphNod
     return e;
 }
 
-// outer WHILE (steps) { cg_init; [pipelined: cg_spmv]; cg_ctl_start;
-//   inner WHILE (iterations) { classic: cg_spmv, cg_update | pipelined: cg_pipe; cg_ctl_iter }; cg_ctl_step }
+// outer WHILE (steps) { cg_init; cg_ctl_start; [pipelined: cg_dir];
+//   inner WHILE (iterations) { classic: cg_dir, cg_res, cg_ctl_iter | pipelined: cg_pipe, cg_ctl_pipe };
+//   classic: cg_xfin | pipelined: cg_ctl_step }
 static cudaError_t build_loop_graph(CgWork* w, const CgArgs& base, bool kvar, int method, double tol2,
                                     int max_iter, cudaGraphExec_t* out) {
     cudaGraph_t top = nullptr;
@@ -1272,51 +1638,51 @@ static cudaError_t build_loop_graph(CgWork* w, const CgArgs& base, bool kvar, in
     cudaGraphConditionalHandle ho = 0, hi = 0;
     cudaGraph_t outer = nullptr, inner = nullptr;
     cudaGraphNode_t n_outer = nullptr, n = nullptr, prev = nullptr;
-    CgArgs ia = base, sp = base, up = base;
-    ia.nblk = sp.nblk = w->spmv_grid[0] * w->spmv_grid[1] * w->spmv_grid[2];
+    const CgLaunch kl(w, base, kvar, method);
+    CgArgs up = base;
     up.nblk = w->upd_blocks;
-    const dim3 sgrid(w->spmv_grid[0], w->spmv_grid[1], w->spmv_grid[2]), sblock(CG_TX, CG_TY);
     CgState* st = w->s;
     CgLoop* L = w->loop;
-    void* a_init[] = {&ia, &tol2, &max_iter};
-    void* a_sp[] = {&sp};
-    void* a_up[] = {&up};
-    void* a_start[] = {&st, &L, &hi};
-    void* a_iter[] = {&st, &L, &hi, &max_iter};
+    auto arg = [](const CgKernel& k) { return const_cast<CgArgs*>(&k.a); };
+    void* a_init[] = {arg(kl.init)};
+    void* a_dir[] = {arg(kl.dir)};
+    void* a_res[] = {arg(kl.res)};
+    void* a_pipe[] = {arg(kl.pipe)};
+    void* a_start[] = {arg(kl.start), &L, &hi, &tol2, &max_iter};
+    void* a_iter[] = {arg(kl.iter), &L, &hi, &max_iter};
+    void* a_pctl[] = {&st, &L, &hi, &max_iter};
     void* a_step[] = {&st, &L, &ho};
+    void* a_fin[] = {&up, &L, &ho};
     e = cudaGraphConditionalHandleCreate(&ho, top, 1, cudaGraphCondAssignDefault);
     if (e == cudaSuccess) e = add_while(top, &n_outer, nullptr, ho, &outer);
-    if (e == cudaSuccess)
-        e = add_kernel(outer, &n, nullptr,
-                       kvar ? (w->o32 ? (const void*)cg_init<true, true> : (const void*)cg_init<true, false>)
-                            : (w->o32 ? (const void*)cg_init<false, true> : (const void*)cg_init<false, false>),
-                       sgrid,
-                       sblock, a_init);
+    if (e == cudaSuccess) e = add_kernel(outer, &n, nullptr, kl.init.fn, kl.init.grid, kl.init.block, a_init);
+    prev = n;
+    if (e == cudaSuccess) e = cudaGraphConditionalHandleCreate(&hi, outer, 0, 0);
+    if (e == cudaSuccess) e = add_kernel(outer, &n, prev, kl.start.fn, kl.start.grid, kl.start.block, a_start);
     prev = n;
     if (e == cudaSuccess && method == WFA_CG_PIPELINED) {
-        e = add_kernel(outer, &n, prev, kvar ? (const void*)cg_spmv<true> : (const void*)cg_spmv<false>, sgrid, sblock,
-                       a_sp);
+        e = add_kernel(outer, &n, prev, kl.dir.fn, kl.dir.grid, kl.dir.block, a_dir);
         prev = n;
     }
-    if (e == cudaSuccess) e = cudaGraphConditionalHandleCreate(&hi, outer, 0, 0);
-    if (e == cudaSuccess) e = add_kernel(outer, &n, prev, (const void*)cg_ctl_start, dim3(1), dim3(32), a_start);
-    prev = n;
     cudaGraphNode_t n_inner = nullptr;
     if (e == cudaSuccess) e = add_while(outer, &n_inner, prev, hi, &inner);
     if (e == cudaSuccess) {
         cudaGraphNode_t ip = nullptr;
         if (method == WFA_CG_PIPELINED) {
-            e = add_kernel(inner, &ip, nullptr, kvar ? (const void*)cg_pipe<true> : (const void*)cg_pipe<false>, sgrid,
-                           sblock, a_sp);
+            e = add_kernel(inner, &ip, nullptr, kl.pipe.fn, kl.pipe.grid, kl.pipe.block, a_pipe);
         } else {
-            e = add_kernel(inner, &ip, nullptr, kvar ? (const void*)cg_spmv<true> : (const void*)cg_spmv<false>, sgrid,
-                           sblock, a_sp);
-            if (e == cudaSuccess)
-                e = add_kernel(inner, &ip, ip, (const void*)cg_update, dim3(w->upd_blocks), dim3(CG_THREADS), a_up);
+            e = add_kernel(inner, &ip, nullptr, kl.dir.fn, kl.dir.grid, kl.dir.block, a_dir);
+            if (e == cudaSuccess) e = add_kernel(inner, &ip, ip, kl.res.fn, kl.res.grid, kl.res.block, a_res);
         }
-        if (e == cudaSuccess) e = add_kernel(inner, &ip, ip, (const void*)cg_ctl_iter, dim3(1), dim3(32), a_iter);
+        if (e == cudaSuccess)
+            e = method == WFA_CG_PIPELINED
+                    ? add_kernel(inner, &ip, ip, (const void*)cg_ctl_pipe, dim3(1), dim3(32), a_pctl)
+                    : add_kernel(inner, &ip, ip, kl.iter.fn, kl.iter.grid, kl.iter.block, a_iter);
     }
-    if (e == cudaSuccess) e = add_kernel(outer, &n, n_inner, (const void*)cg_ctl_step, dim3(1), dim3(32), a_step);
+    if (e == cudaSuccess)
+        e = method == WFA_CG_PIPELINED
+                ? add_kernel(outer, &n, n_inner, (const void*)cg_ctl_step, dim3(1), dim3(32), a_step)
+                : add_kernel(outer, &n, n_inner, (const void*)cg_xfin, dim3(w->upd_blocks), dim3(CG_THREADS), a_fin);
     if (e == cudaSuccess) e = cudaGraphInstantiate(out, top, 0);
     cudaGraphDestroy(top);
     return e;
@@ -1389,7 +1755,7 @@ int wfa_implicit_step(wfa_grid g, double dt, long long n, double rtol, int max_i
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     if (nsm <= 0) nsm = 1;
-    {   // cg_spmv / cg_init grid: 64 x 16 columns, z chunks of about 16 planes,
+    {   // cg_init / cg_pipe grid: 64 x 16 columns, z chunks of about 16 planes,
         // many waves of blocks so the last wave's tail is short; chunks down to
         // 2 planes only where 16 would leave SMs idle (small grids)
         const int gxb = (g->n[0] + 63) / 64, gyb = (g->n[1] + CG_TY - 1) / CG_TY;
@@ -1409,8 +1775,29 @@ int wfa_implicit_step(wfa_grid g, double dt, long long n, double rtol, int max_i
         w->spmv_grid[0] = gxb;
         w->spmv_grid[1] = gyb;
         w->spmv_grid[2] = (int)nch;
+        // cg_dir / cg_res_u: CG_W warps of 16 (narrow grids: 8) x lanes, CG_R rows
+        // a thread; chunks of about 16 planes, shorter where that leaves SMs idle
+        const int lanes = g->n[0] > 32 ? 16 : 8, warps = CG_W;
+        const long long bx = (g->n[0] + 4 * lanes - 1) / (4 * lanes);
+        const int rows = CG_R * warps * 32 / lanes, by = (g->n[1] + rows - 1) / rows;
+        const long long dcols = bx * by;
+        const long long dres = (long long)nsm * 16 / CG_W;   // resident blocks
+        long long dch = std::max(1, g->n[2] / 16);
+        if (dcols * dch < dres) dch = std::min<long long>(g->n[2], std::max<long long>(dch, dres / dcols));
+        dch = std::min<long long>(dch, std::max<long long>(1, CG_MAX_PART / dcols));
+        w->dir_chunk = (int)((g->n[2] + dch - 1) / dch);
+        dch = (g->n[2] + w->dir_chunk - 1) / w->dir_chunk;
+        w->dir_grid[0] = (int)bx;
+        w->dir_grid[1] = by;
+        w->dir_grid[2] = (int)dch;
+        w->dir_lanes = lanes;
+        w->dir_threads = 32 * warps;
+        if (dcols * dch > CG_MAX_PART) {
+            set_error("wfa_implicit_step: grid too large for the partial-sum buffer");
+            return WFA_ERR_ARG;
+        }
         const long long items = (long long)((g->n[0] + 3) / 4) * g->n[1] * g->n[2];
-        w->upd_blocks = (int)std::max<long long>(1, std::min<long long>((items + CG_THREADS - 1) / CG_THREADS, nsm * 8LL));
+        w->upd_blocks = (int)std::max<long long>(1, std::min<long long>((items + CG_THREADS - 1) / CG_THREADS, nsm * 4LL));
     }
     const int method = g->cg_method;
     if (method == WFA_CG_PIPELINED) {   // three more work vectors: r, w and s ping-pong
@@ -1428,7 +1815,7 @@ int wfa_implicit_step(wfa_grid g, double dt, long long n, double rtol, int max_i
     rc = cg_capture(g, w, base, kvar, method);
     if (rc) return rc;
 
-    const int per_iter = method == WFA_CG_PIPELINED ? 1 : 2;   // kernels an iteration
+    const int per_iter = method == WFA_CG_PIPELINED ? 1 : 3;   // kernels an iteration (host-checked runs)
 
     // The device-loop graph: every step and iteration without a host round
     // trip (WFA_CG_LOOP=host keeps the host-checked runs below).
@@ -1473,7 +1860,7 @@ int wfa_implicit_step(wfa_grid g, double dt, long long n, double rtol, int max_i
                 return WFA_ERR_STATE;
             }
             const int extra_per_step = method == WFA_CG_PIPELINED ? 4 : 3;   // init, [spmv], start, step
-            g->launches += extra_per_step * n + (long long)(per_iter + 1) * Lr.total_iters;
+            g->launches += extra_per_step * n + (method == WFA_CG_PIPELINED ? 2LL : 3LL) * Lr.total_iters;
             w->prev_iters = n > 0 ? Lr.total_iters / n : 0;
             g->halo_dirty = true;
             g->steps_done += n;
@@ -1483,28 +1870,23 @@ int wfa_implicit_step(wfa_grid g, double dt, long long n, double rtol, int max_i
         }
     }
 
-    CgArgs ia = base;
-    ia.nblk = w->spmv_grid[0] * w->spmv_grid[1] * w->spmv_grid[2];
-    const dim3 sgrid(w->spmv_grid[0], w->spmv_grid[1], w->spmv_grid[2]), sblock(CG_TX, CG_TY);
+    const CgLaunch kl(w, base, kvar, method);
     long long total = 0;
     double last_rel = 0.0;
     for (long long step = 0; step < n; ++step) {
-        if (kvar)
-            if (w->o32) cg_init<true, true><<<sgrid, sblock, 0, g->stream>>>(ia, rtol * rtol, max_iter);
-            else cg_init<true, false><<<sgrid, sblock, 0, g->stream>>>(ia, rtol * rtol, max_iter);
-        else
-            if (w->o32) cg_init<false, true><<<sgrid, sblock, 0, g->stream>>>(ia, rtol * rtol, max_iter);
-            else cg_init<false, false><<<sgrid, sblock, 0, g->stream>>>(ia, rtol * rtol, max_iter);
-        WFA_CUDA(cudaGetLastError());
-        g->launches += 1;
+        {
+            CgLoop* none = nullptr;
+            cudaGraphConditionalHandle h0 = 0;
+            double tol2 = rtol * rtol;
+            void* args[] = {const_cast<CgArgs*>(&kl.start.a), &none, &h0, &tol2, &max_iter};
+            WFA_CUDA(kl.init.run(g->stream));
+            WFA_CUDA(kl.start.run(g->stream, args));
+            g->launches += 2;
+        }
         if (method == WFA_CG_PIPELINED) {
             // w = A r, delta = w.r and alpha = r.r / delta: the first half of a
             // classic iteration (q = A p with p = r), q keeping its twins
-            if (kvar)
-                cg_spmv<true><<<sgrid, sblock, 0, g->stream>>>(ia);
-            else
-                cg_spmv<false><<<sgrid, sblock, 0, g->stream>>>(ia);
-            WFA_CUDA(cudaGetLastError());
+            WFA_CUDA(kl.dir.run(g->stream));
             g->launches += 1;
         }
         // Runs of captured iterations with one run queued ahead of the flag
@@ -1547,6 +1929,13 @@ int wfa_implicit_step(wfa_grid g, double dt, long long n, double rtol, int max_i
             }
         }
         WFA_CUDA(cudaStreamSynchronize(g->stream));   // the run queued ahead has ended (no-op kernels)
+        if (method != WFA_CG_PIPELINED) {
+            CgArgs fa = base;
+            fa.nblk = w->upd_blocks;
+            cg_xfin<<<w->upd_blocks, CG_THREADS, 0, g->stream>>>(fa, nullptr, cudaGraphConditionalHandle());
+            WFA_CUDA(cudaGetLastError());
+            g->launches += 1;
+        }
         total += st.iter;
         w->prev_iters = st.iter;
         last_rel = st.bb > 0.0 ? sqrt(st.rr / st.bb) : sqrt(st.rr);

@@ -96,6 +96,13 @@ __device__ __forceinline__ f2 f2_fma(f2 a, f2 b, f2 c) {
 __device__ __forceinline__ f2 unpack2(unsigned u) {
     return f2_make(__uint_as_float(u << 16), __uint_as_float(u & 0xffff0000u));
 }
+// Coefficients of two faces from the sums of their cells' 1/k.
+__device__ __forceinline__ f2 pair_face(f2 ra, f2 rb, f2 tcd) {
+    float a, b;
+    f2_get(f2_add(ra, rb), a, b);
+    return f2_mul(tcd, f2_make(rcp_approx(a), rcp_approx(b)));
+}
+
 // A row as loaded: fp32 pairs, or bf16 words converted where they are first used.
 template <typename S> struct RowBuf;
 template <> struct RowBuf<float> {

@@ -29,13 +29,6 @@
 
 namespace wfa {
 
-// Coefficients of two faces from the sums of their cells' 1/k.
-__device__ __forceinline__ f2 face2(f2 ra, f2 rb, f2 tcd) {
-    float a, b;
-    f2_get(f2_add(ra, rb), a, b);
-    return f2_mul(tcd, f2_make(rcp_approx(a), rcp_approx(b)));
-}
-
 // Weights of the 4 cells of a row: x faces as left / right pairs.
 struct RowW {
     f2 xm0, xm1, xp0, xp1;
@@ -172,7 +165,7 @@ __device__ __forceinline__ void pair_k_run(const SweepCoef& c, const void* tin, 
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
             D[j][i] = f2_sub(u[i], v[i]);
-            G1[j][i] = face2(ku[i], kv[i], tcz);
+            G1[j][i] = pair_face(ku[i], kv[i], tcz);
             S0[j][i] = S1[j][i] = DS[j][i] = G0[j][i] = 0;
         }
         WX[j].xm0 = WX[j].xm1 = WX[j].xp0 = WX[j].xp1 = 0;
@@ -228,8 +221,8 @@ __device__ __forceinline__ void pair_k_run(const SweepCoef& c, const void* tin, 
             Tc[0].get(t);
             KH[0].get(h);
             Kc[0].get(k);
-            WY[0][0] = face2(h[0], k[0], tcy);
-            WY[0][1] = face2(h[1], k[1], tcy);
+            WY[0][0] = pair_face(h[0], k[0], tcy);
+            WY[0][1] = pair_face(h[1], k[1], tcy);
 #pragma unroll
             for (int j = 0; j < R; ++j) {
                 f2 up[2], tn[2], ku[2], kn[2], acc[2], v[2], ym[2], yp[2], gm[2], gp[2];
@@ -269,8 +262,8 @@ __device__ __forceinline__ void pair_k_run(const SweepCoef& c, const void* tin, 
                 f2 gz[2];
 #pragma unroll
                 for (int i = 0; i < 2; ++i) {
-                    WY[j + 1][i] = face2(k[i], ku[i], tcy);
-                    gz[i] = face2(k[i], kn[i], tcz);
+                    WY[j + 1][i] = pair_face(k[i], ku[i], tcy);
+                    gz[i] = pair_face(k[i], kn[i], tcz);
                 }
                 add_adv<ADV>(ym, WY[j], c.adv[2]);
                 add_adv<ADV>(yp, WY[j + 1], c.adv[3]);
