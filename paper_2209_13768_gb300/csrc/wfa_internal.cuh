@@ -51,6 +51,44 @@ struct NvtxRange {
     NvtxRange& operator=(const NvtxRange&) = delete;
 };
 
+// Launch with programmatic serialization: the kernel's blocks may become
+// resident while the kernel before it in the stream drains, and start with
+// grid_wait(), which returns when that kernel has ended and its writes are
+// visible. For kernels that call it before anything else. Measured: 333x250x187
+// bf16, per-cell k 31.5 -> 30.0 us a step, 512^3 210 -> 208. Not while the
+// stream is captured: the nodes of a graph follow one another faster without
+// (64^3 runs of 32 passes: 2.9 us a pass against 4.1).
+template <typename... P, typename... A>
+cudaError_t launch_overlapped(void (*k)(P...), dim3 grid, dim3 block, cudaStream_t st, A... args) {
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.stream = st;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) {
+        cudaGetLastError();
+        cap = cudaStreamCaptureStatusActive;
+    }
+    cfg.attrs = at;
+    cfg.numAttrs = cap == cudaStreamCaptureStatusNone ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, k, static_cast<P>(args)...);
+}
+
+#ifdef __CUDACC__
+// Lets the next kernel's blocks in, then waits for the kernel before (nothing
+// to wait for unless launched with launch_overlapped). The pointers that the
+// kernel loads through pass through here: a read-only load could otherwise be
+// moved above the wait.
+template <typename T, typename U>
+__device__ __forceinline__ void grid_wait(T*& a, U*& b) {
+    asm volatile("griddepcontrol.launch_dependents;");
+    asm volatile("griddepcontrol.wait;" : "+l"(a), "+l"(b)::"memory");
+}
+#endif
+
 // ---------------------------------------------------------------- errors --
 void set_error(const char* fmt, ...);
 int cuda_fail(cudaError_t e, const char* what);

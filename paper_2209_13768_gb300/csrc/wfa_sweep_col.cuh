@@ -533,6 +533,9 @@ template <typename S, bool KVAR, bool ADV, bool INL, int V = 4, bool TW = true, 
 __global__ void __launch_bounds__(256, (ColOcc<KVAR, INL, sizeof(S), V>::blocks))
     sweep_col(const __grid_constant__ SweepArgs a) {
     const SweepCoef& c = a.c;
+    const void* tin = a.tin;
+    const float* rk = a.rk;
+    grid_wait(tin, rk);
     const int gx = (blockIdx.x * blockDim.x + threadIdx.x) * V;
     const int gy = blockIdx.y * blockDim.y + threadIdx.y;
     if (gx >= c.n[0] || gy >= c.n[1]) return;
@@ -541,10 +544,10 @@ __global__ void __launch_bounds__(256, (ColOcc<KVAR, INL, sizeof(S), V>::blocks)
     constexpr int U = ColOcc<KVAR, INL, sizeof(S), V>::unroll;
     constexpr ColMode MODE = INL ? COL_INPLACE : COL_THIN;
     if (blockIdx.z & 1)   // odd chunks march down: see col_run
-        col_run<S, KVAR, ADV, false, U, MODE, true, false, -1, V, TW, HELD>(c, (const S*)a.tin, (S*)a.tout, a.rk,
+        col_run<S, KVAR, ADV, false, U, MODE, true, false, -1, V, TW, HELD>(c, (const S*)tin, (S*)a.tout, rk,
                                                                            a.status, gx, gy, z0, z1);
     else
-        col_run<S, KVAR, ADV, false, U, MODE, true, false, 1, V, TW, HELD>(c, (const S*)a.tin, (S*)a.tout, a.rk,
+        col_run<S, KVAR, ADV, false, U, MODE, true, false, 1, V, TW, HELD>(c, (const S*)tin, (S*)a.tout, rk,
                                                                           a.status, gx, gy, z0, z1);
 }
 
@@ -559,6 +562,9 @@ __global__ void __launch_bounds__(256, (ColOcc<KVAR, INL, sizeof(S), V>::blocks)
 template <typename S, bool KVAR, bool SKIPHELD = false>
 __global__ void __launch_bounds__(256) boundary_fix(const __grid_constant__ SweepArgs a) {
     const SweepCoef& c = a.c;
+    const void* tin = a.tin;
+    const float* rk = a.rk;
+    grid_wait(tin, rk);
     const int f = blockIdx.y, ax = f >> 1;
     if (c.periodic[ax] || c.ext[f] || (SKIPHELD && c.held[f])) return;   // no boundary cells to fix on this face
     const int b = ax == 0 ? 1 : 0, d = ax == 2 ? 1 : 2;
@@ -569,7 +575,7 @@ __global__ void __launch_bounds__(256) boundary_fix(const __grid_constant__ Swee
         pos[b] = (int)(t % nb);
         pos[d] = (int)(t / nb);
         const long long i = (long long)pos[2] * c.sz + (long long)pos[1] * c.sy + pos[0];
-        const float v = general_cell<S, KVAR>(c, (const S*)a.tin, a.rk, i, pos[0], pos[1], pos[2], a.status);
+        const float v = general_cell<S, KVAR>(c, (const S*)tin, rk, i, pos[0], pos[1], pos[2], a.status);
         if (c.periodic[0] || c.periodic[1] || c.periodic[2])   // with its periodic copies
             store_with_twins<S>((S*)a.tout, c, pos[0], pos[1], pos[2], from_f32<S>(v), a.status);
         else
@@ -668,22 +674,22 @@ cudaError_t col_launch_v(const SweepArgs& a_in, cudaStream_t st, int nsm, const 
     const bool adv = KVAR && (a.c.adv[0] != 0.0f || a.c.adv[1] != 0.0f || a.c.adv[2] != 0.0f ||
                               a.c.adv[3] != 0.0f || a.c.adv[4] != 0.0f || a.c.adv[5] != 0.0f);
     if (ev) cudaEventRecord(ev[0], st);
+    cudaError_t e;
     if (inl) {
-        if (adv) sweep_col<S, KVAR, true, true><<<grid, block, 0, st>>>(a);
-        else sweep_col<S, KVAR, false, true><<<grid, block, 0, st>>>(a);
+        if (adv) e = launch_overlapped(sweep_col<S, KVAR, true, true>, grid, block, st, a);
+        else e = launch_overlapped(sweep_col<S, KVAR, false, true>, grid, block, st, a);
     } else if (a.c.held[0] || a.c.held[1] || a.c.held[2] || a.c.held[3] || a.c.held[4] || a.c.held[5]) {
         // held cell layers: kept in the pass (copies for any periodic axis too)
-        if (adv) sweep_col<S, KVAR, true, false, V, true, true><<<grid, block, 0, st>>>(a);
-        else sweep_col<S, KVAR, false, false, V, true, true><<<grid, block, 0, st>>>(a);
+        if (adv) e = launch_overlapped(sweep_col<S, KVAR, true, false, V, true, true>, grid, block, st, a);
+        else e = launch_overlapped(sweep_col<S, KVAR, false, false, V, true, true>, grid, block, st, a);
     } else if (a.c.periodic[0] || a.c.periodic[1] || a.c.periodic[2]) {
-        if (adv) sweep_col<S, KVAR, true, false, V, true><<<grid, block, 0, st>>>(a);
-        else sweep_col<S, KVAR, false, false, V, true><<<grid, block, 0, st>>>(a);
+        if (adv) e = launch_overlapped(sweep_col<S, KVAR, true, false, V, true>, grid, block, st, a);
+        else e = launch_overlapped(sweep_col<S, KVAR, false, false, V, true>, grid, block, st, a);
     } else {   // no periodic axis: no copies to store
-        if (adv) sweep_col<S, KVAR, true, false, V, false><<<grid, block, 0, st>>>(a);
-        else sweep_col<S, KVAR, false, false, V, false><<<grid, block, 0, st>>>(a);
+        if (adv) e = launch_overlapped(sweep_col<S, KVAR, true, false, V, false>, grid, block, st, a);
+        else e = launch_overlapped(sweep_col<S, KVAR, false, false, V, false>, grid, block, st, a);
     }
     if (ev) cudaEventRecord(ev[1], st);
-    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || inl || a.c.halo_bc) return e;
     long long plane = 0;   // the largest face with boundary cells to fix (held faces are done)
     for (int ax = 0; ax < 3; ++ax) {
@@ -693,8 +699,7 @@ cudaError_t col_launch_v(const SweepArgs& a_in, cudaStream_t st, int nsm, const 
     }
     if (plane == 0) return cudaSuccess;
     const int nb = (int)std::min<long long>((plane + 255) / 256, (long long)nsm * 2);
-    boundary_fix<S, KVAR, true><<<dim3(nb, 6), 256, 0, st>>>(a);
-    return cudaGetLastError();
+    return launch_overlapped(boundary_fix<S, KVAR, true>, dim3(nb, 6), dim3(256), st, a);
 }
 
 template <typename S, bool KVAR>

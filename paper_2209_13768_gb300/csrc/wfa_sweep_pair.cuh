@@ -222,6 +222,9 @@ template <typename S, bool PER, bool RAG, int R, int WPB, int BLOCKS>
 __global__ void __launch_bounds__(32 * WPB, BLOCKS) sweep_pair(const __grid_constant__ SweepArgs a) {
     constexpr int E = sizeof(S);
     const SweepCoef& c = a.c;
+    const void* tin = a.tin;
+    const float* rk = a.rk;
+    grid_wait(tin, rk);
     const int nx = c.n[0], ny = c.n[1], nz = c.n[2];
     const int lane = threadIdx.x;
     const int gx = blockIdx.x * PAIR_TX - 4 + 4 * lane;
@@ -234,7 +237,7 @@ __global__ void __launch_bounds__(32 * WPB, BLOCKS) sweep_pair(const __grid_cons
     // a periodic x face one period away, or (where a period is no whole number
     // of groups) from the halo's copies, which the RAG passes store
     const int lx = !RAG && perx ? (gx < 0 ? gx + nx : gx < nx ? gx : min(gx - nx, nx)) : min(gx, (nx + 3) & ~3);
-    const char* const tX = reinterpret_cast<const char*>((const S*)a.tin);   // cell (0, 0, 0)
+    const char* const tX = reinterpret_cast<const char*>((const S*)tin);   // cell (0, 0, 0)
     const char* tP = tX + (long long)lx * E + y0 * sy + (z0 - 1) * sz;       // this lane's group, row y0, plane q
     char* oP = reinterpret_cast<char*>((S*)a.tout) + (long long)gx * E + y0 * sy + (z0 - 2) * sz;
     // x faces: the weights of cells 0 and n_x - 1, and the face values that
@@ -421,13 +424,14 @@ cudaError_t pair_launch(const SweepArgs& a_in, cudaStream_t st, int nsm, const c
     nch = (a.c.n[2] + a.zchunk - 1) / a.zchunk;
     const dim3 grid(gxb, gyb, nch), block(32, Cfg::WPB);
     if (ev) cudaEventRecord(ev[0], st);
+    cudaError_t e;
     const bool per = a.c.periodic[0] || a.c.periodic[1] || a.c.periodic[2], rag = a.c.n[0] % 4 != 0;
-    if (per && rag) sweep_pair<S, true, true, Cfg::R, Cfg::WPB, Cfg::BLOCKS><<<grid, block, 0, st>>>(a);
-    else if (per) sweep_pair<S, true, false, Cfg::R, Cfg::WPB, Cfg::BLOCKS><<<grid, block, 0, st>>>(a);
-    else if (rag) sweep_pair<S, false, true, Cfg::R, Cfg::WPB, Cfg::BLOCKS><<<grid, block, 0, st>>>(a);
-    else sweep_pair<S, false, false, Cfg::R, Cfg::WPB, Cfg::BLOCKS><<<grid, block, 0, st>>>(a);
+    if (per && rag) e = launch_overlapped(sweep_pair<S, true, true, Cfg::R, Cfg::WPB, Cfg::BLOCKS>, grid, block, st, a);
+    else if (per) e = launch_overlapped(sweep_pair<S, true, false, Cfg::R, Cfg::WPB, Cfg::BLOCKS>, grid, block, st, a);
+    else if (rag) e = launch_overlapped(sweep_pair<S, false, true, Cfg::R, Cfg::WPB, Cfg::BLOCKS>, grid, block, st, a);
+    else e = launch_overlapped(sweep_pair<S, false, false, Cfg::R, Cfg::WPB, Cfg::BLOCKS>, grid, block, st, a);
     if (ev) cudaEventRecord(ev[1], st);
-    return cudaGetLastError();
+    return e;
 }
 
 }  // namespace wfa

@@ -360,19 +360,22 @@ template <typename S, bool PER, bool RAG, bool ADV>
 __global__ void __launch_bounds__(32 * PairKCfg::W, PairKCfg::BLOCKS)
     sweep_pair_k(const __grid_constant__ SweepArgs a, const __grid_constant__ PairTiles tl) {
     __shared__ __align__(16) float sm[2 * (PairKCfg::R * PairKCfg::W + 2) * 128];
+    const void* tin = a.tin;
+    const float* rk = a.rk;
+    grid_wait(tin, rk);
     const int z0 = blockIdx.z * a.zchunk;
-    pair_k_run<S, PER, RAG, ADV, PairKCfg::R, PairKCfg::W>(a.c, a.tin, a.tout, a.rk, tl, blockIdx.x, blockIdx.y, z0,
+    pair_k_run<S, PER, RAG, ADV, PairKCfg::R, PairKCfg::W>(a.c, tin, a.tout, rk, tl, blockIdx.x, blockIdx.y, z0,
                                                            min(z0 + a.zchunk, a.c.n[2]), sm);
 }
 
 template <typename S, bool ADV>
-void pair_k_dispatch(const SweepArgs& a, const PairTiles& tl, dim3 grid, cudaStream_t st) {
+cudaError_t pair_k_dispatch(const SweepArgs& a, const PairTiles& tl, dim3 grid, cudaStream_t st) {
     const dim3 block(32 * PairKCfg::W);
     const bool per = a.c.periodic[0] || a.c.periodic[1] || a.c.periodic[2], rag = a.c.n[0] % 4 != 0;
-    if (per && rag) sweep_pair_k<S, true, true, ADV><<<grid, block, 0, st>>>(a, tl);
-    else if (per) sweep_pair_k<S, true, false, ADV><<<grid, block, 0, st>>>(a, tl);
-    else if (rag) sweep_pair_k<S, false, true, ADV><<<grid, block, 0, st>>>(a, tl);
-    else sweep_pair_k<S, false, false, ADV><<<grid, block, 0, st>>>(a, tl);
+    if (per && rag) return launch_overlapped(sweep_pair_k<S, true, true, ADV>, grid, block, st, a, tl);
+    if (per) return launch_overlapped(sweep_pair_k<S, true, false, ADV>, grid, block, st, a, tl);
+    if (rag) return launch_overlapped(sweep_pair_k<S, false, true, ADV>, grid, block, st, a, tl);
+    return launch_overlapped(sweep_pair_k<S, false, false, ADV>, grid, block, st, a, tl);
 }
 
 // z chunks of a launch of `tiles` blocks a chunk: whole waves of resident
@@ -402,10 +405,9 @@ cudaError_t pair_k_launch(const SweepArgs& a_in, cudaStream_t st, int nsm, const
     const bool adv = a.c.adv[0] != 0.0f || a.c.adv[1] != 0.0f || a.c.adv[2] != 0.0f || a.c.adv[3] != 0.0f ||
                      a.c.adv[4] != 0.0f || a.c.adv[5] != 0.0f;
     if (ev) cudaEventRecord(ev[0], st);
-    if (adv) pair_k_dispatch<S, true>(a, tl, grid, st);
-    else pair_k_dispatch<S, false>(a, tl, grid, st);
+    const cudaError_t e = adv ? pair_k_dispatch<S, true>(a, tl, grid, st) : pair_k_dispatch<S, false>(a, tl, grid, st);
     if (ev) cudaEventRecord(ev[1], st);
-    return cudaGetLastError();
+    return e;
 }
 
 }  // namespace wfa
