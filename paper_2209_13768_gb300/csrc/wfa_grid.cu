@@ -418,7 +418,7 @@ int refresh_halo(wfa_grid_s* g, int buf) {
 }
 
 // --------------------------------------------------------------- reductions --
-constexpr int RED_BLOCKS = 304;
+constexpr int HEAT_BLOCKS = 152 * 8;   // resident blocks: a warp a row
 // the stability passes are latency-bound (divisions, seven k reads a cell):
 // more warps per SM; their partials fit the 4096-double scratch below the
 // word kept for the k check (index 4095)
@@ -429,22 +429,74 @@ static_assert(RATE_P2 > RATE_BLOCKS + 1 && RATE_P2 + RATE_BLOCKS <= RATE_RISKY &
               "scratch layout");
 constexpr int RED_THREADS = 256;
 
+// a + b = s + e exactly (round to nearest, no overflow).
+__device__ __forceinline__ float two_sum(float a, float b, float* e) {
+    const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
+    *e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
+    return s;
+}
+
+// Sum of the field in fp64. Bound by HBM with a warp per row and 4 cells a
+// lane, once the GPU's fp64 rate (a conversion and an addition a cell) is out
+// of the loop: a thread adds in fp32 with the exact rounding error of every
+// addition, and sums the errors with compensation, which rounds less than fp64
+// additions do. Sums that leave the fp32 range (or inf, NaN) go to fp64.
+// 512^3: 1.39 ms with a 64-bit division and an fp64 addition a cell, 0.36 with
+// one fp64 addition for 4 cells, 0.17 now (3.1 TB/s).
 template <typename S>
 __global__ void __launch_bounds__(RED_THREADS) heat_partial_kernel(const S* __restrict__ origin, const __grid_constant__ Geo geo,
                                                                    double* __restrict__ partials) {
     __shared__ double sh[RED_THREADS];
-    const long long N = (long long)geo.n[0] * geo.n[1] * geo.n[2];
-    const long long sz = geo.px * geo.py;
+    const int nx = geo.n[0], ny = geo.n[1], lane = threadIdx.x & 31;
+    const long long sz = geo.px * geo.py, rows = (long long)ny * geo.n[2];
+    const long long warps = (long long)gridDim.x * (RED_THREADS / 32);
     double acc = 0.0;
-    for (long long i = blockIdx.x * (long long)RED_THREADS + threadIdx.x; i < N;
-         i += (long long)RED_BLOCKS * RED_THREADS) {
-        const int x = (int)(i % geo.n[0]);
-        const long long r = i / geo.n[0];
-        const int y = (int)(r % geo.n[1]);
-        const int z = (int)(r / geo.n[1]);
-        acc += (double)to_f32<S>(origin[z * sz + y * geo.px + x]);
+    float fs = 0.0f, es = 0.0f, ec = 0.0f;   // the fp32 sum; the errors' sum and its compensation
+    auto add4 = [&](const float (&v)[4]) {
+        float e0, e1, e2, e3;
+        const float s0 = two_sum(v[0], v[1], &e0), s1 = two_sum(v[2], v[3], &e1), t = two_sum(s0, s1, &e2),
+                    f = two_sum(fs, t, &e3);
+        const float e = __fadd_rn(__fadd_rn(e0, e1), __fadd_rn(e2, e3));
+        if (fabsf(f) < INFINITY && fabsf(e) < INFINITY) {   // no partial sum left the range
+            fs = f;
+            const float y = __fsub_rn(e, ec), u = __fadd_rn(es, y);
+            ec = __fsub_rn(__fsub_rn(u, es), y);
+            es = u;
+        } else {
+            acc += ((((double)v[0] + (double)v[1]) + (double)v[2]) + (double)v[3]) + (double)fs;
+            fs = 0.0f;
+        }
+    };
+    for (long long row = blockIdx.x * (long long)(RED_THREADS / 32) + (threadIdx.x >> 5); row < rows; row += warps) {
+        const int z = (int)((unsigned long long)row / (unsigned)ny), y = (int)(row - (long long)z * ny);
+        const S* o = origin + z * sz + y * geo.px;
+        for (int x0 = 4 * lane; x0 < nx; x0 += 512) {   // four groups' loads in flight
+            float v[4][4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int x = x0 + 128 * u;
+                v[u][0] = v[u][1] = v[u][2] = v[u][3] = 0.0f;
+                if (x >= nx) continue;
+                if constexpr (sizeof(S) == 4) {
+                    const float4 q = __ldg(reinterpret_cast<const float4*>(o + x));
+                    v[u][0] = q.x; v[u][1] = q.y; v[u][2] = q.z; v[u][3] = q.w;
+                } else {
+                    const uint2 q = __ldg(reinterpret_cast<const uint2*>(o + x));
+                    v[u][0] = __uint_as_float(q.x << 16); v[u][1] = __uint_as_float(q.x & 0xffff0000u);
+                    v[u][2] = __uint_as_float(q.y << 16); v[u][3] = __uint_as_float(q.y & 0xffff0000u);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int x = x0 + 128 * u;
+#pragma unroll
+                for (int i = 1; i < 4; ++i)
+                    if (x + i >= nx) v[u][i] = 0.0f;
+                add4(v[u]);
+            }
+        }
     }
-    sh[threadIdx.x] = acc;
+    sh[threadIdx.x] = (acc + (double)fs) + ((double)es - (double)ec);
     __syncthreads();
     for (int s = RED_THREADS / 2; s > 0; s >>= 1) {
         if (threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s];
@@ -453,7 +505,7 @@ __global__ void __launch_bounds__(RED_THREADS) heat_partial_kernel(const S* __re
     if (threadIdx.x == 0) partials[blockIdx.x] = sh[0];
 }
 
-// Fixed-order finish: one block, a tree over RED_BLOCKS partials.
+// Fixed-order finish: one block, a tree over the blocks' partials.
 __global__ void __launch_bounds__(512) finish_sum_kernel(const double* __restrict__ partials, int n,
                                                          double scale, double* __restrict__ out) {
     __shared__ double sh[512];
@@ -683,14 +735,123 @@ __global__ void __launch_bounds__(RED_THREADS) rate32_partial_kernel(const float
                                                                      double* __restrict__ risky_out) {
     float best = 0.0f;
     int any_risky = 0;
-    for_each_cell(r, [&](const int c[3], long long idx) {
-        const bool inner = rate_inner(r, c);
+    const int nx = r.n[0], ny = r.n[1], lane = threadIdx.x & 31;
+    const bool wx0 = r.kind[0] == WFA_BC_PERIODIC || r.kind[0] == WFA_BC_EXCHANGE,
+               wx1 = r.kind[1] == WFA_BC_PERIODIC || r.kind[1] == WFA_BC_EXCHANGE;
+    const long long sz = r.px * r.py, rows = (long long)ny * r.n[2];
+    const long long warps = (long long)gridDim.x * (RED_THREADS / 32);
+    // on a face: what stands for kD / (kC + kD) (1 makes the term Dirichlet's
+    // 2 kC / h^2; nothing goes through a zero-flux face, nor advection)
+    const float dx0 = r.kind[0] == WFA_BC_DIRICHLET ? 1.0f : 0.0f, dx1 = r.kind[1] == WFA_BC_DIRICHLET ? 1.0f : 0.0f;
+    auto cell = [&](const int (&c)[3], long long idx, bool inner) {
         if (!inner && rate_held(r, c)) return;
         bool risky;
         const float d = rate32(korigin, r, c, idx, &risky, inner);
         if (!risky) best = fmaxf(best, d);
         else any_risky = 1;
-    });
+    };
+    // Rows as for_each_cell deals them (rate_cand_kernel counts on that), 4 cells
+    // a lane: rate32's sum with fewer operations, within the
+    // same 24 units of 2^-24 (a reciprocal within 1 ulp, three products, 9 additions).
+    // 512^3: one cell a lane with rate32 1.25 ms, this 0.43 (issue 74%: 38 fp
+    // operations and 6 reciprocals a cell); rows on a face in the same body, for
+    // a warp's rows share their y: with face rows cell by cell 1.06.
+    for (long long row = blockIdx.x * (long long)(RED_THREADS / 32) + (threadIdx.x >> 5); row < rows; row += warps) {
+        int c[3] = {0, (int)(row % ny), (int)(row / ny)};
+        const long long base = (long long)c[2] * sz + (long long)c[1] * r.px;
+        bool lo_f[3], hi_f[3], in_yz = true;   // the row lies on a y or z face; away from all of them
+        float d_lo[3], d_hi[3], uyz = 0.0f;
+#pragma unroll
+        for (int a = 1; a < 3; ++a) {
+            lo_f[a] = c[a] == 0 && r.kind[2 * a] != WFA_BC_PERIODIC && r.kind[2 * a] != WFA_BC_EXCHANGE;
+            hi_f[a] = c[a] == r.n[a] - 1 && r.kind[2 * a + 1] != WFA_BC_PERIODIC && r.kind[2 * a + 1] != WFA_BC_EXCHANGE;
+            d_lo[a] = r.kind[2 * a] == WFA_BC_DIRICHLET ? 1.0f : 0.0f;
+            d_hi[a] = r.kind[2 * a + 1] == WFA_BC_DIRICHLET ? 1.0f : 0.0f;
+            uyz += (lo_f[a] && d_lo[a] == 0.0f ? 0.0f : r.umf[a]) + (hi_f[a] && d_hi[a] == 0.0f ? 0.0f : r.upf[a]);
+            in_yz = in_yz && !lo_f[a] && !hi_f[a];
+        }
+        if ((lo_f[1] && r.held[2]) || (hi_f[1] && r.held[3]) || (lo_f[2] && r.held[4]) || (hi_f[2] && r.held[5])) continue;
+        const float usum = (r.upf[0] + r.umf[0]) + uyz, ux0 = r.upf[0] + (dx0 != 0.0f ? r.umf[0] : 0.0f) + uyz,
+                    ux1 = r.umf[0] + (dx1 != 0.0f ? r.upf[0] : 0.0f) + uyz;
+        for (int x0 = 0; x0 < nx; x0 += 128) {   // whole warps: shuffles
+            const int x = x0 + 4 * lane;
+            const float* k = korigin + base + min(x, (nx + 3) & ~3);
+            const bool first = !wx0 && x == 0;         // cell 0 on the -x face, cell `last` on the +x face
+            const int last = wx1 ? 4 : nx - 1 - x;
+            auto ld = [](const float* p, float (&v)[4]) {
+                const float4 q = __ldg(reinterpret_cast<const float4*>(p));
+                v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
+            };
+            float kc[4], y0[4], y1[4], z0[4], z1[4];
+            ld(k, kc);
+            ld(k - r.px, y0);
+            ld(k + r.px, y1);
+            ld(k - sz, z0);
+            ld(k + sz, z1);
+            float kl = __shfl_up_sync(0xffffffffu, kc[3], 1), kr = __shfl_down_sync(0xffffffffu, kc[0], 1);
+            if (lane == 0) kl = __ldg(k - 1);
+            if (lane == 31) kr = __ldg(k + 4);
+            if (x >= nx) continue;
+#pragma unroll
+            for (int i = 1; i < 4; ++i)
+                if (x + i >= nx) {   // the halo's: not looked at, but for the neighbour across a periodic face
+                    y0[i] = y1[i] = z0[i] = z1[i] = kc[0];
+                    if (!wx1 || x + i > nx) kc[i] = kc[0];
+                }
+            if (first) kl = kc[0];
+            if (last == 3) kr = kc[3];
+            if (!in_yz) {   // beyond a face: not looked at either
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    y0[i] = lo_f[1] ? kc[i] : y0[i];
+                    y1[i] = hi_f[1] ? kc[i] : y1[i];
+                    z0[i] = lo_f[2] ? kc[i] : z0[i];
+                    z1[i] = hi_f[2] ? kc[i] : z1[i];
+                }
+            }
+            // any value outside [1e-15, 1e15] (0 included): cell by cell
+            unsigned lo = min(__float_as_uint(kl), __float_as_uint(kr)), hi = max(__float_as_uint(kl), __float_as_uint(kr));
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (float v : {kc[i], y0[i], y1[i], z0[i], z1[i]}) {
+                    lo = min(lo, __float_as_uint(v));
+                    hi = max(hi, __float_as_uint(v));
+                }
+            if (lo < __float_as_uint(1e-15f) || hi > __float_as_uint(1e15f)) {
+#pragma unroll 1
+                for (int i = 0; i < 4; ++i) {
+                    c[0] = x + i;
+                    if (x + i < nx) cell(c, base + x + i, in_yz && (wx0 || x + i > 0) && (wx1 || x + i < nx - 1));
+                }
+                continue;
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float kd[6] = {i == 0 ? kl : kc[i > 0 ? i - 1 : 0], i == 3 ? kr : kc[i < 3 ? i + 1 : 3], y0[i], y1[i], z0[i], z1[i]};
+                const float k2 = __fmul_rn(2.0f, kc[i]);
+                float D = 0.0f;
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    float m = __fmul_rn(kd[2 * a], rcp_approx(__fadd_rn(kc[i], kd[2 * a]))),
+                          p = __fmul_rn(kd[2 * a + 1], rcp_approx(__fadd_rn(kc[i], kd[2 * a + 1])));
+                    if (a == 0) {
+                        m = i == 0 && first ? dx0 : m;
+                        p = last == i ? dx1 : p;
+                    } else {
+                        m = lo_f[a] ? d_lo[a] : m;
+                        p = hi_f[a] ? d_hi[a] : p;
+                    }
+                    D = __fmaf_rn(__fmul_rn(k2, __fadd_rn(m, p)), r.inv_h2f[a], D);
+                }
+                float u = usum;
+                if (i == 0) u = first ? ux0 : u;
+                u = last == i ? ux1 : u;
+                const bool ok = x + i < nx && !(i == 0 && first && r.held[0]) && !(last == i && r.held[1]);
+                best = fmaxf(best, ok ? __fadd_rn(D, u) : 0.0f);
+            }
+        }
+    }
     block_max_out((double)best, &partials[blockIdx.x]);
     any_risky = __syncthreads_or(any_risky);
     if (threadIdx.x == 0) risky_out[blockIdx.x] = any_risky ? 1.0 : 0.0;
@@ -1339,15 +1500,15 @@ int wfa_total_heat(wfa_grid g, double* e) {
     }
     const Geo geo = geo_of(g);
     if (g->storage == WFA_BF16)
-        heat_partial_kernel<__nv_bfloat16><<<RED_BLOCKS, RED_THREADS, 0, g->stream>>>(
+        heat_partial_kernel<__nv_bfloat16><<<HEAT_BLOCKS, RED_THREADS, 0, g->stream>>>(
             (const __nv_bfloat16*)g->T[g->cur] + domain_offset(g), geo, g->d_partials);
     else
-        heat_partial_kernel<float><<<RED_BLOCKS, RED_THREADS, 0, g->stream>>>(
+        heat_partial_kernel<float><<<HEAT_BLOCKS, RED_THREADS, 0, g->stream>>>(
             (const float*)g->T[g->cur] + domain_offset(g), geo, g->d_partials);
-    finish_sum_kernel<<<1, 512, 0, g->stream>>>(g->d_partials, RED_BLOCKS, g->h[0] * g->h[1] * g->h[2],
-                                                g->d_partials + RED_BLOCKS);
+    finish_sum_kernel<<<1, 512, 0, g->stream>>>(g->d_partials, HEAT_BLOCKS, g->h[0] * g->h[1] * g->h[2],
+                                                g->d_partials + HEAT_BLOCKS);
     WFA_CUDA(cudaGetLastError());
-    WFA_CUDA(cudaMemcpyAsync(g->h_result, g->d_partials + RED_BLOCKS, sizeof(double), cudaMemcpyDeviceToHost,
+    WFA_CUDA(cudaMemcpyAsync(g->h_result, g->d_partials + HEAT_BLOCKS, sizeof(double), cudaMemcpyDeviceToHost,
                              g->stream));
     rc_ = check_status(g);
     *e = g->h_result[0];
