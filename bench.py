@@ -34,6 +34,7 @@ sys.path.insert(0, ROOT)
 METRIC = "cell-updates/s (GLUPS) and % HBM roofline on 1 GB300; serving p50/p99 latency"
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "traffic.json")
 KERNEL_SOURCES = ["paper_2209_13768_gb300/csrc/wfa_sweep_col.cuh", "paper_2209_13768_gb300/csrc/wfa_sweep.cuh",
+                  "paper_2209_13768_gb300/csrc/wfa_sweep_pair.cuh", "paper_2209_13768_gb300/csrc/wfa_sweep_pair_k.cuh",
                   "paper_2209_13768_gb300/csrc/wfa_internal.cuh"]
 
 
