@@ -54,7 +54,9 @@ struct NvtxRange {
 // Launch with programmatic serialization: the kernel's blocks may become
 // resident while the kernel before it in the stream drains, and start with
 // grid_wait(), which returns when that kernel has ended and its writes are
-// visible. For kernels that call it before anything else. Measured: 333x250x187
+// visible. For kernels that call it before anything else and that read what
+// such a kernel writes by coherent loads only (ld_f4 and so on, wfa_sweep.cuh):
+// the read-only path does not take part in that visibility. Measured: 333x250x187
 // bf16, per-cell k 31.5 -> 30.0 us a step, 512^3 210 -> 208. Not while the
 // stream is captured: the nodes of a graph follow one another faster without
 // (64^3 runs of 32 passes: 2.9 us a pass against 4.1).
@@ -80,8 +82,7 @@ cudaError_t launch_overlapped(void (*k)(P...), dim3 grid, dim3 block, cudaStream
 #ifdef __CUDACC__
 // Lets the next kernel's blocks in, then waits for the kernel before (nothing
 // to wait for unless launched with launch_overlapped). The pointers that the
-// kernel loads through pass through here: a read-only load could otherwise be
-// moved above the wait.
+// kernel loads through pass through here, so that no load is moved above the wait.
 template <typename T, typename U>
 __device__ __forceinline__ void grid_wait(T*& a, U*& b) {
     asm volatile("griddepcontrol.launch_dependents;");

@@ -85,6 +85,41 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, u
         : "memory");
 }
 
+// Loads of the field a pass reads. They are coherent (ld.global, through L1)
+// and not the read-only ones (__ldg, or what the compiler makes of a const
+// __restrict__ pointer): those want data that nobody writes while the kernel
+// lives, and a pass launched with launch_overlapped is resident while the pass
+// before it still writes this field. grid_wait makes those writes visible to
+// coherent loads that follow it; the addresses come from the pointer that
+// passes through it, so the compiler cannot move a load above it. The asm is
+// not volatile, so the loads are scheduled like any other: no kernel that uses
+// them writes what they read.
+__device__ __forceinline__ float4 ld_f4(const void* p) {
+    float4 v;
+    asm("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint4 ld_u4(const void* p) {
+    uint4 v;
+    asm("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint2 ld_u2(const void* p) {
+    uint2 v;
+    asm("ld.global.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float ld_cell(const float* p) {
+    float v;
+    asm("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float ld_cell(const __nv_bfloat16* p) {
+    unsigned short v;
+    asm("ld.global.u16 %0, [%1];" : "=h"(v) : "l"(p));
+    return __uint_as_float((unsigned)v << 16);
+}
+
 // 4 consecutive stored values <-> 4 floats.
 template <typename S> struct Vec4;
 template <> struct Vec4<float> {
@@ -117,12 +152,12 @@ template <> struct Vec4<__nv_bfloat16> {
 // One cell with every boundary rule applied, neighbours read from the field
 // (periodic neighbours from the halo twins). i is the cell's element offset.
 template <typename S, bool KVAR>
-__device__ __forceinline__ float general_cell(const SweepCoef& c, const S* __restrict__ in,
+__device__ __forceinline__ float general_cell(const SweepCoef& c, const S* in,
                                               const float* __restrict__ rk, long long i, int x, int y, int z,
                                               int* status) {
-    const float tc = to_f32<S>(in[i]);
+    const float tc = ld_cell(in + i);
     if (is_held(c, x, y, z)) return tc;
-    const float rc = KVAR ? rk[i] : 0.0f;
+    const float rc = KVAR ? ld_cell(rk + i) : 0.0f;
     const int pos[3] = {x, y, z};
     const long long st[3] = {1, c.sy, c.sz};
     float tn[6], w[6];
@@ -140,8 +175,8 @@ __device__ __forceinline__ float general_cell(const SweepCoef& c, const S* __res
         } else {
             const long long j = i + (side ? st[ax] : -st[ax]);
             if (!WFA_CHK(j >= c.lo && j < c.hi, status, 20, x, y, z, f)) continue;
-            tn[f] = to_f32<S>(in[j]);
-            w[f] = KVAR ? __fadd_rn(face_r(rc, rk[j], c.tcd[ax]), c.adv[f]) : c.w_in[f];
+            tn[f] = ld_cell(in + j);
+            w[f] = KVAR ? __fadd_rn(face_r(rc, ld_cell(rk + j), c.tcd[ax]), c.adv[f]) : c.w_in[f];
         }
     }
     return finish_update(tc, flux_sum(tc, tn[0], tn[1], tn[2], tn[3], tn[4], tn[5], w[0], w[1], w[2], w[3], w[4], w[5]),
@@ -158,8 +193,8 @@ __global__ void __launch_bounds__(256) sweep_simple(const __grid_constant__ Swee
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     if (x >= c.n[0] || y >= c.n[1]) return;
-    const S* __restrict__ in = (const S*)a.tin;
-    S* __restrict__ out = (S*)a.tout;
+    const S* in = (const S*)a.tin;
+    S* out = (S*)a.tout;
     const long long st[3] = {1, c.sy, c.sz};
     for (int z = 0; z < c.n[2]; ++z) {
         const long long i = z * c.sz + y * c.sy + x;

@@ -33,13 +33,14 @@ __device__ __forceinline__ void prefetch_l2_if(const void* p, bool pred) {
 }
 
 // 4 consecutive stored values -> 4 floats, and one value. COH = false reads
-// through the read-only (non-coherent) path; COH = true bypasses L1 (ld.cg),
-// for fields that other blocks rewrite during the same launch.
+// through L1 (ld_f4 and so on: see wfa_sweep.cuh for why not the read-only
+// path); COH = true bypasses L1 (ld.cg), for fields that other blocks rewrite
+// during the same launch.
 template <typename S, bool COH>
 __device__ __forceinline__ void ldg4(const S* p, float v[4]);
 template <>
 __device__ __forceinline__ void ldg4<float, false>(const float* p, float v[4]) {
-    const float4 q = __ldg(reinterpret_cast<const float4*>(p));
+    const float4 q = ld_f4(p);
     v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
 }
 template <>
@@ -54,7 +55,7 @@ __device__ __forceinline__ void unpack_bf16x4(uint2 q, float v[4]) {
 }
 template <>
 __device__ __forceinline__ void ldg4<__nv_bfloat16, false>(const __nv_bfloat16* p, float v[4]) {
-    unpack_bf16x4(__ldg(reinterpret_cast<const uint2*>(p)), v);
+    unpack_bf16x4(ld_u2(p), v);
 }
 template <>
 __device__ __forceinline__ void ldg4<__nv_bfloat16, true>(const __nv_bfloat16* p, float v[4]) {
@@ -64,7 +65,7 @@ template <typename S, bool COH>
 __device__ __forceinline__ float ldg1(const S* p);
 template <>
 __device__ __forceinline__ float ldg1<float, false>(const float* p) {
-    return __ldg(p);
+    return ld_cell(p);
 }
 template <>
 __device__ __forceinline__ float ldg1<float, true>(const float* p) {
@@ -77,7 +78,7 @@ __device__ __forceinline__ float ldg1<__nv_bfloat16, true>(const __nv_bfloat16* 
 }
 template <>
 __device__ __forceinline__ float ldg1<__nv_bfloat16, false>(const __nv_bfloat16* p) {
-    return __bfloat162float(*p);
+    return ld_cell(p);
 }
 
 // One cell with uniform k: boundary faces, held layers and the zero-flux self
@@ -131,7 +132,7 @@ __device__ __forceinline__ void ldgv(const S* p, float v[V]) {
 }
 template <>
 __device__ __forceinline__ void ldgv<__nv_bfloat16, false, 8>(const __nv_bfloat16* p, float v[8]) {
-    const uint4 q = __ldg(reinterpret_cast<const uint4*>(p));
+    const uint4 q = ld_u4(p);
     unpack_bf16x4(make_uint2(q.x, q.y), v);
     unpack_bf16x4(make_uint2(q.z, q.w), v + 4);
 }
@@ -244,11 +245,11 @@ struct ColNb {
         ldgv<S, COH, V>(reinterpret_cast<const S*>(tp + syt), ty_p);
         tx_m = ldg1<S, COH>(reinterpret_cast<const S*>(tp) - 1);
         tx_p = ldg1<S, COH>(reinterpret_cast<const S*>(tp) + V);
-        if (KVAR) {   // 1/k never changes during a launch: read-only path
+        if (KVAR) {
             ldgv<float, false, V>(reinterpret_cast<const float*>(rp - syr), ry_m);
             ldgv<float, false, V>(reinterpret_cast<const float*>(rp + syr), ry_p);
-            rx_m = __ldg(reinterpret_cast<const float*>(rp) - 1);
-            rx_p = __ldg(reinterpret_cast<const float*>(rp) + V);
+            rx_m = ldg1<float, false>(reinterpret_cast<const float*>(rp) - 1);
+            rx_p = ldg1<float, false>(reinterpret_cast<const float*>(rp) + V);
         }
     }
 };

@@ -107,12 +107,12 @@ __device__ __forceinline__ f2 pair_face(f2 ra, f2 rb, f2 tcd) {
 template <typename S> struct RowBuf;
 template <> struct RowBuf<float> {
     float4 q;
-    __device__ __forceinline__ void load(const char* p) { q = __ldg(reinterpret_cast<const float4*>(p)); }
+    __device__ __forceinline__ void load(const char* p) { q = ld_f4(p); }
     __device__ __forceinline__ void get(f2 (&o)[2]) const { o[0] = f2_make(q.x, q.y); o[1] = f2_make(q.z, q.w); }
 };
 template <> struct RowBuf<__nv_bfloat16> {
     uint2 q;
-    __device__ __forceinline__ void load(const char* p) { q = __ldg(reinterpret_cast<const uint2*>(p)); }
+    __device__ __forceinline__ void load(const char* p) { q = ld_u2(p); }
     __device__ __forceinline__ void get(f2 (&o)[2]) const { o[0] = unpack2(q.x); o[1] = unpack2(q.y); }
 };
 template <typename S> __device__ __forceinline__ f2 round2(f2 v) {
