@@ -1339,6 +1339,7 @@ static int prepare_k_halo(wfa_grid g) {
     recip_kernel<<<grid_blocks(all, 256), 256, 0, g->stream>>>(g->k, g->r, all);
     WFA_CUDA(cudaGetLastError());
     g->k_halo_dirty = false;
+    g->k_fresh = true;
     return WFA_OK;
 }
 

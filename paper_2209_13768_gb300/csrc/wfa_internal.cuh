@@ -56,12 +56,13 @@ struct NvtxRange {
 // grid_wait(), which returns when that kernel has ended and its writes are
 // visible. For kernels that call it before anything else and that read what
 // such a kernel writes by coherent loads only (ld_f4 and so on, wfa_sweep.cuh):
-// the read-only path does not take part in that visibility. Measured: 333x250x187
+// the read-only path does not take part in that visibility. overlap = false
+// where the kernel before writes what is read by that path (1/k). Measured: 333x250x187
 // bf16, per-cell k 31.5 -> 30.0 us a step, 512^3 210 -> 208. Not while the
 // stream is captured: the nodes of a graph follow one another faster without
 // (64^3 runs of 32 passes: 2.9 us a pass against 4.1).
 template <typename... P, typename... A>
-cudaError_t launch_overlapped(void (*k)(P...), dim3 grid, dim3 block, cudaStream_t st, A... args) {
+cudaError_t launch_overlapped(void (*k)(P...), dim3 grid, dim3 block, cudaStream_t st, bool overlap, A... args) {
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
@@ -75,7 +76,7 @@ cudaError_t launch_overlapped(void (*k)(P...), dim3 grid, dim3 block, cudaStream
         cap = cudaStreamCaptureStatusActive;
     }
     cfg.attrs = at;
-    cfg.numAttrs = cap == cudaStreamCaptureStatusNone ? 1 : 0;
+    cfg.numAttrs = overlap && cap == cudaStreamCaptureStatusNone ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, k, static_cast<P>(args)...);
 }
 
@@ -164,6 +165,7 @@ struct wfa_grid_s {
     bool limit_valid;
     bool field_set, coeffs_set, dt_set, halo_dirty;
     bool k_halo_dirty;    // k twins / ghost layers and 1/k must be rebuilt before use
+    bool k_fresh;         // 1/k was rebuilt and no pass has been launched since
     long long steps_done;
     int force_depth, force_variant;   // wfa_set_tuning (0 = automatic)
     int force_zchunk;                 // wfa_set_zchunk: planes per z chunk of the column kernels (0 = automatic)

@@ -342,6 +342,8 @@ static SweepArgs base_args(wfa_grid_s* g, const SweepCoef& c, int in_buf, int zc
     a.tout = (char*)g->T[1 - in_buf] + off * g->esize;
     a.rk = g->r ? g->r + off : nullptr;
     a.status = g->d_status;
+    a.fresh_k = g->k_fresh;
+    g->k_fresh = false;
     return a;
 }
 

@@ -35,6 +35,7 @@ struct SweepArgs {
     int tiles_x, tiles_y, zchunk, nzchunk, items;   // column kernels: zchunk > 0 on entry asks for
                                                      // chunks of that many planes (0: automatic)
     int* status;
+    int fresh_k;        // 1/k was written just before: this pass does not overlap that kernel
 };
 
 // --------------------------------------------------------------- PTX helpers --
@@ -157,7 +158,7 @@ __device__ __forceinline__ float general_cell(const SweepCoef& c, const S* in,
                                               int* status) {
     const float tc = ld_cell(in + i);
     if (is_held(c, x, y, z)) return tc;
-    const float rc = KVAR ? ld_cell(rk + i) : 0.0f;
+    const float rc = KVAR ? __ldg(rk + i) : 0.0f;
     const int pos[3] = {x, y, z};
     const long long st[3] = {1, c.sy, c.sz};
     float tn[6], w[6];
@@ -176,7 +177,7 @@ __device__ __forceinline__ float general_cell(const SweepCoef& c, const S* in,
             const long long j = i + (side ? st[ax] : -st[ax]);
             if (!WFA_CHK(j >= c.lo && j < c.hi, status, 20, x, y, z, f)) continue;
             tn[f] = ld_cell(in + j);
-            w[f] = KVAR ? __fadd_rn(face_r(rc, ld_cell(rk + j), c.tcd[ax]), c.adv[f]) : c.w_in[f];
+            w[f] = KVAR ? __fadd_rn(face_r(rc, __ldg(rk + j), c.tcd[ax]), c.adv[f]) : c.w_in[f];
         }
     }
     return finish_update(tc, flux_sum(tc, tn[0], tn[1], tn[2], tn[3], tn[4], tn[5], w[0], w[1], w[2], w[3], w[4], w[5]),

@@ -34,7 +34,7 @@ __device__ __forceinline__ void prefetch_l2_if(const void* p, bool pred) {
 
 // 4 consecutive stored values -> 4 floats, and one value. COH = false reads
 // through L1 (ld_f4 and so on: see wfa_sweep.cuh for why not the read-only
-// path); COH = true bypasses L1 (ld.cg), for fields that other blocks rewrite
+// path, which 1/k takes: ldrk); COH = true bypasses L1 (ld.cg), for fields that other blocks rewrite
 // during the same launch.
 template <typename S, bool COH>
 __device__ __forceinline__ void ldg4(const S* p, float v[4]);
@@ -152,6 +152,17 @@ __device__ __forceinline__ void ldgv<__nv_bfloat16, true, 16>(const __nv_bfloat1
     ldgv<__nv_bfloat16, true, 8>(p, v);
     ldgv<__nv_bfloat16, true, 8>(p + 8, v + 8);
 }
+// 1/k of V cells. It never changes while a pass runs, nor while the pass is
+// resident before it starts (see launch_overlapped): read-only path (coherent
+// loads: periodic grids 3 to 5% slower).
+template <int V>
+__device__ __forceinline__ void ldrk(const float* p, float v[V]) {
+#pragma unroll
+    for (int i = 0; i < V; i += 4) {
+        const float4 q = __ldg(reinterpret_cast<const float4*>(p + i));
+        v[i] = q.x; v[i + 1] = q.y; v[i + 2] = q.z; v[i + 3] = q.w;
+    }
+}
 template <typename S, int V>
 __device__ __forceinline__ void stv(S* p, const float v[V]) {
 #pragma unroll
@@ -246,10 +257,10 @@ struct ColNb {
         tx_m = ldg1<S, COH>(reinterpret_cast<const S*>(tp) - 1);
         tx_p = ldg1<S, COH>(reinterpret_cast<const S*>(tp) + V);
         if (KVAR) {
-            ldgv<float, false, V>(reinterpret_cast<const float*>(rp - syr), ry_m);
-            ldgv<float, false, V>(reinterpret_cast<const float*>(rp + syr), ry_p);
-            rx_m = ldg1<float, false>(reinterpret_cast<const float*>(rp) - 1);
-            rx_p = ldg1<float, false>(reinterpret_cast<const float*>(rp) + V);
+            ldrk<V>(reinterpret_cast<const float*>(rp - syr), ry_m);
+            ldrk<V>(reinterpret_cast<const float*>(rp + syr), ry_p);
+            rx_m = __ldg(reinterpret_cast<const float*>(rp) - 1);
+            rx_p = __ldg(reinterpret_cast<const float*>(rp) + V);
         }
     }
 };
@@ -320,8 +331,8 @@ __device__ __forceinline__ void col_run(const SweepCoef& c, const S* __restrict_
     ldgv<S, COH, V>(tcol + (long long)zs * sz, tc);
     if (KVAR) {
         float rb[V];
-        ldgv<float, false, V>(rcol + (long long)(zs - DIR) * sz, rb);
-        ldgv<float, false, V>(rcol + (long long)zs * sz, rc);
+        ldrk<V>(rcol + (long long)(zs - DIR) * sz, rb);
+        ldrk<V>(rcol + (long long)zs * sz, rc);
 #pragma unroll
         for (int i = 0; i < V; ++i) gzm[i] = face_r(rb[i], rc[i], c.tcd[2]);
     }
@@ -374,7 +385,7 @@ __device__ __forceinline__ void col_run(const SweepCoef& c, const S* __restrict_
             prefetch_l2_if(tP + 3 * dzt, pf_lead && s + 3 <= len);
             if (KVAR) prefetch_l2_if(rP + 3 * dzr, pf_lead && s + 3 <= len);
         }
-        if (KVAR) ldgv<float, false, V>(reinterpret_cast<const float*>(rP + dzr), rz);
+        if (KVAR) ldrk<V>(reinterpret_cast<const float*>(rP + dzr), rz);
         ColNb<S, KVAR, COH, V> nb;                       // x / y neighbours, plane z
         nb.load(tP, rP, (long long)syt, (long long)syr);
         S* const op = reinterpret_cast<S*>(oP);          // this thread's cells at plane z
@@ -677,18 +688,18 @@ cudaError_t col_launch_v(const SweepArgs& a_in, cudaStream_t st, int nsm, const 
     if (ev) cudaEventRecord(ev[0], st);
     cudaError_t e;
     if (inl) {
-        if (adv) e = launch_overlapped(sweep_col<S, KVAR, true, true>, grid, block, st, a);
-        else e = launch_overlapped(sweep_col<S, KVAR, false, true>, grid, block, st, a);
+        if (adv) e = launch_overlapped(sweep_col<S, KVAR, true, true>, grid, block, st, !a.fresh_k, a);
+        else e = launch_overlapped(sweep_col<S, KVAR, false, true>, grid, block, st, !a.fresh_k, a);
     } else if (a.c.held[0] || a.c.held[1] || a.c.held[2] || a.c.held[3] || a.c.held[4] || a.c.held[5]) {
         // held cell layers: kept in the pass (copies for any periodic axis too)
-        if (adv) e = launch_overlapped(sweep_col<S, KVAR, true, false, V, true, true>, grid, block, st, a);
-        else e = launch_overlapped(sweep_col<S, KVAR, false, false, V, true, true>, grid, block, st, a);
+        if (adv) e = launch_overlapped(sweep_col<S, KVAR, true, false, V, true, true>, grid, block, st, !a.fresh_k, a);
+        else e = launch_overlapped(sweep_col<S, KVAR, false, false, V, true, true>, grid, block, st, !a.fresh_k, a);
     } else if (a.c.periodic[0] || a.c.periodic[1] || a.c.periodic[2]) {
-        if (adv) e = launch_overlapped(sweep_col<S, KVAR, true, false, V, true>, grid, block, st, a);
-        else e = launch_overlapped(sweep_col<S, KVAR, false, false, V, true>, grid, block, st, a);
+        if (adv) e = launch_overlapped(sweep_col<S, KVAR, true, false, V, true>, grid, block, st, !a.fresh_k, a);
+        else e = launch_overlapped(sweep_col<S, KVAR, false, false, V, true>, grid, block, st, !a.fresh_k, a);
     } else {   // no periodic axis: no copies to store
-        if (adv) e = launch_overlapped(sweep_col<S, KVAR, true, false, V, false>, grid, block, st, a);
-        else e = launch_overlapped(sweep_col<S, KVAR, false, false, V, false>, grid, block, st, a);
+        if (adv) e = launch_overlapped(sweep_col<S, KVAR, true, false, V, false>, grid, block, st, !a.fresh_k, a);
+        else e = launch_overlapped(sweep_col<S, KVAR, false, false, V, false>, grid, block, st, !a.fresh_k, a);
     }
     if (ev) cudaEventRecord(ev[1], st);
     if (e != cudaSuccess || inl || a.c.halo_bc) return e;
@@ -700,7 +711,7 @@ cudaError_t col_launch_v(const SweepArgs& a_in, cudaStream_t st, int nsm, const 
     }
     if (plane == 0) return cudaSuccess;
     const int nb = (int)std::min<long long>((plane + 255) / 256, (long long)nsm * 2);
-    return launch_overlapped(boundary_fix<S, KVAR, true>, dim3(nb, 6), dim3(256), st, a);
+    return launch_overlapped(boundary_fix<S, KVAR, true>, dim3(nb, 6), dim3(256), st, !a.fresh_k, a);
 }
 
 template <typename S, bool KVAR>

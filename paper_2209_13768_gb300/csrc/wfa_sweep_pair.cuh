@@ -108,6 +108,7 @@ template <typename S> struct RowBuf;
 template <> struct RowBuf<float> {
     float4 q;
     __device__ __forceinline__ void load(const char* p) { q = ld_f4(p); }
+    __device__ __forceinline__ void load_rk(const char* p) { q = __ldg(reinterpret_cast<const float4*>(p)); }   // see ldrk
     __device__ __forceinline__ void get(f2 (&o)[2]) const { o[0] = f2_make(q.x, q.y); o[1] = f2_make(q.z, q.w); }
 };
 template <> struct RowBuf<__nv_bfloat16> {
@@ -426,10 +427,10 @@ cudaError_t pair_launch(const SweepArgs& a_in, cudaStream_t st, int nsm, const c
     if (ev) cudaEventRecord(ev[0], st);
     cudaError_t e;
     const bool per = a.c.periodic[0] || a.c.periodic[1] || a.c.periodic[2], rag = a.c.n[0] % 4 != 0;
-    if (per && rag) e = launch_overlapped(sweep_pair<S, true, true, Cfg::R, Cfg::WPB, Cfg::BLOCKS>, grid, block, st, a);
-    else if (per) e = launch_overlapped(sweep_pair<S, true, false, Cfg::R, Cfg::WPB, Cfg::BLOCKS>, grid, block, st, a);
-    else if (rag) e = launch_overlapped(sweep_pair<S, false, true, Cfg::R, Cfg::WPB, Cfg::BLOCKS>, grid, block, st, a);
-    else e = launch_overlapped(sweep_pair<S, false, false, Cfg::R, Cfg::WPB, Cfg::BLOCKS>, grid, block, st, a);
+    if (per && rag) e = launch_overlapped(sweep_pair<S, true, true, Cfg::R, Cfg::WPB, Cfg::BLOCKS>, grid, block, st, !a.fresh_k, a);
+    else if (per) e = launch_overlapped(sweep_pair<S, true, false, Cfg::R, Cfg::WPB, Cfg::BLOCKS>, grid, block, st, !a.fresh_k, a);
+    else if (rag) e = launch_overlapped(sweep_pair<S, false, true, Cfg::R, Cfg::WPB, Cfg::BLOCKS>, grid, block, st, !a.fresh_k, a);
+    else e = launch_overlapped(sweep_pair<S, false, false, Cfg::R, Cfg::WPB, Cfg::BLOCKS>, grid, block, st, !a.fresh_k, a);
     if (ev) cudaEventRecord(ev[1], st);
     return e;
 }

@@ -143,7 +143,7 @@ __device__ __forceinline__ void pair_k_run(const SweepCoef& c, const void* tin, 
     auto load_wrapped = [&](RowBuf<S>& t, RowBuf<float>& k, int j, int z) {
         if (!PER) {
             t.load(reinterpret_cast<const char*>(tP + j * sy + (z - q) * sz));
-            k.load(reinterpret_cast<const char*>(rP + j * sy + (z - q) * sz));
+            k.load_rk(reinterpret_cast<const char*>(rP + j * sy + (z - q) * sz));
             return;
         }
         int y = yl + j;
@@ -151,7 +151,7 @@ __device__ __forceinline__ void pair_k_run(const SweepCoef& c, const void* tin, 
         if (perz) z = z < 0 ? z + nz : z >= nz ? z - nz : z;
         const long long row = y * sy + z * sz;
         t.load(reinterpret_cast<const char*>(tX + row + lx));
-        k.load(reinterpret_cast<const char*>(rk + row + lx));
+        k.load_rk(reinterpret_cast<const char*>(rk + row + lx));
     };
 #pragma unroll
     for (int j = 0; j < R; ++j) {
@@ -299,12 +299,12 @@ __device__ __forceinline__ void pair_k_run(const SweepCoef& c, const void* tin, 
 #pragma unroll
                 for (int j = 0; j < R; ++j) {
                     Tc[j].load(reinterpret_cast<const char*>(tP + 2 * sz + j * sy));
-                    Kc[j].load(reinterpret_cast<const char*>(rP + 2 * sz + j * sy));
+                    Kc[j].load_rk(reinterpret_cast<const char*>(rP + 2 * sz + j * sy));
                 }
                 H[0].load(reinterpret_cast<const char*>(tP + sz - sy));
                 H[1].load(reinterpret_cast<const char*>(tP + sz + R * sy));
-                KH[0].load(reinterpret_cast<const char*>(rP + sz - sy));
-                KH[1].load(reinterpret_cast<const char*>(rP + sz + R * sy));
+                KH[0].load_rk(reinterpret_cast<const char*>(rP + sz - sy));
+                KH[1].load_rk(reinterpret_cast<const char*>(rP + sz + R * sy));
             }
             if ((lane & 7) == 0 && q + 4 <= z1 + 1) {
 #pragma unroll
@@ -372,10 +372,10 @@ template <typename S, bool ADV>
 cudaError_t pair_k_dispatch(const SweepArgs& a, const PairTiles& tl, dim3 grid, cudaStream_t st) {
     const dim3 block(32 * PairKCfg::W);
     const bool per = a.c.periodic[0] || a.c.periodic[1] || a.c.periodic[2], rag = a.c.n[0] % 4 != 0;
-    if (per && rag) return launch_overlapped(sweep_pair_k<S, true, true, ADV>, grid, block, st, a, tl);
-    if (per) return launch_overlapped(sweep_pair_k<S, true, false, ADV>, grid, block, st, a, tl);
-    if (rag) return launch_overlapped(sweep_pair_k<S, false, true, ADV>, grid, block, st, a, tl);
-    return launch_overlapped(sweep_pair_k<S, false, false, ADV>, grid, block, st, a, tl);
+    if (per && rag) return launch_overlapped(sweep_pair_k<S, true, true, ADV>, grid, block, st, !a.fresh_k, a, tl);
+    if (per) return launch_overlapped(sweep_pair_k<S, true, false, ADV>, grid, block, st, !a.fresh_k, a, tl);
+    if (rag) return launch_overlapped(sweep_pair_k<S, false, true, ADV>, grid, block, st, !a.fresh_k, a, tl);
+    return launch_overlapped(sweep_pair_k<S, false, false, ADV>, grid, block, st, !a.fresh_k, a, tl);
 }
 
 // z chunks of a launch of `tiles` blocks a chunk: whole waves of resident

@@ -12,16 +12,23 @@ def _read(name):
 
 def test_overlapped_kernels_read_by_coherent_loads():
     """A kernel launched with launch_overlapped is resident while the kernel
-    before it writes the field it reads: no read-only (non-coherent) loads, nor
-    plain reads through a const __restrict__ pointer, which the compiler may
-    turn into them; and each waits before anything else."""
+    before it writes the field it reads: no read-only (non-coherent) loads of it,
+    nor plain reads through a const __restrict__ pointer, which the compiler may
+    turn into them; and each waits before anything else. 1/k alone is read by
+    that path: a pass right after the kernel that wrote it does not overlap."""
     launched = set()
     headers = {n: _read(n) for n in sorted(os.listdir(CSRC)) if n.endswith((".cuh", ".cu"))}
     for text in headers.values():
-        launched |= set(re.findall(r"launch_overlapped\((\w+)<", text))
+        calls = re.findall(r"launch_overlapped\((\w+)<[^;]*;", text)
+        launched |= set(calls)
+        assert len(calls) == len(re.findall(r"launch_overlapped\(\w+<[^;]*, st, !a\.fresh_k, a[^;]*;", text))
     assert launched == {"sweep_pair", "sweep_pair_k", "sweep_col", "boundary_fix"}
     for name in ("wfa_sweep.cuh", "wfa_sweep_col.cuh", "wfa_sweep_pair.cuh", "wfa_sweep_pair_k.cuh"):
-        assert not re.search(r"__ldg\b|ld\.global\.nc|ldca|ld\.relaxed", headers[name]), name
+        text = re.sub(r"void (ldrk|load_rk)\((.*?)\n\s*(}|RowBuf|__device__)", "", headers[name], flags=re.S)
+        text = re.sub(r"__ldg\((rk \+ \w|reinterpret_cast<const float\*>\(rp\))", "", text)
+        assert not re.search(r"__ldg\b|ld\.global\.nc|ldca|ld\.relaxed", text), name
+    pair_k = headers["wfa_sweep_pair_k.cuh"]
+    assert not re.search(r"\b(t|T[01n]|Tc\[j\]|H\[\d\])\.load_rk", pair_k)
     whole = "\n".join(headers.values())
     for k in launched:
         body = re.search(r"\b%s\(const __grid_constant__ SweepArgs a[^)]*\) \{(.*?)\n\}\n" % k, whole, re.S).group(1)
@@ -30,3 +37,5 @@ def test_overlapped_kernels_read_by_coherent_loads():
         assert "a.tin" not in body.split("grid_wait", 1)[1] and "a.rk" not in body.split("grid_wait", 1)[1], k
     cell = re.search(r"float general_cell\((.*?)\n\}\n", headers["wfa_sweep.cuh"], re.S).group(1)
     assert not re.search(r"\b(in|rk)\[", cell)
+    prepare = re.search(r"int prepare_k_halo\((.*?)\n\}\n", headers["wfa_grid.cu"], re.S).group(1)
+    assert prepare.index("recip_kernel") < prepare.index("k_fresh = true")
