@@ -273,8 +273,8 @@ struct ColNb {
 // uniform k). Register-level prefetch was slower: it costs the occupancy.
 template <bool KVAR, bool INL = false, int ES = 4, int V = 4> struct ColOcc {
     static constexpr int blocks = V == 16 ? 3 : V == 8 ? (KVAR ? 2 : 4) : INL ? (KVAR ? 3 : 4) : (KVAR ? 4 : 6);
-    // measured: uniform k prefers the z loop unrolled twice (fp32 with 4
-    // cells a thread, bf16 with 8), per-cell k not
+    // measured: uniform k prefers the z loop unrolled twice (fp32 with 4 cells a
+    // thread, bf16 with 8; see sweep_col for the one that spills then), per-cell k not
     static constexpr int unroll = KVAR ? 1 : (V == 4 && ES == 4) || (V == 8 && ES == 2) ? 2 : 1;
 };
 
@@ -553,7 +553,10 @@ __global__ void __launch_bounds__(256, (ColOcc<KVAR, INL, sizeof(S), V>::blocks)
     if (gx >= c.n[0] || gy >= c.n[1]) return;
     const int z0 = blockIdx.z * a.zchunk;
     const int z1 = min(z0 + a.zchunk, c.n[2]);
-    constexpr int U = ColOcc<KVAR, INL, sizeof(S), V>::unroll;
+    // fp32, uniform k, 4 cells, neither copies nor held cells: unrolled twice it
+    // spills 44 bytes, and is 2 to 9% slower (512^3 216 against 199 us a step,
+    // 128^3 8.4 / 7.9); storing copies, twice is 3 to 7% faster
+    constexpr int U = !KVAR && V == 4 && sizeof(S) == 4 && !TW ? 1 : ColOcc<KVAR, INL, sizeof(S), V>::unroll;
     constexpr ColMode MODE = INL ? COL_INPLACE : COL_THIN;
     if (blockIdx.z & 1)   // odd chunks march down: see col_run
         col_run<S, KVAR, ADV, false, U, MODE, true, false, -1, V, TW, HELD>(c, (const S*)tin, (S*)a.tout, rk,
