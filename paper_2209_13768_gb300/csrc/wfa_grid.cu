@@ -169,7 +169,8 @@ int build_coef(const wfa_grid_s* g, SweepCoef* c) {
             const int f = 2 * a + side;
             const double A = side == 0 ? ap : am;
             c->bkind[f] = g->bc_kind[f];
-            c->tb[f] = (float)g->bc_value[f];
+            // other kinds ignore their value (the passes multiply by tb with weight 0 there)
+            c->tb[f] = g->bc_kind[f] == WFA_BC_DIRICHLET ? (float)g->bc_value[f] : 0.0f;
             c->held[f] = g->bc_kind[f] == WFA_BC_DIRICHLET_CELL;
             c->ext[f] = g->bc_kind[f] == WFA_BC_EXCHANGE;
             if (g->bc_kind[f] == WFA_BC_DIRICHLET) c->w_bd[f] = (float)(2.0 * g->k_uniform * cd + A);
