@@ -420,10 +420,11 @@ cudaError_t pair_launch(const SweepArgs& a_in, cudaStream_t st, int nsm, const c
     constexpr int ZMAX = sizeof(S) == 4 ? 16 : 24;
     const long long want = std::max<long long>(1, (4 * resident + tiles - 1) / tiles);
     int nch = (int)std::min<long long>(std::max<long long>(want, (a.c.n[2] + ZMAX - 1) / ZMAX), (a.c.n[2] + 3) / 4);
+    nch = std::min(nch, 65535);
     if (a_in.zchunk > 0) nch = (a.c.n[2] + a_in.zchunk - 1) / a_in.zchunk;
     a.zchunk = (a.c.n[2] + nch - 1) / nch;
     nch = (a.c.n[2] + a.zchunk - 1) / a.zchunk;
-    const dim3 grid(gxb, gyb, nch), block(32, Cfg::WPB);
+    const dim3 grid(gxb, gyb, nch), block(32, Cfg::WPB);   // gyb: see pair_applies
     if (ev) cudaEventRecord(ev[0], st);
     cudaError_t e;
     const bool per = a.c.periodic[0] || a.c.periodic[1] || a.c.periodic[2], rag = a.c.n[0] % 4 != 0;

@@ -379,11 +379,12 @@ cudaError_t pair_k_dispatch(const SweepArgs& a, const PairTiles& tl, dim3 grid, 
 }
 
 // z chunks of a launch of `tiles` blocks a chunk: whole waves of resident
-// blocks against the planes a chunk steps but does not store.
+// blocks against the planes a chunk steps but does not store. At most 1024
+// chunks (three waves of the smallest tile count; the loop runs at every launch).
 inline int pair_k_chunk(int nz, long long tiles, long long resident) {
     int best = nz;
     double cost = 1e300;
-    for (int n = 1; n <= (nz + 3) / 4; ++n) {
+    for (int n = 1; n <= std::min((nz + 3) / 4, 1024); ++n) {
         const int zc = (nz + n - 1) / n;
         const double waves = (double)((tiles * ((nz + zc - 1) / zc) + resident - 1) / resident);
         if (waves * (zc + 4) < cost * 0.995) {
