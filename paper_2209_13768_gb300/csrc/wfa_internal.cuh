@@ -77,7 +77,9 @@ cudaError_t launch_overlapped(void (*k)(P...), dim3 grid, dim3 block, cudaStream
     }
     cfg.attrs = at;
     cfg.numAttrs = overlap && cap == cudaStreamCaptureStatusNone ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, k, static_cast<P>(args)...);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, k, static_cast<P>(args)...);
+    if (e != cudaSuccess) cudaGetLastError();   // reported here, not by the next call too
+    return e;
 }
 
 #ifdef __CUDACC__
