@@ -419,7 +419,7 @@ int refresh_halo(wfa_grid_s* g, int buf) {
 }
 
 // --------------------------------------------------------------- reductions --
-constexpr int HEAT_BLOCKS = 152 * 8;   // resident blocks: a warp a row
+constexpr int HEAT_BLOCKS = 152 * 8;   // resident blocks
 // the stability passes are latency-bound (divisions, seven k reads a cell):
 // more warps per SM; their partials fit the 4096-double scratch below the
 // word kept for the k check (index 4095)
@@ -430,74 +430,77 @@ static_assert(RATE_P2 > RATE_BLOCKS + 1 && RATE_P2 + RATE_BLOCKS <= RATE_RISKY &
               "scratch layout");
 constexpr int RED_THREADS = 256;
 
-// a + b = s + e exactly (round to nearest, no overflow).
+// a + b = s + e exactly (Knuth's error-free sum; round to nearest, no overflow).
 __device__ __forceinline__ float two_sum(float a, float b, float* e) {
     const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
     *e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
     return s;
 }
 
-// Sum of the field in fp64. Bound by HBM with a warp per row and 4 cells a
-// lane, once the GPU's fp64 rate (a conversion and an addition a cell) is out
-// of the loop: a thread adds in fp32 with the exact rounding error of every
-// addition, and sums the errors with compensation, which rounds less than fp64
-// additions do. Sums that leave the fp32 range (or inf, NaN) go to fp64.
-// 512^3: 1.39 ms with a 64-bit division and an fp64 addition a cell, 0.36 with
-// one fp64 addition for 4 cells, 0.17 now (3.1 TB/s).
+// Sum of the field in fp64, with one rounding of an fp64 sum for every 16
+// cells (a thread's block of four 4-cell groups) where an addition a cell has
+// 16: a row takes 32 lanes (short rows fewer), a block's cells are summed in fp32 with the exact error of
+// every addition, the errors likewise, and what that second sum rounds off
+// (2^-48 of the block and less) is kept in fp32 to the end. So the GPU's fp64
+// rate (two conversions and additions a block) is out of the way; blocks that
+// leave the fp32 range (or hold inf, NaN) are added cell by cell. Bound by HBM and issue.
+// A call on 512^3: 1.42 ms with a 64-bit division and an fp64 addition a cell, 0.34
+// now; 31x500x500 0.24 -> 0.19 (a warp a row there: 0.32).
 template <typename S>
 __global__ void __launch_bounds__(RED_THREADS) heat_partial_kernel(const S* __restrict__ origin, const __grid_constant__ Geo geo,
-                                                                   double* __restrict__ partials) {
+                                                                   int lanes, double* __restrict__ partials) {
     __shared__ double sh[RED_THREADS];
-    const int nx = geo.n[0], ny = geo.n[1], lane = threadIdx.x & 31;
+    const int nx = geo.n[0], ny = geo.n[1];
     const long long sz = geo.px * geo.py, rows = (long long)ny * geo.n[2];
-    const long long warps = (long long)gridDim.x * (RED_THREADS / 32);
-    double acc = 0.0;
-    float fs = 0.0f, es = 0.0f, ec = 0.0f;   // the fp32 sum; the errors' sum and its compensation
-    auto add4 = [&](const float (&v)[4]) {
-        float e0, e1, e2, e3;
-        const float s0 = two_sum(v[0], v[1], &e0), s1 = two_sum(v[2], v[3], &e1), t = two_sum(s0, s1, &e2),
-                    f = two_sum(fs, t, &e3);
-        const float e = __fadd_rn(__fadd_rn(e0, e1), __fadd_rn(e2, e3));
-        if (fabsf(f) < INFINITY && fabsf(e) < INFINITY) {   // no partial sum left the range
-            fs = f;
-            const float y = __fsub_rn(e, ec), u = __fadd_rn(es, y);
-            ec = __fsub_rn(__fsub_rn(u, es), y);
-            es = u;
-        } else {
-            acc += ((((double)v[0] + (double)v[1]) + (double)v[2]) + (double)v[3]) + (double)fs;
-            fs = 0.0f;
-        }
-    };
-    for (long long row = blockIdx.x * (long long)(RED_THREADS / 32) + (threadIdx.x >> 5); row < rows; row += warps) {
+    const int per = RED_THREADS / lanes, lane = threadIdx.x & (lanes - 1);   // rows a block takes at a time
+    double acc = 0.0, err = 0.0;   // the blocks' sums; their errors
+    float rest = 0.0f;             // what the errors' sums rounded off
+    for (long long row = blockIdx.x * (long long)per + threadIdx.x / lanes; row < rows; row += (long long)gridDim.x * per) {
         const int z = (int)((unsigned long long)row / (unsigned)ny), y = (int)(row - (long long)z * ny);
         const S* o = origin + z * sz + y * geo.px;
-        for (int x0 = 4 * lane; x0 < nx; x0 += 512) {   // four groups' loads in flight
-            float v[4][4];
+        for (int x0 = 4 * lane; x0 < nx; x0 += 16 * lanes) {   // a block: four groups' loads in flight
+            float v[16];
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                const int x = x0 + 128 * u;
-                v[u][0] = v[u][1] = v[u][2] = v[u][3] = 0.0f;
+                const int x = x0 + 4 * lanes * u;
+                v[4 * u] = v[4 * u + 1] = v[4 * u + 2] = v[4 * u + 3] = 0.0f;
                 if (x >= nx) continue;
                 if constexpr (sizeof(S) == 4) {
                     const float4 q = __ldg(reinterpret_cast<const float4*>(o + x));
-                    v[u][0] = q.x; v[u][1] = q.y; v[u][2] = q.z; v[u][3] = q.w;
+                    v[4 * u] = q.x; v[4 * u + 1] = q.y; v[4 * u + 2] = q.z; v[4 * u + 3] = q.w;
                 } else {
                     const uint2 q = __ldg(reinterpret_cast<const uint2*>(o + x));
-                    v[u][0] = __uint_as_float(q.x << 16); v[u][1] = __uint_as_float(q.x & 0xffff0000u);
-                    v[u][2] = __uint_as_float(q.y << 16); v[u][3] = __uint_as_float(q.y & 0xffff0000u);
+                    v[4 * u] = __uint_as_float(q.x << 16); v[4 * u + 1] = __uint_as_float(q.x & 0xffff0000u);
+                    v[4 * u + 2] = __uint_as_float(q.y << 16); v[4 * u + 3] = __uint_as_float(q.y & 0xffff0000u);
                 }
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int x = x0 + 128 * u;
 #pragma unroll
                 for (int i = 1; i < 4; ++i)
-                    if (x + i >= nx) v[u][i] = 0.0f;
-                add4(v[u]);
+                    if (x + i >= nx) v[4 * u + i] = 0.0f;
+            }
+            float s[16], e[15], c = 0.0f;
+#pragma unroll
+            for (int i = 0; i < 16; ++i) s[i] = v[i];
+#pragma unroll
+            for (int w = 8, k = 0; w >= 1; k += w, w /= 2)   // a tree: pairs, pairs of pairs, ...
+#pragma unroll
+                for (int i = 0; i < w; ++i) s[i] = two_sum(s[i], s[i + w], &e[k + i]);
+#pragma unroll
+            for (int i = 13; i >= 0; --i) {   // the late, larger errors first
+                float d;
+                e[14] = two_sum(e[14], e[i], &d);
+                c = __fadd_rn(c, d);
+            }
+            if (fabsf(s[0]) < INFINITY && fabsf(e[14]) < INFINITY) {   // no partial sum left the range
+                acc += (double)s[0];
+                err += (double)e[14];
+                rest = __fadd_rn(rest, c);
+            } else {
+#pragma unroll
+                for (int i = 0; i < 16; ++i) acc += (double)v[i];
             }
         }
     }
-    sh[threadIdx.x] = (acc + (double)fs) + ((double)es - (double)ec);
+    sh[threadIdx.x] = acc + (err + (double)rest);
     __syncthreads();
     for (int s = RED_THREADS / 2; s > 0; s >>= 1) {
         if (threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s];
@@ -1501,16 +1504,19 @@ int wfa_total_heat(wfa_grid g, double* e) {
         if (rc) return rc;
     }
     const Geo geo = geo_of(g);
+    int lanes = 32;   // lanes a row: the fewest (a power of two) whose 4 cells each cover it, so short rows fill their warps
+    while (lanes > 1 && 2 * lanes >= g->n[0]) lanes /= 2;
+    const long long rows = (long long)g->n[1] * g->n[2], per = RED_THREADS / lanes;
+    const int nb = (int)std::min<long long>(HEAT_BLOCKS, (rows + per - 1) / per);
     if (g->storage == WFA_BF16)
-        heat_partial_kernel<__nv_bfloat16><<<HEAT_BLOCKS, RED_THREADS, 0, g->stream>>>(
-            (const __nv_bfloat16*)g->T[g->cur] + domain_offset(g), geo, g->d_partials);
+        heat_partial_kernel<__nv_bfloat16><<<nb, RED_THREADS, 0, g->stream>>>(
+            (const __nv_bfloat16*)g->T[g->cur] + domain_offset(g), geo, lanes, g->d_partials);
     else
-        heat_partial_kernel<float><<<HEAT_BLOCKS, RED_THREADS, 0, g->stream>>>(
-            (const float*)g->T[g->cur] + domain_offset(g), geo, g->d_partials);
-    finish_sum_kernel<<<1, 512, 0, g->stream>>>(g->d_partials, HEAT_BLOCKS, g->h[0] * g->h[1] * g->h[2],
-                                                g->d_partials + HEAT_BLOCKS);
+        heat_partial_kernel<float><<<nb, RED_THREADS, 0, g->stream>>>(
+            (const float*)g->T[g->cur] + domain_offset(g), geo, lanes, g->d_partials);
+    finish_sum_kernel<<<1, 512, 0, g->stream>>>(g->d_partials, nb, g->h[0] * g->h[1] * g->h[2], g->d_partials + nb);
     WFA_CUDA(cudaGetLastError());
-    WFA_CUDA(cudaMemcpyAsync(g->h_result, g->d_partials + HEAT_BLOCKS, sizeof(double), cudaMemcpyDeviceToHost,
+    WFA_CUDA(cudaMemcpyAsync(g->h_result, g->d_partials + nb, sizeof(double), cudaMemcpyDeviceToHost,
                              g->stream));
     rc_ = check_status(g);
     *e = g->h_result[0];
