@@ -592,12 +592,15 @@ struct CgPlace {
 // ghost value (cg_q4's) put in its place, and cells that are not free get
 // q = 0; next to a y or z face cg_q4 goes row by row. zf: the faces towards
 // z - 1 on entry, towards z + 1 on return; kz: 1/k of the first row at z - 1.
+// dot takes the 4 products of each row at a time: what a plain fp32 sum of them
+// rounds off is all that the compensated sum does not see.
 template <bool KVAR>
-__device__ __forceinline__ float cg_rows(const CgCoef& c, const CgPlace& t, int z, f2 (&pc)[CG_R][2],
+__device__ __forceinline__ void cg_rows(const CgCoef& c, const CgPlace& t, int z, f2 (&pc)[CG_R][2],
                                          const f2 (&pm)[CG_R][2], const f2 (&pp)[CG_R][2], const f2 (&h)[2][2],
                                          const float (&e)[CG_R], f2 (&kc)[KVAR ? CG_R : 1][2],
                                          f2 (&zf)[KVAR ? CG_R : 1][2], const f2 (&kp)[KVAR ? CG_R : 1][2],
-                                         const f2 (&kh)[2][2], const float (&ke)[CG_R], const float* kz, f2 (&q)[CG_R][2]) {
+                                         const f2 (&kh)[2][2], const float (&ke)[CG_R], const float* kz, f2 (&q)[CG_R][2],
+                                        KahanF& dot) {
     constexpr unsigned FULL = 0xffffffffu;
     const int ny = c.n[1], nz = c.n[2];
     float xm[CG_R], xp[CG_R], kxm[CG_R], kxp[CG_R];
@@ -651,7 +654,6 @@ __device__ __forceinline__ float cg_rows(const CgCoef& c, const CgPlace& t, int 
 #pragma unroll
             for (int i = 0; i < 2; ++i) gp[j][i] = pair_face(kc[j][i], kp[j][i], tz);
     }
-    float s = 0.0f;
     if (t.inner_y && (c.periodic[2] || (z > 0 && z < nz - 1))) {
         f2 gy[2][2];
         const f2 ty = f2_make(c.tcd[1], c.tcd[1]);
@@ -659,7 +661,6 @@ __device__ __forceinline__ float cg_rows(const CgCoef& c, const CgPlace& t, int 
 #pragma unroll
             for (int i = 0; i < 2; ++i) gy[0][i] = pair_face(kh[0][i], kc[0][i], ty);
         }
-        f2 d = f2_make(0.0f, 0.0f);
 #pragma unroll
         for (int j = 0; j < CG_R; ++j) {
             const int jk = KVAR ? j : 0;
@@ -685,10 +686,9 @@ __device__ __forceinline__ float cg_rows(const CgCoef& c, const CgPlace& t, int 
                 q[j][0] = f2_make(v[0], v[1]);
                 q[j][1] = f2_make(v[2], v[3]);
             }
-            d = f2_fma(pc[j][0], q[j][0], d);
-            d = f2_fma(pc[j][1], q[j][1], d);
+            const f2 d = f2_fma(pc[j][1], q[j][1], f2_mul(pc[j][0], q[j][0]));
+            dot.add(t.in ? __fadd_rn(f2_lo(d), f2_hi(d)) : 0.0f);
         }
-        s = t.in ? __fadd_rn(f2_lo(d), f2_hi(d)) : 0.0f;
     } else {
 #pragma unroll
         for (int j = 0; j < CG_R; ++j) {
@@ -709,7 +709,7 @@ __device__ __forceinline__ float cg_rows(const CgCoef& c, const CgPlace& t, int 
             }
             const float sj = cg_q4<KVAR, true>(c, edge, t.gx, y, z, pcv, pmv, ppv, ymv, ypv, xm[j], xp[j], kcv, kmv, kpv, kymv,
                                                kypv, kxm[j], kxp[j], qv);
-            if (t.in && y < ny) s = __fadd_rn(s, sj);
+            dot.add(t.in && y < ny ? sj : 0.0f);
             q[j][0] = f2_make(qv[0], qv[1]);
             q[j][1] = f2_make(qv[2], qv[3]);
         }
@@ -719,7 +719,6 @@ __device__ __forceinline__ float cg_rows(const CgCoef& c, const CgPlace& t, int 
 #pragma unroll
         for (int i = 0; i < 2; ++i)
             if (KVAR) zf[j][i] = gp[j][i];
-    return s;
 }
 
 // Where a thread's cells lie: byte offset from the start of the padded arrays
@@ -872,7 +871,7 @@ __global__ void __launch_bounds__(32 * CG_W, 16 / CG_W) cg_dir(const __grid_cons
             pnew_pairs(rh[0], oh[0], beta, h[0]);
             pnew_pairs(rh[1], oh[1], beta, h[1]);
             f2 q[CG_R][2];
-            dot.add(cg_rows<KVAR>(c, t, z, pc, pm, pp, h, e, kc, zf, kp, kh, ke, KVAR ? cg_f(kB, o - dz) : nullptr, q));
+            cg_rows<KVAR>(c, t, z, pc, pm, pp, h, e, kc, zf, kp, kh, ke, KVAR ? cg_f(kB, o - dz) : nullptr, q, dot);
 #pragma unroll
             for (int j = 0; j < CG_R; ++j) {
                 if (twins) {
@@ -1220,12 +1219,13 @@ __global__ void __launch_bounds__(32 * CG_W, 24 / CG_W) cg_res_u(const __grid_co
                     prefetch_l2(rB + (o + 2 * dz + j * dy));
                 }
             }
-            cg_rows<false>(c, t, z, pc, pm, pp, h, e, kd, zf, kd, kh, ke, nullptr, q);
-            float s = 0.0f;
+            KahanF pq;   // not used here
+            cg_rows<false>(c, t, z, pc, pm, pp, h, e, kd, zf, kd, kh, ke, nullptr, q, pq);
 #pragma unroll
             for (int j = 0; j < CG_R; ++j) {
                 r[j][0] = f2_fma(nal, q[j][0], r[j][0]);
                 r[j][1] = f2_fma(nal, q[j][1], r[j][1]);
+                float s = 0.0f;   // 4 products a compensated addition, as in cg_rows
                 if (j == 0 ? t.in : row1) {
                     float v[4];
                     unp(r[j], v);
@@ -1235,6 +1235,7 @@ __global__ void __launch_bounds__(32 * CG_W, 24 / CG_W) cg_res_u(const __grid_co
                         s = __fmaf_rn(u, u, s);
                     }
                 }
+                rr.add(s);
                 if (twins) cg_put_twins(a.r, z, c, t, j, r[j]);
                 else cg_put(rB, o + j * dy, c, t, j, r[j]);
 #pragma unroll
@@ -1243,7 +1244,6 @@ __global__ void __launch_bounds__(32 * CG_W, 24 / CG_W) cg_res_u(const __grid_co
                     pc[j][i] = pp[j][i];
                 }
             }
-            rr.add(s);
         }
     }
     const double bsum = block_sum(rr.value(), red);

@@ -39,3 +39,19 @@ def test_overlapped_kernels_read_by_coherent_loads():
     assert not re.search(r"\b(in|rk)\[", cell)
     prepare = re.search(r"int prepare_k_halo\((.*?)\n\}\n", headers["wfa_grid.cu"], re.S).group(1)
     assert prepare.index("recip_kernel") < prepare.index("k_fresh = true")
+
+
+def _depths(body, call):
+    """Brace depth, from the start of a function's text, of each place of `call`."""
+    return [body[:m.start()].count("{") - body[:m.start()].count("}") for m in re.finditer(re.escape(call), body)]
+
+
+def test_cg_inner_products_add_four_products_at_a_time():
+    """The inner products of CG sum 4 fp32 products (a row's cells of a thread)
+    between compensated additions: those additions stand in the loop over a
+    thread's rows (function, if, loop), not behind it."""
+    text = _read("wfa_implicit.cu")
+    rows = re.search(r"void cg_rows\(.*?\) \{(.*?)\n\}\n", text, re.S).group(1)
+    assert len(_depths(rows, "dot.add(")) == 2 and min(_depths(rows, "dot.add(")) >= 2
+    res = re.search(r"cg_res_u\(const __grid_constant__ CgArgs a\) \{(.*?)\n\}\n", text, re.S).group(1)
+    assert _depths(res, "rr.add(") == [3]   # rows present, planes, rows
