@@ -803,7 +803,7 @@ __global__ void __launch_bounds__(RED_THREADS) rate32_partial_kernel(const float
                     if (!wx1 || x + i > nx) kc[i] = kc[0];
                 }
             if (first) kl = kc[0];
-            if (last == 3) kr = kc[3];
+            if (last == 3 || x + 4 > nx) kr = kc[3];   // (beyond a ragged end: the halo's too)
             if (!in_yz) {   // beyond a face: not looked at either
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
