@@ -254,35 +254,77 @@ bool pair_applies(const wfa_grid_s* g) {
     return true;
 }
 
+// Two steps a pass with per-cell k are cheaper than two one-step passes. Both
+// sides as estimates in us on one GB300, from 356 grids, most of them drawn at
+// random (0.9 to 40 M cells, all faces, both storage types): against one step a
+// pass the worst choice lost 8%, against the better one 30%, nearly all nothing.
+//   two steps: the planes its resident blocks step (pair_k_chunk's cost: tiles
+//     that n_x or n_y fill badly, and few planes a chunk, count in full), 1 us
+//     each; 1.2 on ragged rows, 1.7 where those store periodic copies, 1.12 with
+//     advection;
+//   one step: 2 us and 1.4 us a round of the resident 64 x 16 column blocks (rows
+//     in pairs: a warp's), a fifth more where it stores periodic copies;
+//     on short rows across a periodic x face far more (8x160x3437 76 / 27,
+//     25x160x1100 46 / 29, 33x160x833 28 / 22): two steps.
+// Two / one, us a step: 512^3 213 / 267, 333x250x187 33 / 42, 100^3 4.0 / 5.2;
+// where n_x or n_y leave the tiles half empty 250x97x41 5.2 / 4.4,
+// 130x397x775 125 / 107, 1000x1000x2 8.4 / 6.1, 2000x2x1000 32 / 26;
+// periodic 512^3 232 / 285, 250x397x403 129 / 99, 57x160x482 25 / 18.
+static bool pair_k_pays(const wfa_grid_s* g, bool perx, bool per) {
+    SweepCoef c = {};
+    for (int a = 0; a < 3; ++a) {
+        c.n[a] = g->n[a];
+        c.periodic[a] = g->bc_kind[2 * a] == WFA_BC_PERIODIC;
+    }
+    const PairTiles tl = pair_k_tiles(c);
+    double two = 0.0;
+    pair_k_chunk(c.n[2], (long long)tl.gx * tl.gy, (long long)num_sms() * PairKCfg::BLOCKS, &two);
+    if (c.n[0] % 4) two *= perx ? 1.7 : 1.2;
+    if (g->u[0] != 0.0 || g->u[1] != 0.0 || g->u[2] != 0.0) two *= 1.12;
+    if (perx && c.n[0] <= 33) return true;
+    const double blocks = (double)((c.n[0] + 63) / 64) * ((c.n[1] + 1) / 2) / 8.0 * c.n[2];
+    const double one = (2.0 + 1.4 * blocks / (num_sms() * 4.0)) * (per ? 1.2 : 1.0);
+    return two + 0.6 < 2.0 * one;
+}
+
 // The configuration of a grid that was not tuned, from its sizes and faces:
 // two steps a pass where that was faster. us a step on one GB300, two steps
 // against the one-step column march (fp32; bf16 is within 15%):
 //   uniform k, no periodic axis: 80^3 3.8 / 5.2, 128^3 6.4 / 8.1, 40x300x500
 //     18.4 / 30.8, 512^3 118 / 212; rows of 31 cells 9.5 / 9.1 (a warp's 120
-//     cells are mostly empty); up to 64^3 the launches dominate and boundary
+//     cells are mostly empty); rows just above 120 cells 121x397x1040 94 / 117,
+//     but 47x271x486 26.9 / 24.9; up to 64^3 the launches dominate and boundary
 //     cells in the pass are fastest (64^3 2.9, two steps 3.5, column march
 //     with its boundary launch 4.7);
-//   uniform k, periodic axes: wrapped reads are slower, and a column march
-//     without faces is one launch: 128^3 7.8 / 5.3 to 7.4, 160^3 9.6 / 9.3 to
-//     10.9, 640x500x333 96 / 144, 1024x1024x512 401 / 728; ragged periodic
-//     rows store copies cell by cell: 90x90x400 14.6 / 12.3, 333x250x187 39 / 37;
-//   per-cell k, no periodic axis: 80^3 3.8 / 3.3, 100^3 4.0 / 5.2, 128^3 4.9 /
-//     6.2, 31x200x160 4.6 / 6.4, 333x250x187 33 / 42, 512^3 213 / 267;
-//   per-cell k, periodic axes: 128^3 8.4 / 6.7, 160^3 11.2 / 13.2, 333x250x187
-//     42 / 48, 512^3 232 / 285.
+//   uniform k, periodic axes: wrapped reads are slower, and where every face is
+//     periodic a column march is one launch: 160x160x165 9.6 / 9.3 to 10.9,
+//     224x251x111 10.0 / 11.7, 244x283x257 28 / 36, 1024x1024x512 401 / 728; with
+//     tiles that are emptier than the column march's 256x147x149 12.0 / 10.0,
+//     176x81x433 15.5 / 11.6 (from 8 M cells on two steps win all the same);
+//     2048x2x2048 53 / 45; ragged periodic rows store copies cell by cell:
+//     481x397x261 99 / 80, 723x160x38 14.3 / 12.3, 282x512x287 79 / 75;
+//   per-cell k: pair_k_pays; below 0.9 M cells (4.2 M with a periodic axis)
+//     there is little in it: 80^3 3.8 / 3.3, 128^3 periodic 8.4 / 6.7.
 static Choice default_choice(const wfa_grid_s* g) {
     const long long cells = (long long)g->n[0] * g->n[1] * g->n[2];
     const bool perx = g->bc_kind[0] == WFA_BC_PERIODIC;
-    const bool per = perx || g->bc_kind[2] == WFA_BC_PERIODIC || g->bc_kind[4] == WFA_BC_PERIODIC;
+    const bool pery = g->bc_kind[2] == WFA_BC_PERIODIC, perz = g->bc_kind[4] == WFA_BC_PERIODIC;
+    const bool per = perx || pery || perz, ragged = g->n[0] % 4 != 0;
     const Choice one{COL_VARIANT, 1}, two{PAIR_VARIANT, 2};
     if (!pair_applies(g)) return one;
+    if (g->k) return cells >= (per ? 1LL << 22 : 900000LL) && pair_k_pays(g, perx, per) ? two : one;
+    // how full the rows make the two-step pass's tiles (120 cells a warp), against the column march's (64)
+    const int tx = (g->n[0] + 119) / 120 * 128, cx = (g->n[0] + 63) / 64 * 64;
     if (per) {
-        const bool wide = g->k || g->n[0] >= (perx && g->n[0] % 4 ? 480 : 100);
-        return wide && cells >= (1LL << 22) ? two : one;
+        if (g->n[0] < 100 || cells < (1LL << 22) || (perx && ragged)) return one;
+        const bool all = perx && pery && perz;
+        if (all && std::min(g->n[1], g->n[2]) < 16) return one;
+        if (cells < (1LL << 23) && (double)cx / tx < (all ? 0.78 : 0.6)) return one;
+        return two;
     }
-    if (g->k) return cells >= 900000 ? two : one;
     if (cells <= 300000) return Choice{INPLACE_VARIANT, 1};
-    return g->n[0] >= 40 ? two : one;
+    if (g->n[0] < 40 || (ragged && cells < (1LL << 23) && 2 * g->n[0] < tx)) return one;
+    return two;
 }
 
 static bool two_step_variant(int variant) { return variant == FUSED_VARIANT || variant == PAIR_VARIANT; }

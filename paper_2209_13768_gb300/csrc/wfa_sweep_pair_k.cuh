@@ -381,7 +381,9 @@ cudaError_t pair_k_dispatch(const SweepArgs& a, const PairTiles& tl, dim3 grid, 
 // z chunks of a launch of `tiles` blocks a chunk: whole waves of resident
 // blocks against the planes a chunk steps but does not store. At most 1024
 // chunks (three waves of the smallest tile count; the loop runs at every launch).
-inline int pair_k_chunk(int nz, long long tiles, long long resident) {
+// cost_out: the planes a resident block steps, about a microsecond each on one
+// GB300 (see default_choice).
+inline int pair_k_chunk(int nz, long long tiles, long long resident, double* cost_out = nullptr) {
     int best = nz;
     double cost = 1e300;
     for (int n = 1; n <= std::min((nz + 3) / 4, 1024); ++n) {
@@ -392,6 +394,7 @@ inline int pair_k_chunk(int nz, long long tiles, long long resident) {
             best = zc;
         }
     }
+    if (cost_out) *cost_out = cost;
     return best;
 }
 
