@@ -603,7 +603,7 @@ int batch_launch(wfa_grid* gs, const long long* steps, int count, int slot, bool
     for (int i : order) {
         wfa_grid g = gs[i];
         const bool pairs = mode != 0 && g->r && g->thin[g->cur] == TWINS_ONE;   // the two-step pass reads 4 columns
-        if (g->halo_dirty || g->thin[g->cur] >= TWINS_NONE || pairs) {
+        if (g->halo_dirty || !(g->thin[g->cur] & HAS_LAYER) || pairs) {
             int rc = refresh_halo(g, g->cur);
             if (rc) return rc;
             rc = prepare_coeff_halo(g);

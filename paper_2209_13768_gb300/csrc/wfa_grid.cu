@@ -418,6 +418,32 @@ int refresh_halo(wfa_grid_s* g, int buf) {
     return WFA_OK;
 }
 
+// The periodic copies that one-step passes read and two-step passes leave
+// stale: one layer beyond each periodic face, without corners, and 4 columns
+// beyond the row ends (rows that are no whole number of 4-cell groups: see
+// sweep_pair). blockIdx.y is the axis. Bound by its launch and a few scattered
+// sectors a row.
+template <typename S>
+__global__ void __launch_bounds__(256) copies_kernel(S* origin, const __grid_constant__ HaloSpec h) {
+    if (h.periodic[blockIdx.y])
+        copy_layers<S>(origin, h.n, h.px, h.px * h.py, blockIdx.y, blockIdx.x * 256 + threadIdx.x, gridDim.x * 256);
+}
+
+int refresh_copies(wfa_grid_s* g, int buf) {
+    const HaloSpec h = halo_spec(g);
+    const long long face = std::max(std::max((long long)COPY_COLS * h.n[1] * h.n[2], (long long)h.n[0] * h.n[2]),
+                                    (long long)h.n[0] * h.n[1]);
+    const dim3 grid(grid_blocks(2 * face, 256), 3);
+    const long long off = domain_offset(g);
+    if (g->storage == WFA_BF16)
+        copies_kernel<__nv_bfloat16><<<grid, 256, 0, g->stream>>>((__nv_bfloat16*)g->T[buf] + off, h);
+    else
+        copies_kernel<float><<<grid, 256, 0, g->stream>>>((float*)g->T[buf] + off, h);
+    WFA_CUDA(cudaGetLastError());
+    g->thin[buf] = TWINS_ONE_X;
+    return WFA_OK;
+}
+
 // --------------------------------------------------------------- reductions --
 constexpr int HEAT_BLOCKS = 152 * 8;   // resident blocks
 // the stability passes are latency-bound (divisions, seven k reads a cell):
@@ -1063,6 +1089,7 @@ int wfa_create_grid(int nx, int ny, int nz, double hx, double hy, double hz, int
     g->py = ny + 2LL * HALO;
     g->pz = nz + 2LL * HALO;
     for (int f = 0; f < 6; ++f) { g->bc_kind[f] = WFA_BC_ZEROFLUX; g->bc_value[f] = 0.0; }
+    g->thin[0] = g->thin[1] = TWINS_FULL;
     const size_t bytes = field_elems(g) * g->esize;
     cudaError_t e = cudaSuccess;
     g->own_T = true;

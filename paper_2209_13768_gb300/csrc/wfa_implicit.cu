@@ -1727,7 +1727,7 @@ int wfa_implicit_step(wfa_grid g, double dt, long long n, double rtol, int max_i
     if (iters) *iters = 0;
     if (rel_res) *rel_res = 0.0;
     if (n == 0) return WFA_OK;
-    if (g->halo_dirty || g->thin[g->cur] >= TWINS_NONE) {   // held layers carry their value before the first solve
+    if (g->halo_dirty || !(g->thin[g->cur] & HAS_LAYER)) {   // held layers carry their value before the first solve
         int rc = refresh_halo(g, g->cur);
         if (rc) return rc;
         g->halo_dirty = false;

@@ -40,7 +40,12 @@ constexpr int INPLACE_VARIANT = 5;    // the one-step column-march kernel, bound
 constexpr int WIDE_VARIANT = 6;       // the one-step column-march kernel, 8 cells a thread (16 for bf16, uniform k)
 constexpr int PAIR_VARIANT = 7;       // two steps per pass in registers (uniform k)
 
-enum { TWINS_FULL = 0, TWINS_ONE = 1, TWINS_NONE = 2, TWINS_X = 3 };
+// Which periodic copies a field buffer holds (wfa_grid_s::thin): layers beyond
+// each face (a bit each for one layer, every layer with the corners, and 4
+// columns beyond the row ends). A thin column pass leaves one layer, the
+// two-step pass none (it wraps its reads) or, on ragged rows, the columns.
+enum { TWINS_NONE = 0, HAS_LAYER = 1, HAS_COLS = 2, HAS_ALL = 4 };
+enum { TWINS_FULL = HAS_LAYER | HAS_COLS | HAS_ALL, TWINS_ONE = HAS_LAYER, TWINS_X = HAS_COLS, TWINS_ONE_X = HAS_LAYER | HAS_COLS };
 
 // NVTX range over one API call: a named span on a profiler's timeline
 // (nothing happens unless a tool is attached).
@@ -190,10 +195,7 @@ struct wfa_grid_s {
     void* cg;             // wfa::CgWork (work vectors and graph of the implicit solver)
     int cg_method;        // WFA_CG_CLASSIC / WFA_CG_PIPELINED (wfa_set_cg_method)
     cudaEvent_t xev;      // orders plane exchanges against this grid's stream (wfa_exchange)
-    unsigned char thin[2];   // periodic copies each buffer holds: TWINS_FULL every layer, TWINS_ONE
-                             // one layer without corners (a thin column pass wrote it: enough for
-                             // one-step kernels), TWINS_NONE stale (the two-step pass wraps its reads),
-                             // TWINS_X 4 columns beyond the row ends only (the two-step pass, ragged rows)
+    unsigned char thin[2];   // periodic copies each buffer holds (TWINS_*)
 };
 
 namespace wfa {
@@ -210,7 +212,8 @@ inline bool has_exchange_face(const wfa_grid_s* g) {
 }
 
 int build_coef(const wfa_grid_s* g, SweepCoef* c);       // host: fp64 -> fp32 coefficients
-int refresh_halo(wfa_grid_s* g, int buf);                 // twins + held layers of one buffer
+int refresh_halo(wfa_grid_s* g, int buf);                 // twins + ghost and held layers of both buffers
+int refresh_copies(wfa_grid_s* g, int buf);               // one layer of twins of one buffer (and 4 columns)
 int launch_sweep(wfa_grid_s* g, long long nsteps);        // advance nsteps on g->stream
 bool pair_applies(const wfa_grid_s* g);                   // the two-step passes take this grid
 int check_status(wfa_grid_s* g);                          // sync + report a device-side timeout
@@ -319,6 +322,35 @@ __device__ __forceinline__ void twin_range(int x, int n, bool periodic, int* fir
     } else {
         *first = x;
         *count = 1;
+    }
+}
+
+// The first layer beyond both faces of periodic axis a (the first and last
+// COPY_COLS columns for x), for the rows of the domain: thread t of `stride`.
+constexpr int COPY_COLS = 4;
+template <typename S>
+__device__ __forceinline__ void copy_layers(S* origin, const int (&nn)[3], long long sy, long long sz, int a, unsigned t,
+                                            unsigned stride) {
+    const unsigned nx = nn[0], ny = nn[1], nz = nn[2], n = nn[a];
+    const unsigned layers = a == 0 ? min((unsigned)COPY_COLS, nx) : 1u;
+    const long long st = a == 0 ? 1 : a == 1 ? sy : sz;
+    const unsigned total = a == 0 ? 2 * layers * ny * nz : 2 * nx * (a == 1 ? nz : ny);
+    for (; t < total; t += stride) {
+        unsigned p[3], k;   // the cell copied, and which of its line's copies
+        if (a == 0) {
+            const unsigned r = t / (2 * layers);
+            k = t - r * 2 * layers;
+            p[1] = r % ny;
+            p[2] = r / ny;
+        } else {
+            const unsigned r = t / nx;
+            p[0] = t - r * nx;
+            k = r & 1;
+            p[1] = p[2] = r >> 1;
+        }
+        p[a] = k < layers ? k : n - 1 - (k - layers);   // the first layers, then the last ones
+        const long long o = p[0] + p[1] * sy + p[2] * sz;
+        origin[o + (k < layers ? (long long)n : -(long long)n) * st] = origin[o];
     }
 }
 

@@ -421,9 +421,17 @@ static bool pair_reads_copies(const wfa_grid_s* g) { return g->bc_kind[0] == WFA
 // kernels read every layer, the one-step kernels one.
 static bool lacks_twins(const wfa_grid_s* g, int buf, int depth, int variant) {
     const int have = g->thin[buf];
-    if (two_step_variant(variant) && depth == 2) return pair_reads_copies(g) && (have == TWINS_ONE || have == TWINS_NONE);
-    if (variant >= 1 && variant <= NUM_TILE_VARIANTS) return have != TWINS_FULL;
-    return have == TWINS_NONE || have == TWINS_X;
+    if (two_step_variant(variant) && depth == 2) return pair_reads_copies(g) && !(have & HAS_COLS);
+    return !(have & (variant >= 1 && variant <= NUM_TILE_VARIANTS ? HAS_ALL : HAS_LAYER));
+}
+// Completes them. Everything that leaves copies stale keeps the ghost layers,
+// so the tiled kernels alone need the whole halo again. An odd count after a
+// two-step pass pays this at every call (us, 3 steps, one step a pass / the
+// whole halo of both buffers / this): 256^3 torus
+// uniform k 108 / 172 / 95, channel per-cell k 137 / 196 / 136, 160x165x165 torus
+// per-cell k 50 / 84 / 48.
+static int complete_twins(wfa_grid_s* g, int variant) {
+    return variant >= 1 && variant <= NUM_TILE_VARIANTS ? refresh_halo(g, g->cur) : refresh_copies(g, g->cur);
 }
 // The periodic copies a pass leaves in the buffer it writes.
 static unsigned char twins_written(const wfa_grid_s* g, const SweepCoef& c, int depth, int variant) {
@@ -436,7 +444,7 @@ static unsigned char twins_written(const wfa_grid_s* g, const SweepCoef& c, int 
 // (zc: planes per z chunk of the column kernels, 0 = automatic).
 static int one_pass(wfa_grid_s* g, const SweepCoef& c, int depth, int variant, int zc = 0) {
     if (lacks_twins(g, g->cur, depth, variant)) {   // complete the copies first
-        const int rc = refresh_halo(g, g->cur);
+        const int rc = complete_twins(g, variant);
         if (rc) return rc;
     }
     g->thin[1 - g->cur] = twins_written(g, c, depth, variant);
@@ -591,16 +599,21 @@ int launch_sweep(wfa_grid_s* g, long long nsteps) {
     const long long cells = (long long)g->n[0] * g->n[1] * g->n[2];
     if (two_step_variant(ch.variant) && ch.depth == 2 && nsteps % 2) {
         // an odd count: its single step first, while the periodic copies it
-        // reads are current (the two-step passes leave them stale)
-        rc = one_pass(g, c, 1, ch.variant, ch.zc);
-        if (rc) return rc;
-        --nsteps;
+        // reads are current (the two-step passes leave them stale). Three
+        // steps of a smaller periodic grid: single steps, so that the next call
+        // need not complete them (203x160x150 channel per-cell k 56 us for 60)
+        const bool keep = nsteps == 3 && cells < (1LL << 23) && (c.periodic[0] || c.periodic[1] || c.periodic[2]);
+        do {
+            rc = one_pass(g, c, 1, ch.variant, ch.zc);
+            if (rc) return rc;
+            --nsteps;
+        } while (keep && nsteps > 0);
     }
     const long long runs = nsteps / ((long long)ch.depth * GRAPH_PASSES);
     if (cells <= GRAPH_MAX_CELLS && runs >= 2) {
         cudaGraphExec_t exec = nullptr;
         if (lacks_twins(g, g->cur, ch.depth, ch.variant)) {   // not inside the graph
-            rc = refresh_halo(g, g->cur);
+            rc = complete_twins(g, ch.variant);
             if (rc) return rc;
         }
         const int every = g->timing_every;
