@@ -89,13 +89,14 @@ struct MgGrid {
     PairTiles pt;
     int pzchunk, npblocks, pblock0;
     int odd;
+    int copies;           // its input's periodic copies are stale: completed before the first round
     long long steps;
 };
 
 // One step of unit u of a grid: thread t takes pair u * 256 + t, pairs
 // numbered chunk-major over (z chunk, column). COH: the field was written by
 // other blocks of the same launch (persistent kernel), so it is read through
-// L2 (ld.cg) instead of the read-only path.
+// L2 (ld.cg) instead of L1.
 template <typename S, bool KVAR, bool ADV, bool GHOST, bool COH>
 __device__ __forceinline__ void mg_unit(const MgGrid& sg, int u, long long step, int* status) {
     const int p = u * MG_THREADS + (int)threadIdx.x;
@@ -199,6 +200,20 @@ __global__ void __launch_bounds__(PAIR_THREADS, PairKCfg::BLOCKS)
     const int z0 = bz * sg.pzchunk, b = (pass + sg.odd) & 1;
     pair_k_run<S, PER, true, ADV, PairKCfg::R, PairKCfg::W>(sg.c, sg.tb[b], const_cast<void*>(sg.tb[b ^ 1]), sg.rk, sg.pt, bx,
                                                             by, z0, min(z0 + sg.pzchunk, sg.c.n[2]), sm);
+}
+
+// The periodic copies of the grids that need them (refresh_copies for a batch:
+// one launch for all of them; a launch a grid cost 64 small periodic grids 190
+// us a call). COPY_BLOCKS blocks a grid; blockIdx.y is the axis.
+constexpr int COPY_BLOCKS = 16;
+__global__ void __launch_bounds__(256) mg_copies(const MgGrid* __restrict__ grids) {
+    const MgGrid& g = grids[blockIdx.x / COPY_BLOCKS];
+    const int a = blockIdx.y;
+    if (!g.copies || !g.c.periodic[a]) return;
+    const unsigned t = blockIdx.x % COPY_BLOCKS * 256 + threadIdx.x;
+    void* const p = const_cast<void*>(g.tb[0]);
+    if (g.cls < NKIND) copy_layers<float>((float*)p, g.c.n, g.c.sy, g.c.sz, a, t, COPY_BLOCKS * 256);
+    else copy_layers<__nv_bfloat16>((__nv_bfloat16*)p, g.c.n, g.c.sy, g.c.sz, a, t, COPY_BLOCKS * 256);
 }
 
 template <typename S>
@@ -602,8 +617,7 @@ int batch_launch(wfa_grid* gs, const long long* steps, int count, int slot, bool
     // halos, held layers and 1/k of grids changed since their last step
     for (int i : order) {
         wfa_grid g = gs[i];
-        const bool pairs = mode != 0 && g->r && g->thin[g->cur] == TWINS_ONE;   // the two-step pass reads 4 columns
-        if (g->halo_dirty || !(g->thin[g->cur] & HAS_LAYER) || pairs) {
+        if (g->halo_dirty) {
             int rc = refresh_halo(g, g->cur);
             if (rc) return rc;
             rc = prepare_coeff_halo(g);
@@ -654,6 +668,23 @@ int batch_launch(wfa_grid* gs, const long long* steps, int count, int slot, bool
         b.nblocks = (int)((pairs + MG_THREADS - 1) / MG_THREADS);
         b.steps = steps[order[k]];
         b.pt = pair_k_tiles(b.c);
+    }
+    // the periodic copies that the last pass left stale and this call reads:
+    // one layer by single steps, 4 columns by two-step passes across a
+    // periodic x face (they wrap the other reads)
+    bool copies = false;
+    for (int k = 0; k < ng; ++k) {
+        wfa_grid g = gs[order[k]];
+        const bool two = mode != 0 && pair_kind(cls[k] % NKIND), single = !two || mg[k].steps % 2;
+        const int have = g->thin[g->cur];
+        if (!((single && !(have & HAS_LAYER)) || (two && mg[k].c.periodic[0] && !(have & HAS_COLS)))) continue;
+        if (mode == 0) {
+            const int rc = refresh_copies(g, g->cur);
+            if (rc) return rc;
+        } else {
+            mg[k].copies = 1;
+            copies = true;
+        }
     }
     BatchCtx* c = context_for(st, slot);
     int rc = batch_wait(st, slot);   // a launch of this slot still in flight
@@ -854,8 +885,12 @@ int batch_launch(wfa_grid* gs, const long long* steps, int count, int slot, bool
             WFA_CUDA(cudaStreamBeginCapture(ls, cudaStreamCaptureModeThreadLocal));
         }
         cudaError_t e = cudaMemcpyAsync(c->dev, c->host, bytes, cudaMemcpyHostToDevice, ls);
-        if (mode == 1 && e == cudaSuccess) e = cudaEventRecord(c->fork, ls);
         const MgGrid* dgrids = reinterpret_cast<const MgGrid*>(c->dev);
+        if (copies && e == cudaSuccess) {
+            mg_copies<<<dim3(ng * COPY_BLOCKS, 3), 256, 0, ls>>>(dgrids);
+            e = cudaGetLastError();
+        }
+        if (mode == 1 && e == cudaSuccess) e = cudaEventRecord(c->fork, ls);
         const int* dmap = reinterpret_cast<const int*>(c->dev + grid_bytes);
         int* status = gs[order[0]]->d_status;
         // per branch, the grids with more than s steps are a prefix
@@ -929,6 +964,7 @@ int batch_launch(wfa_grid* gs, const long long* steps, int count, int slot, bool
     for (int k = 0; k < ng; ++k) {
         wfa_grid g = gs[order[k]];
         const bool per = mg[k].c.periodic[0] || mg[k].c.periodic[1] || mg[k].c.periodic[2];
+        if (mg[k].copies) g->thin[g->cur] = TWINS_ONE_X;
         if (mode != 0 && pair_kind(cls[k] % NKIND)) {   // two steps a pass, an odd count's single step first
             const long long odd = mg[k].steps & 1, pairs = mg[k].steps / 2;
             g->cur = (int)((g->cur + odd + pairs) & 1);

@@ -34,3 +34,25 @@ def test_odd_counts_after_two_step_passes(shape, faces, kvar, storage):
             g.step(n)
             done += n
             np.testing.assert_array_equal(g.read_field(), run_gpu(p, steps=done, storage=storage, variant=-1), err_msg=f"after {done}")
+
+
+@pytest.mark.parametrize("mode", ["rounds", "stream", "persistent"])
+def test_odd_counts_in_batches(mode, monkeypatch):
+    monkeypatch.setenv("WFA_BATCH_MODE", mode)
+    cases = [(shape, faces, kvar, storage) for shape in SHAPES for faces in FACES for kvar in (False, True)
+             for storage in (wfa.F32, wfa.BF16)]
+    probs = [_problem(shape, faces, kvar, i) for i, (shape, faces, kvar, _) in enumerate(cases)]
+    grids = [make_grid(p, storage=c[3]) for p, c in zip(probs, cases)]
+    done = np.zeros(len(grids), int)
+    for r in range(5):
+        steps = [(3 * i + 5 * r + i // 7) % 6 for i in range(len(grids))]
+        wfa.batch_run(grids, steps)
+        done += steps
+        if r in (1, 3):   # a two-step pass of its own in between
+            for g in grids:
+                g.set_tuning(2, 7)
+                g.step(2)
+            done += 2
+    for p, c, g, n in zip(probs, cases, grids, done):
+        np.testing.assert_array_equal(g.read_field(), run_gpu(p, steps=int(n), storage=c[3], variant=-1), err_msg=str(c))
+        g.close()
