@@ -14,7 +14,8 @@
 // type x conductivity mode x advection x ghost-layer faces) over the active
 // units, one block per unit. Classes whose ghost layers hold every face
 // (per-cell k) take two steps a round with the single grid's two-step pass
-// (sweep_pair_k; an odd count takes its single step first): 256 grids of 16 to
+// where that is cheaper (two_step_classes; sweep_pair_k; an odd count takes its
+// single step first): 256 grids of 16 to
 // 128 cells an edge 302 -> 370 GLUPS, 14 grids of 0.1 to 2.7 M cells 345 ->
 // 375, one of 1.9 M cells 132 -> 216. (Uniform k keeps one step a round: the
 // two-step pass there, whose warps recompute their ring rows, ran 191 against
@@ -55,10 +56,11 @@ namespace {
 
 constexpr int MG_THREADS = 256;
 // {f32, bf16} x {uniform k, per-cell k, per-cell k with advection, the last
-// two with every boundary face in the ghost layers, and those with a periodic
-// axis (per-round launches only: the two-step pass wraps its reads there)}
-constexpr int NKIND = 7;
-constexpr int KIND_PAIR = 3;
+// two with every boundary face in the ghost layers; per-round launches only:
+// those two taking two steps a launch, and the same with a periodic axis (the
+// two-step pass wraps its reads there)}
+constexpr int NKIND = 9;
+constexpr int KIND_GHOST = 3, KIND_PAIR = 5;
 constexpr bool pair_kind(int kind) { return kind >= KIND_PAIR; }   // per-round launches take two steps
 constexpr int PAIR_THREADS = 32 * PairKCfg::W;
 constexpr int NCLASS = 2 * NKIND;
@@ -219,9 +221,9 @@ __global__ void __launch_bounds__(256) mg_copies(const MgGrid* __restrict__ grid
 template <typename S>
 cudaError_t launch_pair(int kind, int blocks, const MgGrid* grids, const int* map, int pass, cudaStream_t st) {
     switch (kind) {
-        case 3: mg_pair_k<S, false, false><<<blocks, PAIR_THREADS, 0, st>>>(grids, map, pass); break;
-        case 4: mg_pair_k<S, false, true><<<blocks, PAIR_THREADS, 0, st>>>(grids, map, pass); break;
-        case 5: mg_pair_k<S, true, false><<<blocks, PAIR_THREADS, 0, st>>>(grids, map, pass); break;
+        case 5: mg_pair_k<S, false, false><<<blocks, PAIR_THREADS, 0, st>>>(grids, map, pass); break;
+        case 6: mg_pair_k<S, false, true><<<blocks, PAIR_THREADS, 0, st>>>(grids, map, pass); break;
+        case 7: mg_pair_k<S, true, false><<<blocks, PAIR_THREADS, 0, st>>>(grids, map, pass); break;
         default: mg_pair_k<S, true, true><<<blocks, PAIR_THREADS, 0, st>>>(grids, map, pass); break;
     }
     return cudaGetLastError();
@@ -235,7 +237,8 @@ cudaError_t launch_kind(int kind, int blocks, const MgGrid* grids, const int* bl
         case 1: mg_sweep<S, true, false, false><<<blocks, MG_THREADS, 0, st>>>(grids, block_grid, step, status); break;
         case 2: mg_sweep<S, true, true, false><<<blocks, MG_THREADS, 0, st>>>(grids, block_grid, step, status); break;
         case 3:
-        case 5: mg_sweep<S, true, false, true><<<blocks, MG_THREADS, 0, st>>>(grids, block_grid, step, status); break;
+        case 5:
+        case 7: mg_sweep<S, true, false, true><<<blocks, MG_THREADS, 0, st>>>(grids, block_grid, step, status); break;
         default: mg_sweep<S, true, true, true><<<blocks, MG_THREADS, 0, st>>>(grids, block_grid, step, status); break;
     }
     return cudaGetLastError();
@@ -540,6 +543,33 @@ int graph_for(BatchCtx* c, int cls) {
     return WFA_OK;
 }
 
+// Moves the grids whose ghost layers hold every face (kinds 3 and 4) to the
+// two-step classes where that is cheaper, per storage type. With a periodic axis
+// it always is: single steps store every copy cell by cell (100 steps of 64
+// small grids: 10.8 -> 3.4 ms). Without one the two-step pass pays for its
+// tiles' ring and empty cells, which many small or badly filling grids in a
+// saturated launch do not hide: estimates in us a step, from 44 batches of
+// equal grids drawn at random, the launch itself 5 us. Two steps / one, ms a
+// call of 20 steps: 7 grids of 102x164x47 0.40 / 0.47, 98 of 24x98x26 0.52 /
+// 0.73, one of 204x159x15 0.15 / 0.30, but 13 of 70x73x90 0.60 / 0.52, two of
+// 160^3 0.62 / 0.53, 123 of 8x190x32 1.24 / 1.08, 126 of 109x109x4 0.58 / 0.53.
+void two_step_classes(wfa_grid* gs, const std::vector<int>& order, const std::vector<MgGrid>& mg, std::vector<int>& cls) {
+    double two[2] = {2.5, 2.5}, one[2] = {5.0, 5.0};   // by storage type
+    std::vector<char> may(mg.size(), 0);
+    auto periodic = [](const MgGrid& m) { return m.c.periodic[0] || m.c.periodic[1] || m.c.periodic[2]; };
+    for (size_t k = 0; k < mg.size(); ++k) {
+        const MgGrid& m = mg[k];
+        may[k] = cls[k] % NKIND >= KIND_GHOST && pair_applies(gs[order[k]]);
+        if (!may[k] || periodic(m)) continue;
+        const int s = cls[k] / NKIND, nz = m.c.n[2];
+        two[s] += 1.55 * m.pt.gx * m.pt.gy * nz / 608.0 * (1.0 + 4.0 / std::min(nz, 32));
+        one[s] += (double)m.ncols * nz / (MG_THREADS * 608.0) * (1.4 + 27.0 / m.c.n[0]);
+    }
+    for (size_t k = 0; k < mg.size(); ++k)
+        if (may[k] && (periodic(mg[k]) || two[cls[k] / NKIND] < one[cls[k] / NKIND]))
+            cls[k] += periodic(mg[k]) ? KIND_PAIR + 2 - KIND_GHOST : KIND_PAIR - KIND_GHOST;
+}
+
 }  // namespace
 
 // Waits for the launch that batch_launch(..., slot, false) left running on
@@ -641,14 +671,8 @@ int batch_launch(wfa_grid* gs, const long long* steps, int count, int slot, bool
         b.rk = g->r ? g->r + off : nullptr;
         bool adv = false;
         for (int f = 0; f < 6; ++f) adv = adv || b.c.adv[f] != 0.0f;
-        int kind = g->r ? (adv ? 2 : 1) + (b.c.halo_bc ? 2 : 0) : 0;
-        if (mode == 0) {   // the persistent kernel's classes
-            cls[k] = (g->storage == WFA_BF16 ? PKIND : 0) + kind;
-        } else {
-            if (pair_kind(kind) && !pair_applies(g)) kind -= 2;
-            if (pair_kind(kind) && (b.c.periodic[0] || b.c.periodic[1] || b.c.periodic[2])) kind += 2;
-            cls[k] = (g->storage == WFA_BF16 ? NKIND : 0) + kind;
-        }
+        const int kind = g->r ? (adv ? 2 : 1) + (b.c.halo_bc ? 2 : 0) : 0;
+        cls[k] = (g->storage == WFA_BF16 ? (mode == 0 ? PKIND : NKIND) : 0) + kind;   // mode 0: the persistent kernel's
         b.ncx = (g->n[0] + 3) / 4;
         b.ncols = b.ncx * g->n[1];
         // z chunks of about 16 planes with per-cell k (boundary cells in the pass)
@@ -669,6 +693,7 @@ int batch_launch(wfa_grid* gs, const long long* steps, int count, int slot, bool
         b.steps = steps[order[k]];
         b.pt = pair_k_tiles(b.c);
     }
+    if (mode != 0) two_step_classes(gs, order, mg, cls);
     // the periodic copies that the last pass left stale and this call reads:
     // one layer by single steps, 4 columns by two-step passes across a
     // periodic x face (they wrap the other reads)
@@ -789,7 +814,7 @@ int batch_launch(wfa_grid* gs, const long long* steps, int count, int slot, bool
             // costs least, in waves of resident blocks (whole ones while there are
             // few) times the planes a block steps
             int zmax = 64;
-            if (pair_class(t) && cls_first[t] < cls_first[t + 1]) {
+            if (pair_class(t) && cls_first[t] < cls_first[t + 1] && mg[idx[cls_first[t]]].steps >= 2) {
                 const double resident = (double)sms * PairKCfg::BLOCKS;
                 double best = 1e300;
                 for (int z = 64; z >= 4; z = z > 16 ? z * 7 / 8 : z - 1) {
@@ -816,7 +841,7 @@ int batch_launch(wfa_grid* gs, const long long* steps, int count, int slot, bool
                     const int nz = m.c.n[2], nch = (nz + zmax - 1) / zmax;
                     m.odd = (int)(m.steps & 1);
                     m.pzchunk = (nz + nch - 1) / nch;
-                    m.npblocks = m.pt.gx * m.pt.gy * ((nz + m.pzchunk - 1) / m.pzchunk);
+                    m.npblocks = m.steps < 2 ? 0 : m.pt.gx * m.pt.gy * ((nz + m.pzchunk - 1) / m.pzchunk);
                     m.pblock0 = (int)bp;
                     bp += m.npblocks;
                     if (!m.odd) continue;   // no single step: no units
