@@ -172,7 +172,7 @@ struct wfa_grid_s {
     bool limit_valid;
     bool field_set, coeffs_set, dt_set, halo_dirty;
     bool k_halo_dirty;    // k twins / ghost layers and 1/k must be rebuilt before use
-    bool k_fresh;         // 1/k was rebuilt and no pass has been launched since
+    bool k_fresh;         // 1/k was rebuilt, or its planes handed out, and no pass has been launched since
     long long steps_done;
     int force_depth, force_variant;   // wfa_set_tuning (0 = automatic)
     int force_zchunk;                 // wfa_set_zchunk: planes per z chunk of the column kernels (0 = automatic)

@@ -74,6 +74,7 @@ static int planes(wfa_grid_s* g, int face, int what, void** send, void** recv, s
     if (send) *send = base + own * plane;
     if (recv) *recv = base + halo * plane;
     if (bytes) *bytes = plane;
+    if (what == WFA_PLANES_RECIP_K) g->k_fresh = true;   // the caller is about to write 1/k
     return WFA_OK;
 }
 

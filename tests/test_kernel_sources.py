@@ -39,6 +39,8 @@ def test_overlapped_kernels_read_by_coherent_loads():
     assert not re.search(r"\b(in|rk)\[", cell)
     prepare = re.search(r"int prepare_k_halo\((.*?)\n\}\n", headers["wfa_grid.cu"], re.S).group(1)
     assert prepare.index("recip_kernel") < prepare.index("k_fresh = true")
+    planes = re.search(r"static int planes\((.*?)\n\}\n", headers["wfa_slabs.cu"], re.S).group(1)
+    assert "if (what == WFA_PLANES_RECIP_K) g->k_fresh = true;" in planes   # its caller writes the halo plane of 1/k
 
 
 def _depths(body, call):
