@@ -547,23 +547,33 @@ int graph_for(BatchCtx* c, int cls) {
 // two-step classes where that is cheaper, per storage type. With a periodic axis
 // it always is: single steps store every copy cell by cell (100 steps of 64
 // small grids: 10.8 -> 3.4 ms). Without one the two-step pass pays for its
-// tiles' ring and empty cells, which many small or badly filling grids in a
-// saturated launch do not hide: estimates in us a step, from 44 batches of
-// equal grids drawn at random, the launch itself 5 us. Two steps / one, ms a
-// call of 20 steps: 7 grids of 102x164x47 0.40 / 0.47, 98 of 24x98x26 0.52 /
-// 0.73, one of 204x159x15 0.15 / 0.30, but 13 of 70x73x90 0.60 / 0.52, two of
-// 160^3 0.62 / 0.53, 123 of 8x190x32 1.24 / 1.08, 126 of 109x109x4 0.58 / 0.53.
+// tiles' ring and empty cells. Estimates in us a step (the last terms: the
+// launches), fitted to 44 batches of equal grids drawn at random and 7 others:
+//   two steps: the planes its blocks step; a fifth less from 64 grids on, whose
+//     two branches fill one another's gaps (rows of 8 cells do not gain from it);
+//   one step: 256 (4-cell column, plane) pairs a block, more on short rows.
+// Two steps / one, ms a call of 20 steps: 7 grids of 102x164x47 0.40 / 0.47, 98
+// of 24x98x26 0.52 / 0.73, one of 204x159x15 0.15 / 0.30, but 13 of 70x73x90 0.60
+// / 0.52, two of 160^3 0.62 / 0.53, 123 of 8x190x32 1.24 / 1.08; 256 grids of 16 to
+// 128 cells an edge, 50 to 500 steps, 32 / 39.
 void two_step_classes(wfa_grid* gs, const std::vector<int>& order, const std::vector<MgGrid>& mg, std::vector<int>& cls) {
-    double two[2] = {2.5, 2.5}, one[2] = {5.0, 5.0};   // by storage type
+    struct Cost { double two0, two, one0, one, row; };
+    const Cost cost[2] = {{3.4, 1.3, 7.2, 1.07, 25.0}, {3.6, 1.16, 8.0, 0.93, 33.0}};   // fp32, bf16
+    double two[2] = {cost[0].two0, cost[1].two0}, one[2] = {cost[0].one0, cost[1].one0};
+    int count[2] = {0, 0};
     std::vector<char> may(mg.size(), 0);
     auto periodic = [](const MgGrid& m) { return m.c.periodic[0] || m.c.periodic[1] || m.c.periodic[2]; };
     for (size_t k = 0; k < mg.size(); ++k) {
+        may[k] = mg[k].steps >= 2 && cls[k] % NKIND >= KIND_GHOST && pair_applies(gs[order[k]]);
+        if (may[k] && !periodic(mg[k])) ++count[cls[k] / NKIND];
+    }
+    for (size_t k = 0; k < mg.size(); ++k) {
         const MgGrid& m = mg[k];
-        may[k] = cls[k] % NKIND >= KIND_GHOST && pair_applies(gs[order[k]]);
         if (!may[k] || periodic(m)) continue;
-        const int s = cls[k] / NKIND, nz = m.c.n[2];
-        two[s] += 1.55 * m.pt.gx * m.pt.gy * nz / 608.0 * (1.0 + 4.0 / std::min(nz, 32));
-        one[s] += (double)m.ncols * nz / (MG_THREADS * 608.0) * (1.4 + 27.0 / m.c.n[0]);
+        const int s = cls[k] / NKIND, nx = m.c.n[0], nz = m.c.n[2];
+        two[s] += cost[s].two * (count[s] >= 64 && nx >= 16 ? 0.82 : 1.0) * m.pt.gx * m.pt.gy * nz / 608.0 *
+                  (1.0 + 4.0 / std::min(nz, 32));
+        one[s] += (double)m.ncols * nz / (MG_THREADS * 608.0) * (cost[s].one + cost[s].row / nx);
     }
     for (size_t k = 0; k < mg.size(); ++k)
         if (may[k] && (periodic(mg[k]) || two[cls[k] / NKIND] < one[cls[k] / NKIND]))

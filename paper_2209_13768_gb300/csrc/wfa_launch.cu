@@ -232,14 +232,16 @@ static void tune_save_locked() {
 // y extent whose tiles a launch can index (the column march's are taller).
 bool pair_applies(const wfa_grid_s* g) {
     if (g->n[0] < 8) return false;
-    SweepCoef c = {};
-    for (int a = 0; a < 3; ++a) {
-        c.n[a] = g->n[a];
-        c.periodic[a] = g->bc_kind[2 * a] == WFA_BC_PERIODIC;
+    if (g->n[1] > 65535) {
+        SweepCoef c = {};
+        for (int a = 0; a < 3; ++a) {
+            c.n[a] = g->n[a];
+            c.periodic[a] = g->bc_kind[2 * a] == WFA_BC_PERIODIC;
+        }
+        const int rows = g->storage == WFA_BF16 ? PairCfg<__nv_bfloat16>::R * PairCfg<__nv_bfloat16>::WPB
+                                                : PairCfg<float>::R * PairCfg<float>::WPB;
+        if ((g->k ? pair_k_tiles(c).gy : (g->n[1] + rows - 1) / rows) > 65535) return false;
     }
-    const int rows = g->storage == WFA_BF16 ? PairCfg<__nv_bfloat16>::R * PairCfg<__nv_bfloat16>::WPB
-                                            : PairCfg<float>::R * PairCfg<float>::WPB;
-    if ((g->k ? pair_k_tiles(c).gy : (g->n[1] + rows - 1) / rows) > 65535) return false;
     const bool adv = g->u[0] != 0.0 || g->u[1] != 0.0 || g->u[2] != 0.0;
     for (int f = 0; f < 6; ++f) {
         if (g->bc_kind[f] == WFA_BC_DIRICHLET_CELL || g->bc_kind[f] == WFA_BC_EXCHANGE) return false;
