@@ -1775,13 +1775,31 @@ int wfa_implicit_step(wfa_grid g, double dt, long long n, double rtol, int max_i
         w->spmv_grid[0] = gxb;
         w->spmv_grid[1] = gyb;
         w->spmv_grid[2] = (int)nch;
-        // cg_dir / cg_res_u: CG_W warps of 16 (narrow grids: 8) x lanes, CG_R rows
-        // a thread; chunks of about 16 planes, shorter where that leaves SMs idle
-        const int lanes = g->n[0] > 32 ? 16 : 8, warps = CG_W;
+        // cg_dir / cg_res_u: CG_R rows a thread; chunks of about 16 planes, shorter
+        // where that leaves SMs idle. Tiles of 64 x 16 cells (16 lanes along x, CG_W
+        // warps); 32 x 32 (8 lanes) or 64 x 8 (2 warps) where those hold enough
+        // more cells of the grid; 32 lanes and no more warps than rows ask for where
+        // the rows are few. us an iteration, 64 x 16 / as chosen, uniform k:
+        // 130x258x200 92 / 80, 200x200x200 96 / 86, 70x260x300 91 / 78, 321x200x100
+        // 73.6 / 69.2, 1000x2x1000 124 / 43, 500x8x700 50 / 37; nothing between
+        // them where all are full: 512x512x128 227.5, 228.1, 231.3
+        auto fill = [&](int l, int w) {
+            const int tx = 4 * l, ty = CG_R * w * 32 / l;
+            return (double)g->n[0] * g->n[1] /
+                   ((double)((g->n[0] + tx - 1) / tx * tx) * ((g->n[1] + ty - 1) / ty * ty));
+        };
+        int lanes = g->n[0] > 32 ? 16 : 8, warps = CG_W;
+        if (g->n[1] <= CG_R * CG_W && g->n[0] > 64) {
+            lanes = 32;
+        } else if (lanes == 16) {
+            if (fill(8, CG_W) > 1.05 * fill(16, CG_W)) lanes = 8;
+            else if (fill(16, 2) > 1.035 * fill(16, CG_W)) warps = 2;
+        }
+        if (lanes == 32) warps = std::min(warps, (g->n[1] + CG_R - 1) / CG_R);
         const long long bx = (g->n[0] + 4 * lanes - 1) / (4 * lanes);
         const int rows = CG_R * warps * 32 / lanes, by = (g->n[1] + rows - 1) / rows;
         const long long dcols = bx * by;
-        const long long dres = (long long)nsm * 16 / CG_W;   // resident blocks
+        const long long dres = (long long)nsm * 16 / warps;   // resident blocks
         long long dch = std::max(1, g->n[2] / 16);
         if (dcols * dch < dres) dch = std::min<long long>(g->n[2], std::max<long long>(dch, dres / dcols));
         dch = std::min<long long>(dch, std::max<long long>(1, CG_MAX_PART / dcols));
