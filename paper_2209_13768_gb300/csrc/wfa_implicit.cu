@@ -428,15 +428,15 @@ __global__ void __launch_bounds__(CG_TX * CG_TY, CgOcc<KVAR>::blocks) cg_init(co
 // boundary faces and masks held cells and cells beyond the x end; without
 // it every neighbour is inside the domain or across a periodic face. Both
 // evaluate the same expression, so an interior cell gets the same bits
-// either way. FM: the faces that may be near the warp's cells (see cg_r4).
-template <bool KVAR, bool EDGE, int FM = 63>
+// either way.
+template <bool KVAR, bool EDGE>
 __device__ __forceinline__ float cg_q4(const CgCoef& c, const CgEdge& e, int gx, int gy, int z, const float pc[4],
                                        const float pm[4], const float pp[4], const float ym[4], const float yp[4],
                                        float xm, float xp, const float kc[4], const float km[4], const float kp[4],
                                        const float kym[4], const float kyp[4], float kxm, float kxp, float q[4]) {
     float psum = 0.0f;
-    const bool zlo = EDGE && (FM & 16) && !c.periodic[2] && z == 0,
-               zhi = EDGE && (FM & 32) && !c.periodic[2] && z == c.n[2] - 1;
+    const bool zlo = EDGE && !c.periodic[2] && z == 0,
+               zhi = EDGE && !c.periodic[2] && z == c.n[2] - 1;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         float pw = i == 0 ? xm : pc[i - 1], pe = i == 3 ? xp : pc[i + 1];
@@ -451,10 +451,10 @@ __device__ __forceinline__ float cg_q4(const CgCoef& c, const CgEdge& e, int gx,
             kz1 = kp[i];
         }
         if (EDGE) {
-            if ((FM & 1) && i == 0 && (e.bits & 1u)) { pw = ghost(c, 0, pc[i]); kw = kc[i]; }
-            if ((FM & 2) && i == e.ih) { pe = ghost(c, 1, pc[i]); ke = kc[i]; }
-            if ((FM & 4) && (e.bits & 2u)) { y0 = ghost(c, 2, pc[i]); ky0 = kc[i]; }
-            if ((FM & 8) && (e.bits & 4u)) { y1 = ghost(c, 3, pc[i]); ky1 = kc[i]; }
+            if (i == 0 && (e.bits & 1u)) { pw = ghost(c, 0, pc[i]); kw = kc[i]; }
+            if (i == e.ih) { pe = ghost(c, 1, pc[i]); ke = kc[i]; }
+            if ((e.bits & 2u)) { y0 = ghost(c, 2, pc[i]); ky0 = kc[i]; }
+            if ((e.bits & 4u)) { y1 = ghost(c, 3, pc[i]); ky1 = kc[i]; }
             if (zlo) { z0 = ghost(c, 4, pc[i]); kz0 = kc[i]; }
             if (zhi) { z1 = ghost(c, 5, pc[i]); kz1 = kc[i]; }
         }
@@ -475,7 +475,7 @@ __device__ __forceinline__ float cg_q4(const CgCoef& c, const CgEdge& e, int gx,
             qi = __fmaf_rn(-c.cu[2], __fadd_rn(z0, z1), acc);
         }
         if (EDGE) {
-            const bool isfree = gx + i < c.n[0] && gy < c.n[1] && !cg_held_m<FM>(c, gx + i, gy, z);
+            const bool isfree = gx + i < c.n[0] && gy < c.n[1] && !cg_held(c, gx + i, gy, z);
             qi = isfree ? qi : 0.0f;
             psum = isfree ? __fmaf_rn(pc[i], qi, psum) : psum;
         } else {
@@ -1416,7 +1416,7 @@ struct CgWork {
     CgArgs key;        // arguments the graph was captured with
     int kvar = -1;
     int method = -1;   // WFA_CG_CLASSIC / WFA_CG_PIPELINED of the captured graphs
-    int spmv_grid[3] = {0, 0, 0};   // cg_init, cg_pipe
+    int init_grid[3] = {0, 0, 0};   // cg_init, cg_pipe
     int dir_grid[3] = {0, 0, 0};    // cg_dir, cg_res_u
     int dir_threads = 0, dir_chunk = 0, dir_lanes = 0;
     int upd_blocks = 0;
@@ -1547,10 +1547,10 @@ struct CgLaunch {
         iter.block = dim3(CG_CTL);
         iter.a = res.a;
         pipe.fn = kvar ? (const void*)cg_pipe<true> : (const void*)cg_pipe<false>;
-        pipe.grid = dim3(w->spmv_grid[0], w->spmv_grid[1], w->spmv_grid[2]);
+        pipe.grid = dim3(w->init_grid[0], w->init_grid[1], w->init_grid[2]);
         pipe.block = dim3(CG_TX, CG_TY);
         pipe.a = base;
-        pipe.a.nblk = w->spmv_grid[0] * w->spmv_grid[1] * w->spmv_grid[2];
+        pipe.a.nblk = w->init_grid[0] * w->init_grid[1] * w->init_grid[2];
         init = pipe;
         init.fn = kvar ? (w->o32 ? (const void*)cg_init<true, true> : (const void*)cg_init<true, false>)
                        : (w->o32 ? (const void*)cg_init<false, true> : (const void*)cg_init<false, false>);
@@ -1775,9 +1775,9 @@ int wfa_implicit_step(wfa_grid g, double dt, long long n, double rtol, int max_i
             set_error("wfa_implicit_step: grid too large for the partial-sum buffer");
             return WFA_ERR_ARG;
         }
-        w->spmv_grid[0] = gxb;
-        w->spmv_grid[1] = gyb;
-        w->spmv_grid[2] = (int)nch;
+        w->init_grid[0] = gxb;
+        w->init_grid[1] = gyb;
+        w->init_grid[2] = (int)nch;
         // cg_dir / cg_res_u: CG_R rows a thread; chunks of about 16 planes, shorter
         // where that leaves SMs idle. Tiles of 64 x 16 cells (16 lanes along x, CG_W
         // warps); 32 x 32 (8 lanes) or 64 x 8 (2 warps) where those hold enough
@@ -1880,7 +1880,7 @@ int wfa_implicit_step(wfa_grid g, double dt, long long n, double rtol, int max_i
                 set_error("wfa_implicit_step: the device loop ran %lld of %lld steps", Lr.steps_done, n);
                 return WFA_ERR_STATE;
             }
-            const int extra_per_step = method == WFA_CG_PIPELINED ? 4 : 3;   // init, [spmv], start, step
+            const int extra_per_step = method == WFA_CG_PIPELINED ? 4 : 3;   // init, start, [the first cg_dir], end of the step
             g->launches += extra_per_step * n + (method == WFA_CG_PIPELINED ? 2LL : 3LL) * Lr.total_iters;
             w->prev_iters = n > 0 ? Lr.total_iters / n : 0;
             g->halo_dirty = true;

@@ -38,7 +38,7 @@ constexpr int COL_VARIANT = 3;        // the one-step column-march kernel
 constexpr int FUSED_VARIANT = 4;      // the same kernel as PAIR_VARIANT
 constexpr int INPLACE_VARIANT = 5;    // the one-step column-march kernel, boundaries in place
 constexpr int WIDE_VARIANT = 6;       // the one-step column-march kernel, 8 cells a thread (16 for bf16, uniform k)
-constexpr int PAIR_VARIANT = 7;       // two steps per pass in registers (uniform k)
+constexpr int PAIR_VARIANT = 7;       // two steps per pass in registers
 
 // Which periodic copies a field buffer holds (wfa_grid_s::thin): layers beyond
 // each face (a bit each for one layer, every layer with the corners, and 4

@@ -157,7 +157,7 @@ static int num_sms() {
 // Kernel configuration of a pass: variant (COL_VARIANT = column march, one
 // step; INPLACE_VARIANT = the same with boundaries and periodic copies in the
 // pass itself; WIDE_VARIANT = column march, 8 cells a thread (16 for bf16 with uniform k);
-// PAIR_VARIANT (and FUSED_VARIANT) = two steps in registers, uniform k; 1..NUM_TILE_VARIANTS
+// PAIR_VARIANT (and FUSED_VARIANT) = two steps in registers; 1..NUM_TILE_VARIANTS
 // = tiled TMA kernel, `depth` fused steps; -1 = the plain one-column kernel)
 // and depth.
 struct Choice {
@@ -401,8 +401,8 @@ static SweepArgs base_args(wfa_grid_s* g, const SweepCoef& c, int in_buf, int zc
     return a;
 }
 
-// Kernels one pass launches (the column kernels add a boundary fix-up and a
-// copy per periodic axis, see col_launch / col2_launch).
+// Kernels one pass launches (the thin column pass adds a boundary fix-up where
+// the ghost layers do not hold the faces, see col_launch_v).
 static int pass_launches(const wfa_grid_s* g, const SweepCoef& c, int depth, int variant) {
     if (two_step_variant(variant) && depth == 2) return 1;
     if (variant == COL_VARIANT || variant == WIDE_VARIANT || two_step_variant(variant)) {   // thin pass

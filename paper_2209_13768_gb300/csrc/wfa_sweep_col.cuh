@@ -110,19 +110,6 @@ __device__ __forceinline__ float uniform_cell(const SweepCoef& c, float tc, floa
     return is_held(c, x, y, z) ? tc : v;
 }
 
-// Interior cell (no face on the boundary, not held, no self term).
-__device__ __forceinline__ float uniform_inner(const SweepCoef& c, float tc, float txm, float txp, float tym,
-                                               float typ, float tzm, float tzp) {
-    return __fadd_rn(tc, flux_sum(tc, txm, txp, tym, typ, tzm, tzp, c.w_in[0], c.w_in[1], c.w_in[2], c.w_in[3],
-                                  c.w_in[4], c.w_in[5]));
-}
-
-// Outside the domain on a non-periodic axis (a ghost or padding cell).
-__device__ __forceinline__ bool outside_np(const SweepCoef& c, int x, int y, int z) {
-    return (!c.periodic[0] && (x < 0 || x >= c.n[0])) || (!c.periodic[1] && (y < 0 || y >= c.n[1])) ||
-           (!c.periodic[2] && (z < 0 || z >= c.n[2]));
-}
-
 // V consecutive stored values <-> V floats (V = 4, 8 or 16; 8 fp32 values
 // are two 128-bit accesses, 8 bf16 values one).
 template <typename S, bool COH, int V>
@@ -280,10 +267,8 @@ template <bool KVAR, bool INL = false, int ES = 4, int V = 4> struct ColOcc {
 
 // How a column pass treats boundary cells and periodic copies.
 enum ColMode {
-    COL_MAIN = 0,    // every cell takes the interior formula; boundary cells and periodic copies
-                     // are rewritten afterwards (the batched sweep's boundary and copy launches)
-    COL_INPLACE = 1, // boundary cells in place, every periodic copy of a written cell stored (full halo)
-    COL_THIN = 2     // every cell takes the interior formula, and one layer of periodic copies
+    COL_INPLACE,     // boundary cells in place, every periodic copy of a written cell stored (full halo)
+    COL_THIN         // every cell takes the interior formula, and one layer of periodic copies
                      // (no corners: all that a one-step pass reads) is stored in the pass; the
                      // boundary cells, if the ghost layers do not hold the faces, follow in a
                      // short launch (boundary_fix) that stores their copies too
@@ -424,7 +409,7 @@ __device__ __forceinline__ void col_run(const SweepCoef& c, const S* __restrict_
         }
         // the new values in fp32; every store rounds them to S once
         float out[V];
-        if (MODE == COL_MAIN || MODE == COL_THIN || fast) {   // interior formula (see ColMode)
+        if (MODE == COL_THIN || fast) {   // interior formula (see ColMode)
 #pragma unroll
             for (int i = 0; i < V; ++i) {
                 const float txm = i == 0 ? nb.tx_m : tc[i - 1];
@@ -500,13 +485,7 @@ __device__ __forceinline__ void col_run(const SweepCoef& c, const S* __restrict_
             }
         } else {
             const bool plain = plain_xy && !(perz && (z < HALO || z >= c.n[2] - HALO));
-            // partial vector at the x end with per-cell k: the halo keeps its ghost
-            // values (uniform k never reads them, and the unmasked store is faster)
-            if (MODE == COL_MAIN && KVAR && !full_x) {
-#pragma unroll
-                for (int i = 0; i < V; ++i)
-                    if (gx + i < c.n[0]) op[i] = from_f32<S>(out[i]);
-            } else if (MODE == COL_MAIN || plain) {
+            if (plain) {
                 stv<S, V>(op, out);
             } else if (!perx && !pery && !perz) {   // the x end of a row, no copies to store
 #pragma unroll
@@ -596,72 +575,6 @@ __global__ void __launch_bounds__(256) boundary_fix(const __grid_constant__ Swee
         else
             ((S*)a.tout)[i] = from_f32<S>(v);
     }
-}
-
-// Periodic halo copies of one axis, over the full extent of the other two
-// (their halos included, so corners are right when the axes go x, y, z).
-// Element order: for x copies the 16 halo columns of a row are consecutive,
-// for y and z copies whole padded rows are, so loads and stores coalesce.
-// Totals fit 32-bit arithmetic (the caller checks).
-template <typename S>
-__global__ void __launch_bounds__(256) twin_copy(const __grid_constant__ SweepCoef c, S* origin, int ax) {
-    const unsigned ex = c.n[0] + 2 * HALO, ey = c.n[1] + 2 * HALO, ez = c.n[2] + 2 * HALO;
-    const unsigned total = 2u * HALO * (ax == 0 ? ey * ez : ex * (ax == 1 ? ez : ey));
-    const int n = c.n[ax];
-    for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x) {
-        int p[3], k;
-        if (ax == 0) {            // (layer, y, z)
-            k = (int)(t & (2 * HALO - 1));
-            const unsigned r = t / (2 * HALO);
-            p[1] = (int)(r % ey) - HALO;
-            p[2] = (int)(r / ey) - HALO;
-        } else if (ax == 1) {     // (x, layer, z)
-            p[0] = (int)(t % ex) - HALO;
-            const unsigned r = t / ex;
-            k = (int)(r & (2 * HALO - 1));
-            p[2] = (int)(r / (2 * HALO)) - HALO;
-        } else {                  // (x, y, layer)
-            p[0] = (int)(t % ex) - HALO;
-            const unsigned r = t / ex;
-            p[1] = (int)(r % ey) - HALO;
-            k = (int)(r / ey);
-        }
-        const int dst = k < HALO ? k - HALO : n + (k - HALO);
-        int src = dst % n;
-        if (src < 0) src += n;
-        p[ax] = dst;
-        const long long od = (long long)p[2] * c.sz + (long long)p[1] * c.sy + p[0];
-        p[ax] = src;
-        const long long os = (long long)p[2] * c.sz + (long long)p[1] * c.sy + p[0];
-        origin[od] = origin[os];
-    }
-}
-
-// After a branch-free main pass: the boundary cells (unless the ghost layers
-// hold the faces), then the periodic copies of the written buffer.
-template <typename S, bool KVAR>
-cudaError_t fix_and_twins(const SweepArgs& a, cudaStream_t st, int nsm) {
-    long long plane = 0;   // the largest face
-    for (int ax = 0; ax < 3; ++ax) {
-        const int b = ax == 0 ? 1 : 0, d = ax == 2 ? 1 : 2;
-        if (!a.c.periodic[ax]) plane = std::max(plane, (long long)a.c.n[b] * a.c.n[d]);
-    }
-    if (plane > 0 && !a.c.halo_bc) {
-        const int nb = (int)std::min<long long>((plane + 255) / 256, (long long)nsm * 2);
-        boundary_fix<S, KVAR><<<dim3(nb, 6), 256, 0, st>>>(a);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-    }
-    for (int ax = 0; ax < 3; ++ax) {
-        if (!a.c.periodic[ax]) continue;
-        const int b = ax == 0 ? 1 : 0, d = ax == 2 ? 1 : 2;
-        const long long total = 2LL * HALO * (a.c.n[b] + 2 * HALO) * (a.c.n[d] + 2 * HALO);
-        const int nb = (int)std::min<long long>((total + 255) / 256, (long long)nsm * 8);
-        twin_copy<S><<<nb, 256, 0, st>>>(a.c, (S*)a.tout, ax);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
 }
 
 // One column pass (variant 3: V = 4, variant 6: V = 8, or 16 for bf16 with
