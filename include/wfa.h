@@ -125,10 +125,12 @@ int wfa_set_dt(wfa_grid g, double dt);
  * tiled TMA kernel (depth steps per pass); 3 = the column-march kernel (one
  * step per pass, register queue along z, no shared memory; boundary cells by
  * ghost layers or a short fix-up launch); 4 and 7 = two steps per pass with
- * both steps' planes in registers (not with held layers, exchange faces, or
- * zero-flux faces that meet advection with per-cell k: there they act as 3); 5 = the column-march kernel with boundary
- * cells and periodic copies inside the pass (one launch per step; for small
- * grids); 6 = the column-march kernel with 8 cells a thread (16 for bf16
+ * both steps' planes in registers (not with rows of fewer than 8 cells, more
+ * rows than a launch can index (262140 and up), held layers, exchange faces,
+ * zero-flux faces that meet advection with per-cell k, or a bf16 field whose
+ * Dirichlet values bf16 does not hold: there they act as 3); 5 = the
+ * column-march kernel with boundary cells and periodic copies inside the pass
+ * (one launch per step; for small grids); 6 = the column-march kernel with 8 cells a thread (16 for bf16
  * fields with uniform k); -1 = the plain
  * one-thread-per-column kernel (one step per pass; a
  * second, independent realisation of the same per-cell arithmetic).
@@ -186,7 +188,8 @@ int wfa_steps_done(wfa_grid g, long long* n);
 int wfa_read_field(wfa_grid g, float* host_dense);
 
 /* Total heat E = sum_C T_C hx hy hz, summed on the device in fp64 in a fixed
- * order (bit-reproducible for a given grid). Synchronises the stream.
+ * order (bit-reproducible for a given grid; blocks of 16 cells exactly, in fp32
+ * sums with their rounding errors, before they enter the fp64 sums). Synchronises the stream.
  * Sec. 3, reduction of a field to one value. */
 int wfa_total_heat(wfa_grid g, double* e);
 
@@ -236,7 +239,7 @@ int wfa_implicit_step(wfa_grid g, double dt, long long n, double rtol, int max_i
 
 /* CG variant of wfa_implicit_step (the iterates are the same in exact
  * arithmetic; the default is WFA_CG_CLASSIC):
- *   WFA_CG_CLASSIC    classic CG, two inner products and two kernels an
+ *   WFA_CG_CLASSIC    classic CG, two inner products and three kernels an
  *                     iteration (Sec. 1.1.2);
  *   WFA_CG_PIPELINED  Chronopoulos and Gear's CG, both inner products in one
  *                     reduction and one kernel an iteration (the

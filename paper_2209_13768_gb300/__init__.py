@@ -280,7 +280,7 @@ class Grid:
         return n.value
 
     def set_cg_method(self, method):
-        """"classic" (two kernels and two reductions an iteration) or
+        """"classic" (three kernels and two reductions an iteration) or
         "pipelined" (Chronopoulos-Gear: one of each); see wfa_set_cg_method."""
         m = {"classic": CG_CLASSIC, "pipelined": CG_PIPELINED}.get(method, method)
         check(lib().wfa_set_cg_method(self.handle, int(m)), "wfa_set_cg_method")

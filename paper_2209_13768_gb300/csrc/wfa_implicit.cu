@@ -61,7 +61,7 @@ constexpr int CG_THREADS = 256;
 constexpr int CG_CTL = 512;             // threads of the one-block control kernels (16 warps: see block_sum)
 constexpr int CG_MAX_PART = 16384;      // per-block partials of one launch
 constexpr int CG_FOLD = 512;            // most blocks of cg_dir whose partials every block of cg_res sums
-constexpr int CG_R = 2, CG_W = 4;       // cg_dir / cg_res_u: rows a thread, warps of a block
+constexpr int CG_R = 2, CG_W = 4;       // cg_dir / cg_res_u: rows a thread, most warps of a block
 constexpr int CG_NRUN = 4;              // captured runs of 1, 2, 4 and 8 iterations
 constexpr int CG_RUN_LEN[CG_NRUN] = {1, 2, 4, 8};
 
@@ -764,8 +764,8 @@ __device__ __forceinline__ void cg_put_twins(float* dom, int z, const CgCoef& c,
 // has CG_R rows whose y neighbours and faces are its own registers, x
 // neighbours come by shuffle, and an address is one add (O32; 64-bit address
 // arithmetic: +30 us with per-cell k). Warps on an x face run the same body
-// with ghost values (cg_rows). 16 lanes along x: 32 and 8 are 1 - 3% slower on
-// 512^3 and 390 x 322 x 257; chunks of 32 planes 2%, of 64 planes 10% slower.
+// with ghost values (cg_rows). Lanes along x: as many of 16 or 8 as fill their
+// tiles best (wfa_implicit_step); chunks of 32 planes 2%, of 64 planes 10% slower.
 // 512^3, uniform k: 444 us (2.8 GB, 6.3 TB/s) + cg_res_u 254 us (1.68 GB, 6.6
 // TB/s), where q stored and x updated with r took 371 + 481 us; 390 x 322 x
 // 257, per-cell k: 197 us (1.03 GB, 5.2 TB/s) + cg_res_k 66 us for 183 + 123.

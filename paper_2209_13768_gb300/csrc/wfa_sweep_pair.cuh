@@ -186,9 +186,10 @@ __device__ __forceinline__ void edge_self(const SweepCoef& c, const f2 (&t)[2], 
 
 constexpr int PAIR_TX = 120;   // cells a warp updates along x
 
-// Registers decide: 168 a thread (a few spilled words) for 12 warps an SM,
-// as blocks of 1 or 2 warps so that no tail of a larger block holds them
-// (fp32 2 warps 1366 GLUPS, 4 warps 1355; bf16 1 warp 1382, 4 warps 1355).
+// Registers decide: 168 a thread for 12 warps an SM (65 to 80 words spilled in
+// fp32, 21 to 28 in bf16), as blocks of 1 or 2 warps so that no tail of a
+// larger block holds them (fp32 2 warps 1366 GLUPS, 4 warps 1355; bf16 1 warp
+// 1382, 4 warps 1355).
 template <typename S> struct PairCfg {
     static constexpr int R = 4;                              // rows a warp updates
     static constexpr int WPB = sizeof(S) == 4 ? 2 : 1;       // warps a block
