@@ -1796,7 +1796,9 @@ int wfa_implicit_step(wfa_grid g, double dt, long long n, double rtol, int max_i
             lanes = 32;
         } else if (lanes == 16) {
             if (fill(8, CG_W) > 1.05 * fill(16, CG_W)) lanes = 8;
-            else if (fill(16, 2) > 1.035 * fill(16, CG_W)) warps = 2;
+            else if (fill(16, 2) > 1.035 * fill(16, CG_W) &&   // twice the tiles: only where their partials have room
+                     (long long)((g->n[0] + 63) / 64) * ((g->n[1] + 7) / 8) <= CG_MAX_PART)
+                warps = 2;
         }
         if (lanes == 32) warps = std::min(warps, (g->n[1] + CG_R - 1) / CG_R);
         const long long bx = (g->n[0] + 4 * lanes - 1) / (4 * lanes);

@@ -17,3 +17,8 @@ pytestmark = pytest.mark.gpu
     (64, 16, 17), (128, 32, 5)])                                                     # 64 x 16
 def test_every_tile_matches_oracle(shape, faces, kvar):
     _check(_problem(faces, shape, kvar, seed=sum(shape) + 3 * faces))
+
+
+def test_wide_grids_keep_tiles_whose_partials_fit():
+    # 64 x 8 would fill better (200 rows), but 1094 x 25 tiles have more partials than there is room for
+    _check(_problem(0, (70016, 200, 3), False, seed=1), m=2)
